@@ -91,7 +91,7 @@ void free_game(pg_game* g) {
                     g->tiles, g->tsum,   g->cnt,    g->scan_tmp, g->stage, g->loop_iters, g->ws, g->wsB, g->gdB, g->key128,
                     g->d_anc, g->d_sc, g->d_podd, g->d_peven, g->d_oddL, g->d_evenL, g->d_nxt, g->d_wt, g->d_loc,
                     g->d_own, g->d_rid, g->d_rl, g->d_val, g->d_rnx, g->pl_vid[0], g->pl_vid[1], g->pl_off[0],
-                    g->pl_off[1], g->pl_tgt[0], g->pl_tgt[1], g->rv_off, g->rv_src, g->omark};
+                    g->pl_off[1], g->pl_tgt[0], g->pl_tgt[1], g->rv, g->rv_src, g->omark, g->emark, g->inc};
     int prev = -1;
     const bool switched =
         cudaGetDevice(&prev) == cudaSuccess && prev != g->device && cudaSetDevice(g->device) == cudaSuccess;
@@ -347,10 +347,13 @@ pg_status apply_profile(pg_game* g, const int32_t* sigma, const int32_t* tau, co
 
 // Loop condition of the device-side loop: continue while a game is active,
 // no device error was recorded and the hard cap is not reached.
+// iters[0] counts iterations (k_inc adds its own; a body that was for Even's
+// pass alone, or none, is the one that counts its valuation), iters[1] bodies.
 __global__ void k_loop_cond(cudaGraphConditionalHandle h, const int32_t* gactive, const Counters* c, int64_t* iters,
                             int64_t hard_cap) {
-    const int64_t it = *iters + 1;
-    *iters = it;
+    const int64_t it = iters[0] + 1;
+    iters[0] = it;
+    iters[1] += 1;
     cudaGraphSetConditional(h, (gactive[0] > 0 && c->err == 0 && c->deep == 0 && it < hard_cap) ? 1u : 0u);
 }
 
@@ -362,6 +365,14 @@ pg_status enqueue_iteration(pg_game* g, int64_t cap, bool even) {
     if (!st && even) st = cmp ? enqueue_switch_cmp(g, 0) : enqueue_switch(g, 0);
     if (!st) st = enqueue_bookkeeping(g, cap, even);
     if (!st && even && g->reset_tau) st = enqueue_reset(g);
+    return st;
+}
+
+// One body of the loop graph: an iteration over the whole game and, for one
+// game, the incremental iterations that can follow it.
+pg_status enqueue_body(pg_game* g, int64_t cap, bool even) {
+    pg_status st = enqueue_iteration(g, cap, even);
+    if (!st && loop_compares(g) && omark_of(g) && inc_applies(g)) st = enqueue_inc(g, cap, even, false);
     return st;
 }
 
@@ -410,7 +421,7 @@ bool build_loop_graph(pg_game* g, int64_t cap, bool even, int64_t limit) {
         ok = cudaStreamBeginCaptureToGraph(ctx->cap_stream, body, nullptr, nullptr, 0,
                                            cudaStreamCaptureModeThreadLocal) == cudaSuccess;
         if (ok) {
-            bool enq = enqueue_iteration(g, cap, even) == PG_OK;
+            bool enq = enqueue_body(g, cap, even) == PG_OK;
             if (enq) {
                 k_loop_cond<<<1, 1, 0, ctx->cap_stream>>>(h, g->gactive, g->cnt, g->loop_iters, limit);
                 enq = cudaGetLastError() == cudaSuccess;
@@ -444,6 +455,12 @@ bool build_loop_graph(pg_game* g, int64_t cap, bool even, int64_t limit) {
     return true;
 }
 
+// One game of at most kIncWhole ids: k_inc runs the whole loop, over all ids
+// where an iteration is not incremental.
+bool runs_whole(const pg_game* g, const Timer& tm) {
+    return !tm.on && g->ctx->graphs && loop_compares(g) && inc_applies(g) && g->n <= kIncWhole;
+}
+
 // Algorithm 1 for every game of g at once: each iteration computes the
 // valuation of every game, switches Odd in active games, switches Even in
 // games whose inner loop has converged (no Odd switch this iteration), and
@@ -461,19 +478,33 @@ pg_status run_loop_once(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t l
     *ran = 0;
     const bool cmp = loop_compares(g);
     const int64_t hard = limit > 0 ? std::min<int64_t>(limit, cap + 2) : cap + 2;
+    if (runs_whole(g, tm)) {  // the whole loop is one launch
+        cudaStream_t s = ctx->stream;
+        PG_CUDA_TRY(ctx, cudaMemsetAsync(g->loop_iters, 0, 2 * sizeof(int64_t), s));
+        PG_CUDA_TRY(ctx, cudaMemsetAsync(g->cnt, 0, sizeof(Counters), s));
+        pg_status st = enqueue_inc(g, cap, even, true);
+        if (st) return st;
+        int64_t* it = (int64_t*)ctx->pinned;
+        PG_CUDA_TRY(ctx, cudaMemcpyAsync(it, g->loop_iters, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+        st = sync_counters(g);
+        *ran = *it;
+        g->t_vals += *it;
+        g->last_graph = true;
+        return st;
+    }
     if (!tm.on && ctx->graphs && build_loop_graph(g, cap, even, hard)) {
         const int w = even ? 1 : 0;
         cudaStream_t s = ctx->stream;
-        PG_CUDA_TRY(ctx, cudaMemsetAsync(g->loop_iters, 0, sizeof(int64_t), s));
+        PG_CUDA_TRY(ctx, cudaMemsetAsync(g->loop_iters, 0, 2 * sizeof(int64_t), s));
         PG_CUDA_TRY(ctx, cudaGraphLaunch(g->loop_exec[w], s));
         int64_t* it = (int64_t*)ctx->pinned;
-        PG_CUDA_TRY(ctx, cudaMemcpyAsync(it, g->loop_iters, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+        PG_CUDA_TRY(ctx, cudaMemcpyAsync(it, g->loop_iters, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
         pg_status st = sync_counters(g);
-        const int64_t iters = *it;
+        const int64_t iters = it[0], bodies = it[1];
         *ran = iters;
         g->t_vals += iters;
-        ctx->launches += g->loop_launch[w] * iters;
-        for (int i = 0; i < KID_COUNT; ++i) g->klaunch[i] += g->loop_klaunch[w][i] * iters;
+        ctx->launches += g->loop_launch[w] * bodies;
+        for (int i = 0; i < KID_COUNT; ++i) g->klaunch[i] += g->loop_klaunch[w][i] * bodies;
         g->last_graph = true;
         if (st) return st;
         if (iters > hard) return fail(ctx, PG_ECUDA, "device-side loop exceeded its iteration cap");
@@ -507,12 +538,16 @@ pg_status run_loop_once(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t l
 // game continues from the same profile with the ruling-set ranks (for the
 // rest of this call), so the trajectory is unchanged.
 pg_status run_loop(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t limit) {
-    if (loop_compares(g) && !g->pl_ok) {
+    if (runs_whole(g, tm)) {
+        pg_status st = build_reverse(g, 0);
+        if (st) return st;
+    } else if (loop_compares(g) && !g->pl_ok) {
         pg_status st = build_player_split(g);
         if (st) return st;
     }
     if (omark_of(g))  // the first Odd pass of the call evaluates every Odd vertex (a nonzero flag)
         PG_CUDA_TRY(g->ctx, cudaMemsetAsync(g->gactive + 1, 0xff, sizeof(int32_t), g->ctx->stream));
+    if (g->inc) PG_CUDA_TRY(g->ctx, cudaMemsetAsync(g->inc, 0, sizeof(IncState), g->ctx->stream));
     int64_t done = 0;
     for (;;) {
         int64_t ran = 0;

@@ -59,6 +59,95 @@ __device__ inline bool g32_none(uint32_t w) { return (w & kG32None) != 0; }
 __device__ inline bool g32_sink(uint32_t w) { return (w & kG32Sink) != 0; }
 __device__ inline int32_t g32_ptr(uint32_t w) { return (int32_t)(w & 0x3fffffffu); }
 
+// Words of the iterations that compare valuations (k_walk_cmp, k_jump32_coop,
+// k_inc). A word with both the none and the sink
+// bit set is pending: its low bits are a jump pointer (every vertex strictly
+// between v and it on the play is below v, and so is the pointer). A word
+// with only the sink bit (g(v) is the game's sink slot, which the word does
+// not repeat) carries v's priority parity in bit 0, so that the vertex that
+// ends a chain gives its top's parity with no further read.
+constexpr uint32_t kG32Pend = kG32None | kG32Sink;
+__device__ inline bool g32_pending(uint32_t w) { return (w & kG32Pend) == kG32Pend; }
+__device__ inline uint32_t g32_sink_word(uint8_t fl) { return kG32Sink | ((fl & kPriOdd) ? 1u : 0u); }
+
+// After k_classify, bit 31 of a g-word marks a TOP vertex (its play ends in
+// a cycle); finite words are unchanged (bit 30: g(v) is the game's sink slot).
+constexpr uint32_t kG32Top = 0x80000000u;
+// k_classify also writes one "top word" per vertex: bit 31 = TOP; for a finite
+// vertex bits 0..29 = its top, the last vertex of its g-chain below the sink
+// slot (a child of the sink in the g-forest), and bit 30 = that top's priority
+// is odd.
+constexpr uint32_t kTopOdd = 0x40000000u;
+__device__ inline int32_t top_id(uint32_t t) { return (int32_t)(t & 0x3fffffffu); }
+
+template <bool CG>
+__device__ inline uint32_t ld_word(const uint32_t* p) {
+    return CG ? __ldcg(p) : *p;
+}
+
+// Compares the valuations of two finite vertices u and w of one game with the
+// same top: walk both g-chains (words wu, ww) upwards, always advancing the
+// smaller id, until they meet (at the top at the latest). The larger of the
+// last two vertices passed below the meeting point is the largest vertex of
+// the symmetric difference of the two plays; its side is better for Even
+// when its priority is even. Returns > 0 if Val(u) is better for Even, < 0 if
+// worse, 0 if u == w. g(x) > x for every vertex below the top, so each step
+// raises a or b. CG: the words change during the kernel (k_inc) and are read
+// from L2.
+template <bool CG = false>
+__device__ inline int cmp_walk(int32_t u, int32_t w, const uint32_t* __restrict__ gd32,
+                               const uint8_t* __restrict__ flags) {
+    int32_t a = u, b = w, pa = -1, pb = -1;
+    uint32_t wa = 0, wb = 0;
+    if (a != b) {
+        wa = ld_word<CG>(gd32 + a);
+        wb = ld_word<CG>(gd32 + b);
+    }
+    while (a != b) {
+        if (a < b) {
+            pa = a;
+            a = g32_ptr(wa);
+            if (a <= pa) return 0;  // g-chains rise (a guard that keeps every walk finite; never taken)
+            wa = ld_word<CG>(gd32 + a);
+        } else {
+            pb = b;
+            b = g32_ptr(wb);
+            if (b <= pb) return 0;
+            wb = ld_word<CG>(gd32 + b);
+        }
+    }
+    if (pa == pb) return 0;  // u == w
+    const bool u_side = pa > pb;
+    const bool even = !(flags[u_side ? pa : pb] & kPriOdd);
+    return u_side == even ? 1 : -1;
+}
+
+// Order of the valuations of u and w (vertices of one game, with their top
+// words tu, tw): > 0 if Val(u) is better for Even than Val(w), < 0 if worse,
+// 0 if equal. TOP is above every finite valuation and equal to TOP. Finite
+// plays with different tops differ above everything else at the larger top,
+// which decides by its parity; with the same top the chains are walked.
+template <bool CG = false>
+__device__ inline int cmp_val(int32_t u, uint32_t tu, int32_t w, uint32_t tw, const uint32_t* __restrict__ gd32,
+                              const uint8_t* __restrict__ flags) {
+    const int xu = (tu & kG32Top) ? 1 : 0, xw = (tw & kG32Top) ? 1 : 0;
+    if (xu | xw) return xu - xw;
+    const int32_t hu = top_id(tu), hw = top_id(tw);
+    if (hu != hw) {
+        const bool u_side = hu > hw;
+        const bool even = !((u_side ? tu : tw) & kTopOdd);
+        return u_side == even ? 1 : -1;
+    }
+    return cmp_walk<CG>(u, w, gd32, flags);
+}
+
+// Against the sink's empty valuation: the top of a finite play is its largest
+// vertex, so Val(u) is better for Even exactly when that top is even.
+__device__ inline int cmp_sink(uint32_t tu) {
+    if (tu & kG32Top) return 1;
+    return (tu & kTopOdd) ? -1 : 1;
+}
+
 // The sink slot of v's game.
 __device__ inline int32_t sink_of(int32_t v, const int32_t* vgame, const int32_t* gsink, int32_t sink0) {
     return vgame ? gsink[vgame[v]] : sink0;

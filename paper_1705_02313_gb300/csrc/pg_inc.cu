@@ -1,0 +1,635 @@
+// Incremental iterations of the compare-mode loop, for one game.
+//
+// After a switching pass only vertices whose play passes a switched vertex
+// can change their valuation (Section 3: a valuation is a function of the
+// play). Past the first iterations of a best response these are few: on the
+// 10M-vertex random game (G': 13.3M vertices) 23% and 3% of the vertices in
+// the first two iterations, under 0.1% from the fourth on, and after an Even
+// switch 50%, 27%, 5%, 1%, 0.2%, ... k_inc therefore runs whole iterations of
+// Algorithm 1 on that set alone:
+//   closure   A = the switched vertices and everything upstream of them in the
+//             strategy graph, found through the reverse adjacency of G' (a
+//             predecessor y of x belongs to x's tree when strat[y] = x); the
+//             g-word of each becomes a one-step jump pointer
+//   resolve   nearest greater vertices of A by walking jump pointers inside A
+//             and g-chains outside it, in rounds
+//   classify  class and top of A from the g-chains; predecessors of a vertex
+//             whose top changed, and predecessors whose last decision compared
+//             chains (their tie mark), are queued for their player
+//   switch    Odd's queue, or Even's when Odd had nothing to switch, with the
+//             rules of k_switch_cmp_pl
+// so that the decisions, and with them the trajectory, are those of full
+// iterations. One thread-block cluster runs all of them in one launch: an
+// iteration is a chain of dependent reads whatever its size, so what counts is
+// the number of dependent reads and barriers, not throughput. Every block keeps
+// its share of A, of the queues and of the switched vertices in its shared
+// memory (a vertex stays with the block that found it; a closure level costs a
+// block barrier, and its two dependent reads are the predecessors and, issued
+// together, their strategies, words and own list bounds); the blocks meet at
+// the hardware cluster barrier (about 0.3 us) after each step and pass their
+// counts through distributed shared memory. Random games, load and solve,
+// before and after (full iterations only; then these): 1k vertices 2.26 -> 1.11
+// ms, 30k 2.94 -> 1.76, 1M 5.05 -> 4.23, 10M 29.5 -> 23.1; the 10M ladder 43.0
+// -> 29.4 ms.
+#include <cooperative_groups.h>
+
+#include "pg_device.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace pg {
+namespace {
+
+constexpr int kIncThreads = 1024;
+constexpr int kIncCluster = 16;      // blocks of the cluster (non-portable size; fewer when the device refuses it)
+constexpr int kIncSet = 10240;       // vertices of A a block holds
+constexpr int kIncQueue = 8192;      // Odd's queue of a block (the rest spills to global memory)
+constexpr int kIncEven = 16384;      // Even's queue of a block (beyond it Even's next pass is full)
+constexpr int kIncFanIn = 1024;      // a vertex of A with more predecessors ends the incremental iteration
+constexpr int kIncLevels = 256;      // levels of the closure
+constexpr int kIncRounds = 128;      // rounds of the resolution
+constexpr int kIncSteps = 128;       // steps of one resolution round
+constexpr size_t kIncShared = sizeof(int32_t) * (3 * kIncSet + kIncQueue + kIncEven);
+constexpr int32_t kIncBig = 1 << 24;  // (16 blocks' counts sum below 2^31)
+// A full iteration follows a pass that switched more vertices than this. Large
+// games: against 270 us for a full iteration of the 10M random game, an
+// incremental one took 102 us from 7.4k switched vertices, 425 us from 11.8k
+// and 1,025 us from 27.9k; against 62 us on the 1M game, 48 us from 1.3k and
+// 125 us from 4.7k.
+constexpr int kIncSeedShare = 1024, kIncSeeds = 8192;
+// In a launch that runs the whole loop (41k ids): an iteration over all ids
+// takes 17-32 us, an incremental one 13 us (a few switched vertices) to 35 us
+// (a hundred, for the levels of the closure).
+constexpr int kIncWholeShare = 512;
+
+struct IncArgs {
+    int32_t n;       // ids, the sink slot included
+    int32_t sink0;
+    const int32_t* off;
+    const int32_t* tgt;
+    const uint8_t* flags;
+    const int2* rv;
+    const int32_t* rv_src;
+    int32_t* strat;
+    uint32_t* gd32;
+    uint32_t* topw;
+    uint8_t* omark;
+    uint8_t* emark;
+    const int32_t* alist;  // the switched vertices of the last full pass (cnt->n_list of them)
+    int32_t* qlist;        // [n] Odd's queue beyond the blocks' own
+    GameState* gst;
+    Counters* cnt;
+    IncState* st;
+    int32_t* gactive;
+    int64_t* loop_iters;
+    int64_t cap;
+    int32_t max_seeds;  // more switched vertices than this take a full iteration
+    int32_t whole;      // 1: the launch runs the whole loop, full iterations included (over all ids)
+    int32_t even;       // 0: best response (the inner loop only)
+    int32_t reset;      // SI-Reset
+    int32_t deep_cut;
+    int32_t deep_fallback;
+};
+
+// Sets bit b of byte p (in a 4-byte aligned array); returns whether it was clear.
+__device__ inline bool claim_byte(uint8_t* base, int32_t i, uint32_t b) {
+    const uint32_t sh = 8u * (uint32_t)(i & 3);
+    return !((atomicOr((uint32_t*)base + (i >> 2), b << sh) >> sh) & b);
+}
+
+// Decision of one vertex (the rules of k_switch_cmp): returns whether it
+// switched; *tie_out: the decision compared the chains of two finite
+// successors.
+template <int PLAYER>
+__device__ inline bool inc_switch(const IncArgs& a, int32_t v, bool* tie_out) {
+    const int32_t e0 = a.off[v], e1 = a.off[v + 1];
+    const int32_t cur = __ldcg(a.strat + v);
+    int32_t best = PLAYER == 0 ? a.sink0 : -1;
+    uint32_t tbest = 0;
+    bool cur_top = false, tie = false;
+    for (int32_t e = e0; e < e1; e += 4) {
+        int32_t t[4];
+        uint32_t tt[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) t[j] = e + j < e1 ? a.tgt[e + j] : -1;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) tt[j] = t[j] >= 0 ? __ldcg(a.topw + t[j]) : 0u;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (t[j] < 0) continue;
+            const bool first = PLAYER == 0 ? best == a.sink0 : best < 0;
+            if (PLAYER == 0 && t[j] == cur) cur_top = (tt[j] & kG32Top) != 0;
+            tie |= !first && !((tt[j] | tbest) & kG32Top) && top_id(tt[j]) == top_id(tbest);
+            bool take;
+            if (PLAYER == 1) take = first || cmp_val<true>(t[j], tt[j], best, tbest, a.gd32, a.flags) < 0;
+            else take = (first ? cmp_sink(tt[j]) : cmp_val<true>(t[j], tt[j], best, tbest, a.gd32, a.flags)) > 0;
+            if (take) {
+                best = t[j];
+                tbest = tt[j];
+            }
+        }
+    }
+    *tie_out = tie;
+    const bool sw = best != cur && (PLAYER == 0 ? !cur_top : !(tbest & kG32Top));
+    if (sw) __stcg(a.strat + v, best);
+    return sw;
+}
+
+__global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
+    cg::cluster_group cl = cg::this_cluster();
+    const int32_t CL = (int32_t)cl.num_blocks(), rank = (int32_t)cl.block_rank(), tid = threadIdx.x;
+    const int32_t T = CL * kIncThreads, t0 = rank * kIncThreads + tid;
+    extern __shared__ int32_t dyn[];
+    int32_t* la = dyn;             // this block's part of A: vertex,
+    int32_t* ls = la + kIncSet;    //    start of its predecessors,
+    int32_t* lc = ls + kIncSet;    //    their number << 16 | Odd's among them
+    int32_t* lq = lc + kIncSet;    // its part of Odd's queue
+    int32_t* le = lq + kIncQueue;  //    and of Even's
+    __shared__ int2 xb[2][kIncCluster];
+    __shared__ int32_t lvl[3], c_bad, c_left, c_q, c_spill, c_odd, c_s, c_e, c_zero;
+    int par = 0;
+    // The sums over the cluster of two counts, final in each block when all its threads call: every block stores
+    // its pair in every block's shared memory and sums after the barrier. Two buffers in turn: a block that is
+    // ahead writes the other one.
+    auto exchange = [&](const int32_t* pa, const int32_t* pb) {
+        __syncthreads();
+        if (tid < CL) cl.map_shared_rank(&xb[par][0], tid)[rank] = make_int2(*pa, *pb);
+        cl.sync();
+        int2 sum = make_int2(0, 0);
+        for (int i = 0; i < CL; ++i) {
+            const int2 x = xb[par][i];
+            sum.x += x.x;
+            sum.y += x.y;
+        }
+        par ^= 1;
+        return sum;
+    };
+    // every decision below is taken by all threads from sums that they share, so the cluster stays uniform
+    GameState gs;
+    gs.phase = __ldcg(&a.gst->phase);
+    gs.inner = __ldcg(&a.gst->inner);
+    gs.major = __ldcg(&a.gst->major);
+    const bool dead = __ldcg(&a.cnt->err) || __ldcg(&a.cnt->deep) || gs.phase != kPhaseActive;
+    // every Odd vertex is evaluated (the first iteration, or after an SI-Reset: gactive[1], set by k_bookkeep)
+    bool fresh = a.whole || __ldcg(a.gactive + 1);
+    bool even_full = a.whole || __ldcg(&a.st->even_full);
+    int32_t ns = fresh ? 0 : __ldcg(&a.cnt->n_list);  // switched vertices, all blocks
+    // nothing to do here (the state stays as k_bookkeep left it: a full iteration is next)
+    if (dead || (!a.whole && (fresh || ns > a.max_seeds))) return;
+    int32_t nsl = ns > rank ? (ns - rank + CL - 1) / CL : 0;  // this block's, in la
+    for (int32_t i = tid; i < nsl; i += kIncThreads) la[i] = __ldcg(a.alist + rank + i * CL);
+    if (tid == 0) c_e = c_zero = 0;
+    int32_t mode = kIncFull;
+    int64_t iters = 0;
+    bool done = false;
+    cl.sync();
+    while (!done) {
+        bool all = fresh || ns > a.max_seeds;
+        if (all && !a.whole) break;
+        if (tid == 0) {
+            c_bad = c_left = c_q = c_spill = c_odd = 0;
+            lvl[1] = 0;
+        }
+        if (t0 == 0) a.st->n_q = 0;
+        __syncthreads();
+        int32_t na = nsl;
+        if (!all) {
+            for (int32_t i = tid; i < nsl; i += kIncThreads) {
+                const int32_t v = la[i];
+                const int2 r = a.rv[v];
+                const int32_t k = a.rv[v + 1].x - r.x;
+                __stcg(a.gd32 + v, kG32Pend | (uint32_t)__ldcg(a.strat + v));
+                ls[i] = r.x;
+                lc[i] = k << 16 | ((r.y - r.x) & 0xffff);
+                if (k > kIncFanIn) c_bad = 1;
+            }
+            cl.sync();
+            // level r expands la[lo .. na) into la[na ..]; lvl[] rotates, so a count is stable while it is read. A
+            // level that cannot be held (kIncBig) ends the closure.
+            bool bad = c_bad != 0;
+            int32_t lo = 0;
+            for (int32_t r = 0; !bad && lo < na; ++r) {
+                int32_t* next = &lvl[(r + 1) % 3];
+                if (tid == 0) lvl[(r + 2) % 3] = 0;
+                for (int32_t i = lo + tid; i < na; i += kIncThreads) {
+                    const int32_t x = la[i], e0 = ls[i], e1 = e0 + (lc[i] >> 16);
+                    for (int32_t e = e0; e < e1; e += 4) {
+                        int32_t y[4], s[4], r1[4];
+                        uint32_t w[4];
+                        int2 r0[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) y[j] = e + j < e1 ? a.rv_src[e + j] : x;  // (x: not below itself)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            s[j] = __ldcg(a.strat + y[j]);
+                            w[j] = __ldcg(a.gd32 + y[j]);
+                            r0[j] = a.rv[y[j]];
+                            r1[j] = a.rv[y[j] + 1].x;
+                        }
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            // one thread reads all of x's predecessors: a repeated edge shows in its own earlier
+                            // write, or inside this group of four
+                            bool in = s[j] == x && !g32_pending(w[j]);
+#pragma unroll
+                            for (int q = 0; q < j; ++q) in = in && y[q] != y[j];
+                            if (!in) continue;
+                            __stcg(a.gd32 + y[j], kG32Pend | (uint32_t)x);
+                            const int32_t p = na + atomicAdd(next, 1), k = r1[j] - r0[j].x;
+                            if (p >= kIncSet || k > kIncFanIn) {
+                                atomicOr(next, kIncBig);
+                                continue;
+                            }
+                            la[p] = y[j];
+                            ls[p] = r0[j].x;
+                            lc[p] = k << 16 | (r0[j].y - r0[j].x);
+                        }
+                    }
+                }
+                __syncthreads();
+                const int32_t found = *next;
+                bad = found >= kIncBig || r + 1 >= kIncLevels;
+                lo = na;
+                if (!bad) na += found;
+            }
+            if (bad && tid == 0) c_bad = 1;
+            all = exchange(&c_bad, &c_zero).x != 0;
+            if (all && !a.whole) break;
+        }
+        if (all) {
+            even_full = true;
+            if (tid == 0) c_bad = 0;
+            for (int32_t v = t0; v < a.n; v += T)
+                __stcg(a.gd32 + v, v == a.sink0 ? kG32Sink : kG32Pend | (uint32_t)__ldcg(a.strat + v));
+            cl.sync();
+        }
+        // ids [i0, i1) in steps of st are this thread's, or la[i] of them
+        const int32_t i0 = all ? t0 : tid, i1 = all ? a.n : na, step = all ? T : kIncThreads;
+        // resolve: words of A turn from jump pointers into g-words; any word read is valid whenever it is read
+        bool unresolved = false;
+        for (int32_t r = 0;; ++r) {
+            int32_t left = 0;
+            for (int32_t i = i0; i < i1; i += step) {
+                const int32_t v = all ? i : la[i];
+                const uint32_t w = __ldcg(a.gd32 + v);
+                if (!g32_pending(w)) continue;
+                int32_t x = g32_ptr(w);
+                bool top = false;
+                for (int k = 0; k < kIncSteps && x < v; ++k) {
+                    const uint32_t wx = __ldcg(a.gd32 + x);
+                    if (g32_none(wx) && !g32_pending(wx)) {  // TOP: v's play ends in the same cycle
+                        top = true;
+                        break;
+                    }
+                    x = g32_sink(wx) && !g32_pending(wx) ? a.sink0 : g32_ptr(wx);
+                }
+                uint32_t nw;
+                if (top) nw = kG32None | (uint32_t)a.sink0;  // (a pointer that no cycle maximum has)
+                else if (x > v) nw = x == a.sink0 ? g32_sink_word(a.flags[v]) : (uint32_t)x;
+                else if (x == v) nw = kG32None | (uint32_t)v;
+                else {
+                    nw = kG32Pend | (uint32_t)x;
+                    left = 1;
+                }
+                __stcg(a.gd32 + v, nw);
+            }
+            if (left) c_left = 1;
+            const int32_t rem = exchange(&c_left, &c_zero).x;
+            if (rem == 0) break;
+            if (r + 1 >= kIncRounds) {
+                unresolved = true;
+                break;
+            }
+            if (tid == 0) c_left = 0;
+            __syncthreads();
+        }
+        if (unresolved) {
+            if (!a.whole) break;  // the full iteration decides
+            if (!all) {           // over all ids once
+                ns = a.n;
+                __syncthreads();
+                continue;
+            }
+            if (t0 == 0) {
+                if (a.deep_fallback) a.cnt->deep = 1;
+                else atomicOr(&a.cnt->err, kErrJumpRounds);
+            }
+            ++iters;
+            break;
+        }
+        // classify (as k_classify)
+        for (int32_t i = i0; i < i1; i += step) {
+            const int32_t v = all ? i : la[i];
+            const uint32_t w0 = __ldcg(a.gd32 + v), old = all ? 0u : __ldcg(a.topw + v);
+            int32_t x = g32_sink(w0) ? v : g32_ptr(w0);
+            bool top = g32_none(w0), odd = g32_sink(w0) && (w0 & 1u);
+            if (top && x == v && (a.flags[v] & kPriOdd)) c_odd = 1;
+            if (!top && !g32_sink(w0)) {
+                for (int32_t len = 1;; ++len) {
+                    if (len > a.deep_cut) {  // a deep forest: the iteration is abandoned
+                        c_bad = 1;
+                        break;
+                    }
+                    const uint32_t wx = __ldcg(a.gd32 + x);
+                    if (wx & kG32Top) {
+                        top = true;
+                        break;
+                    }
+                    if (g32_sink(wx)) {
+                        odd = wx & 1u;
+                        break;
+                    }
+                    const int32_t nx = g32_ptr(wx);
+                    if (nx <= x) break;  // g-chains rise (a guard, never taken)
+                    x = nx;
+                }
+                if (top) __stcg(a.gd32 + v, w0 | kG32Top);
+            }
+            const uint32_t tw = top ? kG32Top : (odd ? kTopOdd : 0u) | (uint32_t)x;
+            if (all) {  // everyone is evaluated: no queues
+                __stcg(a.topw + v, tw);
+                continue;
+            }
+            const bool changed = tw != old;
+            if (changed) __stcg(a.topw + v, tw);
+            const int32_t e0 = ls[i], em = e0 + (lc[i] & 0xffff), e1 = even_full ? em : e0 + (lc[i] >> 16);
+            for (int32_t e = e0; e < e1; e += 4) {
+                int32_t y[4];
+                bool want[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) y[j] = e + j < e1 ? a.rv_src[e + j] : -1;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    want[j] = y[j] >= 0 && (changed || (__ldcg((e + j < em ? a.omark : a.emark) + y[j]) & kMarkTie));
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    want[j] = want[j] && claim_byte(e + j < em ? a.omark : a.emark, y[j], kMarkQueued);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (!want[j]) continue;
+                    if (e + j < em) {
+                        const int32_t p = atomicAdd(&c_q, 1);
+                        if (p < kIncQueue) {
+                            lq[p] = y[j];
+                        } else {
+                            atomicAdd(&c_spill, 1);
+                            __stcg(a.qlist + atomicAdd(&a.st->n_q, 1), y[j]);
+                        }
+                    } else {
+                        const int32_t p = atomicAdd(&c_e, 1);
+                        if (p < kIncEven) le[p] = y[j];
+                    }
+                }
+            }
+        }
+        if (tid == 0) c_s = 0;
+        const int2 bad_odd = exchange(&c_bad, &c_odd);
+        if (bad_odd.x) {  // the iteration is abandoned
+            if (t0 == 0) a.cnt->deep = 1;
+            ++iters;
+            break;
+        }
+        // Odd's pass; the switched vertices are the next iteration's seeds
+        auto odd_vertex = [&](int32_t v) {
+            bool tie;
+            const bool sw = inc_switch<1>(a, v, &tie);
+            a.omark[v] = tie ? kMarkTie : 0;
+            if (!sw) return;
+            const int32_t p = atomicAdd(&c_s, 1);
+            if (p < kIncSet) la[p] = v;
+        };
+        if (all) {
+            for (int32_t v = t0; v < a.n; v += T)
+                if ((a.flags[v] & (kOwnerOdd | kSinkSlot)) == kOwnerOdd) odd_vertex(v);
+        } else {
+            const int32_t nq = min(c_q, kIncQueue), spill = __ldcg(&a.st->n_q);
+            for (int32_t i = tid; i < nq; i += kIncThreads) odd_vertex(lq[i]);
+            for (int32_t i = t0; i < spill; i += T) odd_vertex(__ldcg(a.qlist + i));
+        }
+        // (a block that switched more than it can hold makes the next iteration a full one)
+        __syncthreads();
+        if (tid == 0 && c_s > kIncSet) c_s = kIncBig;
+        if (tid == 0) c_bad = c_e > kIncEven;
+        const int2 odd_sum = exchange(&c_s, &c_bad);
+        ns = odd_sum.x;
+        nsl = c_s;
+        even_full |= odd_sum.y != 0;
+        int32_t nse = 0;
+        if (ns == 0 && a.even) {
+            if (!a.whole && (even_full || a.reset)) {  // Even's pass over its view; it counts this iteration
+                mode = kIncEvenOnly;
+                if (t0 == 0 && bad_odd.y) a.gst->nodd = 1;
+                break;
+            }
+            auto even_vertex = [&](int32_t v) {
+                bool tie;
+                const bool sw = inc_switch<0>(a, v, &tie);
+                a.emark[v] = tie ? kMarkTie : 0;
+                if (!sw) return;
+                const int32_t p = atomicAdd(&c_s, 1);
+                if (p < kIncSet) la[p] = v;
+            };
+            if (even_full) {
+                for (int32_t v = t0; v < a.n; v += T)
+                    if (!(a.flags[v] & (kOwnerOdd | kSinkSlot))) even_vertex(v);
+            } else {
+                for (int32_t i = tid; i < c_e; i += kIncThreads) even_vertex(le[i]);
+            }
+            __syncthreads();
+            if (tid == 0 && c_s > kIncSet) c_s = kIncBig;
+            nse = exchange(&c_s, &c_zero).x;
+            nsl = c_s;
+            even_full = false;
+            __syncthreads();
+            if (tid == 0) c_e = 0;
+        }
+        // bookkeeping (as k_bookkeep)
+        fresh = false;
+        ++iters;
+        ++gs.inner;
+        if (bad_odd.y) gs.phase = kPhaseOddCycle;
+        else if (ns == 0) {
+            if (nse == 0) gs.phase = kPhaseDone;
+            else {
+                ++gs.major;
+                ns = nse;
+                if (a.reset) {  // Odd restarts from its first edges
+                    for (int32_t v = t0; v < a.n; v += T)
+                        if ((a.flags[v] & (kOwnerOdd | kSinkSlot)) == kOwnerOdd) __stcg(a.strat + v, a.tgt[a.off[v]]);
+                    fresh = true;
+                    cl.sync();
+                }
+            }
+        }
+        if (gs.phase == kPhaseActive && gs.inner >= a.cap) gs.phase = kPhaseTimeout;
+        done = gs.phase != kPhaseActive;
+    }
+    cl.sync();  // no block writes this one's shared memory, or reads the state below, any more
+    if (t0 == 0) {
+        a.gst->phase = gs.phase;
+        a.gst->inner = gs.inner;
+        a.gst->major = gs.major;
+        a.gst->sw_odd = a.gst->sw_even = a.gst->reset = 0;
+        a.gactive[0] = gs.phase == kPhaseActive;
+        a.st->mode = mode;
+        a.st->even_full = even_full;
+        *a.loop_iters += iters;
+    }
+}
+
+// In-degree of every id: all edges in the low half, Odd's in the high half.
+template <typename OffT>
+__global__ void __launch_bounds__(kBlock) k_rv_count(int32_t n, const OffT* __restrict__ off,
+                                                     const int32_t* __restrict__ tgt,
+                                                     const uint8_t* __restrict__ flags, int odd_only,
+                                                     unsigned long long* __restrict__ deg) {
+    for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+        const bool odd = (flags[v] & kOwnerOdd) != 0;
+        if (odd_only && !odd) continue;
+        const unsigned long long one = odd ? (1ull << 32) + 1ull : 1ull;
+        const OffT e1 = off[v + 1];
+        for (OffT e = off[v]; e < e1; ++e) atomicAdd(deg + tgt[e], one);
+    }
+}
+
+// List bounds from the scanned in-degrees (start in rv[].x), and the fill
+// cursors (Odd's, Even's) in place of the degrees.
+__global__ void __launch_bounds__(kBlock) k_rv_bounds(int32_t n, const int32_t* __restrict__ start, uint64_t* deg,
+                                                      int2* __restrict__ rv) {
+    for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v <= n; v += gridDim.x * blockDim.x) {
+        const int32_t s = start[v];
+        const int2 r = make_int2(s, v < n ? s + (int32_t)(deg[v] >> 32) : s);
+        rv[v] = r;
+        if (v < n) reinterpret_cast<int2*>(deg)[v] = r;
+    }
+}
+
+template <typename OffT>
+__global__ void __launch_bounds__(kBlock) k_rv_fill(int32_t n, const OffT* __restrict__ off,
+                                                    const int32_t* __restrict__ tgt,
+                                                    const uint8_t* __restrict__ flags, int odd_only,
+                                                    int2* __restrict__ cur, int32_t* __restrict__ rv_src) {
+    for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+        const bool odd = (flags[v] & kOwnerOdd) != 0;
+        if (odd_only && !odd) continue;
+        const OffT e1 = off[v + 1];
+        for (OffT e = off[v]; e < e1; ++e) {
+            int2* c = cur + tgt[e];
+            rv_src[atomicAdd(odd ? &c->x : &c->y, 1)] = v;
+        }
+    }
+}
+
+}  // namespace
+
+bool inc_applies(const pg_game* g) { return !g->vgame && g->ngames == 1 && g->off != nullptr && !g->cv; }
+
+pg_status build_reverse(pg_game* g, int64_t odd_edges) {
+    if (g->rv) return PG_OK;
+    pg_ctx* ctx = g->ctx;
+    cudaStream_t s = ctx->stream;
+    const int32_t n = g->n;
+    // packed games take no incremental iterations: their lists hold Odd's edges only (the marks of k_classify)
+    const int odd_only = inc_applies(g) ? 0 : 1;
+    const size_t edges = (size_t)(odd_only ? odd_edges : g->m), mark_bytes = ((size_t)n + 16) & ~(size_t)15;
+    PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->rv, sizeof(int2) * ((size_t)n + 1), s));
+    PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->rv_src, sizeof(int32_t) * std::max<size_t>(edges, 1), s));
+    PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->omark, mark_bytes, s));
+    PG_CUDA_TRY(ctx, cudaMemsetAsync(g->omark, 0, mark_bytes, s));
+    if (!odd_only) {
+        PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->emark, mark_bytes, s));
+        PG_CUDA_TRY(ctx, cudaMemsetAsync(g->emark, 0, mark_bytes, s));
+        if (!g->inc) PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->inc, sizeof(IncState), s));
+    }
+    // the valuation's scratch is free before a loop: degrees and cursors in gd, the scan's output in hugelist/coff
+    unsigned long long* deg = (unsigned long long*)g->gd;
+    const unsigned grid = grid_for(n);
+    PG_CUDA_TRY(ctx, cudaMemsetAsync(deg, 0, sizeof(uint64_t) * (size_t)n, s));
+    if (g->off64) k_rv_count<int64_t><<<grid, kBlock, 0, s>>>(n, g->off64, g->tgt, g->flags, odd_only, deg);
+    else k_rv_count<int32_t><<<grid, kBlock, 0, s>>>(n, g->off, g->tgt, g->flags, odd_only, deg);
+    PG_CUDA_TRY(ctx, exclusive_scan_low32(g->gd, g->coff, n, g->scan_tmp, g->scan_tmp_bytes, s));
+    k_rv_bounds<<<grid, kBlock, 0, s>>>(n, g->coff, g->gd, g->rv);
+    if (g->off64)
+        k_rv_fill<int64_t><<<grid, kBlock, 0, s>>>(n, g->off64, g->tgt, g->flags, odd_only, (int2*)g->gd, g->rv_src);
+    else
+        k_rv_fill<int32_t><<<grid, kBlock, 0, s>>>(n, g->off, g->tgt, g->flags, odd_only, (int2*)g->gd, g->rv_src);
+    PG_CUDA_TRY(ctx, cudaGetLastError());
+    ctx->launches += 6;
+    return PG_OK;
+}
+
+int32_t inc_max_seeds(const pg_game* g) { return std::max(1, std::min(g->n / kIncSeedShare, kIncSeeds)); }
+
+static int inc_cluster_for(int want) {
+    cudaFuncSetAttribute(k_inc, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaFuncSetAttribute(k_inc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kIncShared);
+    for (int c = want; c > 1; c >>= 1) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(c);
+        cfg.blockDim = dim3(kIncThreads);
+        cfg.dynamicSmemBytes = kIncShared;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = c;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int k = 0;
+        if (cudaOccupancyMaxActiveClusters(&k, k_inc, &cfg) == cudaSuccess && k > 0) return c;
+        cudaGetLastError();
+    }
+    return 1;
+}
+
+pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole) {
+    pg_ctx* ctx = g->ctx;
+    IncArgs a = {};
+    a.n = g->n;
+    a.sink0 = g->sink0;
+    a.off = g->off;
+    a.tgt = g->tgt;
+    a.flags = g->flags;
+    a.rv = g->rv;
+    a.rv_src = g->rv_src;
+    a.strat = g->strat;
+    a.gd32 = g->gd32;
+    a.topw = (uint32_t*)g->wgt;
+    a.omark = g->omark;
+    a.emark = g->emark;
+    // lists in the valuation's scratch, free during a loop
+    a.alist = g->plist;
+    a.qlist = g->hugelist;
+    a.gst = g->gst;
+    a.cnt = g->cnt;
+    a.st = g->inc;
+    a.gactive = g->gactive;
+    a.loop_iters = g->loop_iters;
+    a.cap = cap;
+    a.whole = whole ? 1 : 0;
+    a.even = even ? 1 : 0;
+    a.reset = even && g->reset_tau ? 1 : 0;
+    a.deep_cut = g->tune.deep_cut;
+    a.deep_fallback = ctx->deep_fallback ? 1 : 0;
+    int want = kIncCluster;
+    if (whole)
+        while (want > 1 && (int64_t)want * kIncThreads / 2 >= g->n) want >>= 1;
+    if (!g->inc_cluster) g->inc_cluster = inc_cluster_for(kIncCluster);
+    const int c = std::min(want, g->inc_cluster);
+    a.max_seeds = std::min(whole ? std::max(1, g->n / kIncWholeShare) : inc_max_seeds(g), c * (kIncSet / 2));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(c);
+    cfg.blockDim = dim3(kIncThreads);
+    cfg.dynamicSmemBytes = kIncShared;
+    cfg.stream = ctx->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = c;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    PG_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, k_inc, a));
+    ctx->launches += 1;
+    return PG_OK;
+}
+
+}  // namespace pg

@@ -78,6 +78,7 @@ struct Counters {
     int32_t n_huge;      // parents ranked by the id-ordered scan
     int32_t n_big;       // parents ranked by one block each
     int32_t n_switch;    // switched vertices in the last switching pass (all games)
+    int32_t n_list;      // vertices switched since the valuation, listed for k_inc as far as it takes them
     int32_t err;         // device-side error bits (kErr*)
     int32_t sink_rank;   // rank of game 0's sink (its empty valuation)
     uint32_t bar_count;  // software grid barrier
@@ -92,6 +93,23 @@ struct Counters {
     int32_t rs_rounds;    //   pointer-jumping rounds over the rulers
     int32_t rs_buf;       //   the buffer holding the rulers' suffix sums
 };
+// State of the incremental iterations (pg_inc.cu), kept across the loop's launches.
+struct IncState {
+    int32_t mode;       // what the loop's next full body is for (kIncFull, kIncEvenOnly)
+    int32_t even_full;  // the next Even pass evaluates every Even vertex
+    int32_t n_q;        // k_inc: Odd's queue beyond the blocks' own
+};
+// Games of up to this many ids run their whole loop in one launch of k_inc (41k ids: 17-32 us for an iteration
+// over all ids, against 45 us for the passes of a full iteration as graph nodes; they grow with the ids, and
+// the passes barely do until 1M).
+constexpr int32_t kIncWhole = 1 << 16;
+constexpr int32_t kIncFull = 0;      // a whole iteration
+constexpr int32_t kIncEvenOnly = 1;  // the valuation is current and Odd has nothing to switch: Even's pass only
+
+// omark[v], emark[v] (the vertices of one player by id)
+constexpr uint8_t kMarkTie = 1;     // the last decision compared chains, or (Odd) a successor's top word changed
+constexpr uint8_t kMarkQueued = 2;  // k_inc: in its player's queue
+
 constexpr int32_t kErrJumpRounds = 1;   // pointer jumping exceeded its round cap
 constexpr int32_t kErrBarrier = 2;      // a grid barrier waited past its spin limit
 constexpr int32_t kErrRulers = 4;       // the list ranking's rulers overflowed their scratch, or a sublist never ended
@@ -119,6 +137,9 @@ extern const char* const kKernelNames[KID_COUNT];
 cudaError_t exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, int64_t* total_dev, void* tmp,
                                size_t tmp_bytes, cudaStream_t s);
 size_t scan_tmp_bytes(int64_t n);
+// Exclusive scan of the low halves of 64-bit words.
+cudaError_t exclusive_scan_low32(const uint64_t* in, int32_t* out, int64_t n, void* tmp, size_t tmp_bytes,
+                                 cudaStream_t s);
 // Exclusive scan of 0/1 bytes.
 cudaError_t exclusive_scan_u8(const uint8_t* in, int32_t* out, int64_t n, void* tmp, size_t tmp_bytes,
                               cudaStream_t s);
@@ -253,7 +274,7 @@ struct pg_game {
     int coop_blocks = 0;         // co-resident blocks for the cooperative kernels
     int chain1_blocks = 0;       // k_chain1 blocks resident at once (0: one block per 8 tiles)
     void* stage = nullptr;       // staging for host outputs
-    int64_t* loop_iters = nullptr;  // [1] iterations run by the device-side loop
+    int64_t* loop_iters = nullptr;  // [2] iterations and loop bodies run by the device-side loop
     // instantiated loop graphs: [0] inner loop only, [1] both players; built for loop_cap[i]
     cudaGraphExec_t loop_exec[2] = {nullptr, nullptr};
     int64_t loop_cap[2] = {0, 0};
@@ -270,13 +291,16 @@ struct pg_game {
     int32_t* pl_off[2] = {nullptr, nullptr};
     int32_t* pl_tgt[2] = {nullptr, nullptr};
     int64_t pl_n[2] = {0, 0};
-    // built with the views: Odd's reverse view (for every id t, rv_src[rv_off[t] .. rv_off[t+1]) are the
-    // positions in Odd's view of the vertices with an edge to t) and omark (one byte per position of Odd's
-    // view, zero padded to a multiple of 16): the vertices that the next Odd switching pass evaluates unless
-    // it is full; the others keep their decision (see k_classify)
-    int32_t* rv_off = nullptr;
+    // the reverse adjacency (build_reverse): for every id t, rv_src[rv[t].x .. rv[t].y) are the Odd vertices
+    // with an edge to t and rv_src[rv[t].y .. rv[t+1].x) the Even ones (none in packed games); omark (one byte
+    // per id, zero padded to a multiple of 16): the Odd vertices that the next Odd switching pass evaluates
+    // unless it is full, the others keep their decision (see k_classify); emark: Even's tie marks (see k_inc)
+    int2* rv = nullptr;
     int32_t* rv_src = nullptr;
     uint8_t* omark = nullptr;
+    uint8_t* emark = nullptr;
+    pg::IncState* inc = nullptr;  // incremental iterations (pg_inc.cu; single games)
+    int inc_cluster = 0;          // blocks of their cluster (0: not yet asked)
     // ruling-set ranks (pg_deep.cu), for games whose g-forest is deep
     bool deep_mode = false;      // every valuation of the current call takes the ruling-set path
     bool val_deep = false;       // the last valuation took it (its depths are written; no depth pass)
@@ -398,6 +422,13 @@ pg_status enqueue_switch_cmp(pg_game* g, int player);
 pg_status finish_loop(pg_game* g);
 // Builds the switching players' views (pl_*) if they are missing; not under stream capture.
 pg_status build_player_split(pg_game* g);
+// Incremental iterations (pg_inc.cu): whether the game takes them, the reverse adjacency they and the marks
+// use (odd_edges: the edges of Odd's vertices, for packed games), one launch of k_inc. whole: the launch is
+// the entire loop; otherwise it follows a full iteration whose passes listed at most inc_max_seeds switches.
+bool inc_applies(const pg_game* g);
+pg_status build_reverse(pg_game* g, int64_t odd_edges);
+int32_t inc_max_seeds(const pg_game* g);
+pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole);
 // K1 alone (counters cleared, nearest-greater walks and pointer jumping with walk lengths).
 pg_status enqueue_k1(pg_game* g);
 // The valuation through the ruling-set ranks of an Euler tour (pg_deep.cu): cls, depth, key, dom.

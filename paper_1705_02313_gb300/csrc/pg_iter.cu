@@ -194,15 +194,8 @@ __global__ void __launch_bounds__(kBlock) k_jump_coop(const int32_t* __restrict_
 }
 
 // Compare-mode K1 (loop iterations that compare valuations): the same walks
-// and jumps with 4-byte g-words only. A word with both the none and the sink
-// bit set is pending: its low bits are a jump pointer (every vertex strictly
-// between v and it on the play is below v, and so is the pointer). A word
-// with only the sink bit (g(v) is the game's sink slot, which the word does
-// not repeat) carries v's priority parity in bit 0, so that the vertex that
-// ends a chain gives its top's parity with no further read.
-constexpr uint32_t kG32Pend = kG32None | kG32Sink;
-__device__ inline bool g32_pending(uint32_t w) { return (w & kG32Pend) == kG32Pend; }
-__device__ inline uint32_t g32_sink_word(uint8_t fl) { return kG32Sink | ((fl & kPriOdd) ? 1u : 0u); }
+// and jumps with 4-byte g-words only (kG32Pend: a word that is still a jump
+// pointer; a sink word carries its vertex's parity).
 
 // Packed games: a warp tile of consecutive ids inside one game that is no
 // longer active is skipped by the loop's chain passes (its words are not read
@@ -221,7 +214,9 @@ __global__ void __launch_bounds__(kBlock, 2048 / kBlock) k_walk_cmp(int32_t n, c
                                                      const int32_t* __restrict__ vgame,
                                                      const int32_t* __restrict__ gsink, int32_t sink0,
                                                      uint32_t* __restrict__ gd32, int32_t* __restrict__ more,
-                                                     int32_t* more_count, const GameState* __restrict__ gst) {
+                                                     int32_t* more_count, const GameState* __restrict__ gst,
+                                                     const IncState* __restrict__ inc) {
+    if (!BATCH && inc && inc->mode == kIncEvenOnly) return;  // the valuation is current
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t tile = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; (tile * 32 * ILP) < n;
@@ -1163,13 +1158,18 @@ __global__ void __launch_bounds__(kBlock) k_switch(int32_t n, int player, const 
 // player switched (or, for best responses, when Odd did not), count a major
 // iteration when Even switched, stop at the cap. Counts the games still active.
 // With reset_mode, a game whose Even player switched is marked for k_reset_odd.
+// inc: the state of the incremental iterations that may follow (one game).
 __global__ void k_bookkeep(int32_t ngames, GameState* gst, int64_t cap, int even_phase, int reset_mode,
-                           int32_t* gactive, const Counters* cnt) {
+                           int32_t* gactive, const Counters* cnt, IncState* inc) {
     if (cnt->deep) return;  // an abandoned iteration: nothing counted, no game active (the loop stops)
     int32_t act = 0;
     for (int32_t gi = blockIdx.x * blockDim.x + threadIdx.x; gi < ngames; gi += gridDim.x * blockDim.x) {
         GameState st = gst[gi];
         st.reset = 0;
+        if (inc) {  // one game: Even's marks are exact after an Even pass, and not kept by a full iteration
+            inc->mode = kIncFull;
+            inc->even_full = !(even_phase && st.sw_odd == 0);
+        }
         if (st.phase == kPhaseActive) {
             st.inner += 1;
             if (st.nodd > 0) st.phase = kPhaseOddCycle;
@@ -1222,16 +1222,6 @@ __global__ void __launch_bounds__(kBlock) k_reset_odd(int32_t n, const OffT* __r
 // each other. The dense ranks, depths and classes of the outputs come from a
 // full valuation after the loop.
 
-// After k_classify, bit 31 of a g-word marks a TOP vertex (its play ends in
-// a cycle); finite words are unchanged (bit 30: g(v) is the game's sink slot).
-constexpr uint32_t kG32Top = 0x80000000u;
-// k_classify also writes one "top word" per vertex: bit 31 = TOP; for a finite
-// vertex bits 0..29 = its top, the last vertex of its g-chain below the sink
-// slot (a child of the sink in the g-forest), and bit 30 = that top's priority
-// is odd.
-constexpr uint32_t kTopOdd = 0x40000000u;
-__device__ inline int32_t top_id(uint32_t t) { return (int32_t)(t & 0x3fffffffu); }
-
 // Class and top of every vertex from its g-chain: a chain that ends at a
 // "none" vertex (above its whole infinite future) or passes a vertex already
 // marked TOP is TOP, and its g-word gets bit 31; a chain that reaches the sink
@@ -1243,8 +1233,8 @@ __device__ inline int32_t top_id(uint32_t t) { return (int32_t)(t & 0x3fffffffu)
 // (sigma not admissible).
 //
 // With omark, a top word is written only when it differs from the previous
-// iteration's, and then every Odd vertex with an edge to v (rv_off, rv_src)
-// is marked for the next Odd switching pass. An Odd vertex decides from its
+// iteration's, and then every Odd vertex with an edge to v (rv, rv_src) is
+// marked for the next Odd switching pass. An Odd vertex decides from its
 // successors' top words alone, unless two finite successors with the best
 // top tie (a chain comparison, which leaves its mark set): so an unmarked
 // vertex, none of whose successors changed since it was last evaluated,
@@ -1255,8 +1245,9 @@ template <int ILP = kIlp>
 __global__ void __launch_bounds__(kBlock, 2048 / kBlock)
     k_classify(int32_t n, uint32_t* gd32, const uint8_t* __restrict__ flags, uint32_t* __restrict__ topw,
                const int32_t* __restrict__ vgame, GameState* gst, Counters* cnt, int32_t deep_cut,
-               const int32_t* __restrict__ rv_off, const int32_t* __restrict__ rv_src, uint8_t* omark,
-               const int32_t* __restrict__ full) {
+               const int2* __restrict__ rv, const int32_t* __restrict__ rv_src, uint8_t* omark,
+               const int32_t* __restrict__ full, const IncState* __restrict__ inc) {
+    if (inc && inc->mode == kIncEvenOnly) return;  // the valuation is current
     if (cnt->err || cnt->deep) return;  // unfinished jumping: g-words may point downwards, no chain walk would end
     if (omark && *full) omark = nullptr;  // the next Odd pass evaluates every Odd vertex: no marks
     const int lane = threadIdx.x & 31;
@@ -1317,71 +1308,11 @@ __global__ void __launch_bounds__(kBlock, 2048 / kBlock)
                 topw[v[j]] = tw;
             } else if (tw != ot[j]) {
                 topw[v[j]] = tw;
-                const int32_t e1 = rv_off[v[j] + 1];
-                for (int32_t e = rv_off[v[j]]; e < e1; ++e) omark[rv_src[e]] = 1;
+                const int2 r = rv[v[j]];
+                for (int32_t e = r.x; e < r.y; ++e) omark[rv_src[e]] = kMarkTie;
             }
         }
     }
-}
-
-// Compares the valuations of two finite vertices u and w of one game with the
-// same top: walk both g-chains (words wu, ww) upwards, always advancing the
-// smaller id, until they meet (at the top at the latest). The larger of the
-// last two vertices passed below the meeting point is the largest vertex of
-// the symmetric difference of the two plays; its side is better for Even
-// when its priority is even. Returns > 0 if Val(u) is better for Even, < 0 if
-// worse, 0 if u == w. g(x) > x for every vertex below the top, so each step
-// raises a or b.
-__device__ inline int cmp_walk(int32_t u, int32_t w, const uint32_t* __restrict__ gd32,
-                               const uint8_t* __restrict__ flags) {
-    int32_t a = u, b = w, pa = -1, pb = -1;
-    uint32_t wa = 0, wb = 0;
-    if (a != b) {
-        wa = gd32[a];
-        wb = gd32[b];
-    }
-    while (a != b) {
-        if (a < b) {
-            pa = a;
-            a = g32_ptr(wa);
-            if (a <= pa) return 0;  // g-chains rise (a guard that keeps every walk finite; never taken)
-            wa = gd32[a];
-        } else {
-            pb = b;
-            b = g32_ptr(wb);
-            if (b <= pb) return 0;
-            wb = gd32[b];
-        }
-    }
-    if (pa == pb) return 0;  // u == w
-    const bool u_side = pa > pb;
-    const bool even = !(flags[u_side ? pa : pb] & kPriOdd);
-    return u_side == even ? 1 : -1;
-}
-
-// Order of the valuations of u and w (vertices of one game, with their top
-// words tu, tw): > 0 if Val(u) is better for Even than Val(w), < 0 if worse,
-// 0 if equal. TOP is above every finite valuation and equal to TOP. Finite
-// plays with different tops differ above everything else at the larger top,
-// which decides by its parity; with the same top the chains are walked.
-__device__ inline int cmp_val(int32_t u, uint32_t tu, int32_t w, uint32_t tw, const uint32_t* __restrict__ gd32,
-                              const uint8_t* __restrict__ flags) {
-    const int xu = (tu & kG32Top) ? 1 : 0, xw = (tw & kG32Top) ? 1 : 0;
-    if (xu | xw) return xu - xw;
-    const int32_t hu = top_id(tu), hw = top_id(tw);
-    if (hu != hw) {
-        const bool u_side = hu > hw;
-        const bool even = !((u_side ? tu : tw) & kTopOdd);
-        return u_side == even ? 1 : -1;
-    }
-    return cmp_walk(u, w, gd32, flags);
-}
-
-// Against the sink's empty valuation: the top of a finite play is its largest
-// vertex, so Val(u) is better for Even exactly when that top is even.
-__device__ inline int cmp_sink(uint32_t tu) {
-    if (tu & kG32Top) return 1;
-    return (tu & kTopOdd) ? -1 : 1;
 }
 
 // K3 with comparisons: as k_switch (one thread per vertex of the switching
@@ -1504,39 +1435,17 @@ __global__ void __launch_bounds__(kBlock) k_pl_copy(int32_t np, const int32_t* _
     }
 }
 
-// Odd's reverse view: the in-degree of every id from Odd's edges, then each
-// edge's source (its position in Odd's view) at the next free slot of its
-// target, cur[t] starting at rv_off[t] (the order within a list is arbitrary;
-// the lists only mark).
-__global__ void __launch_bounds__(kBlock) k_rv_count(int32_t np, const int32_t* __restrict__ poff,
-                                                     const int32_t* __restrict__ ptgt, int32_t* __restrict__ cnt) {
-    const int32_t m = poff[np];
-    for (int32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < m; e += gridDim.x * blockDim.x)
-        atomicAdd(cnt + ptgt[e], 1);
-}
-
-__global__ void __launch_bounds__(kBlock) k_rv_fill(int32_t np, const int32_t* __restrict__ poff,
-                                                    const int32_t* __restrict__ ptgt, int32_t* __restrict__ cur,
-                                                    int32_t* __restrict__ rv_src) {
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < np; i += gridDim.x * blockDim.x) {
-        const int32_t e1 = poff[i + 1];
-        for (int32_t e = poff[i]; e < e1; ++e) rv_src[atomicAdd(cur + ptgt[e], 1)] = i;
-    }
-}
-
-// One vertex of k_switch_cmp_pl: view position i (vertex vid[i]), with the
-// rules of k_switch_cmp. Returns whether it switched; *tie tells whether the
-// decision took a chain comparison (two finite successors with the best top
-// so far), *gi is its game. Vertices of games that do not switch this player
-// now are left alone (tie set, no switch).
+// One vertex of k_switch_cmp_pl, its edges at tgt[e0 .. e1), with the rules of
+// k_switch_cmp. Returns whether it switched; *tie tells whether the decision
+// took a chain comparison (two finite successors with the best top so far),
+// *gi is its game. Vertices of games that do not switch this player now are
+// left alone (tie set, no switch).
 template <int PLAYER, bool BATCH>
-__device__ inline bool switch_at(int32_t i, const int32_t* __restrict__ vid,
-                                 const int32_t* __restrict__ poff, const int32_t* __restrict__ ptgt,
+__device__ inline bool switch_at(int32_t v, int64_t e0, int64_t e1, const int32_t* __restrict__ tgt,
                                  const uint8_t* __restrict__ flags, const uint32_t* __restrict__ gd32,
                                  const uint32_t* __restrict__ topw, const int32_t* __restrict__ vgame,
                                  const int32_t* __restrict__ gsink, int32_t sink0, const GameState* gst,
                                  int32_t* strat, bool* tie_out, int32_t* gi_out) {
-    const int32_t v = vid[i];
     const int32_t gi = BATCH ? vgame[v] : 0;
     *gi_out = gi;
     *tie_out = true;
@@ -1544,28 +1453,28 @@ __device__ inline bool switch_at(int32_t i, const int32_t* __restrict__ vid,
         const GameState st = gst[gi];
         if (st.phase != kPhaseActive || (PLAYER == 0 && st.sw_odd != 0)) return false;
     }
-    const int32_t e0 = poff[i], e1 = poff[i + 1];
     const int32_t cur = strat[v];
     const int32_t sk = PLAYER == 0 ? (BATCH ? gsink[gi] : sink0) : -1;
     int32_t best = sk;  // Even: the sink first; Odd: none yet
     uint32_t tbest = 0;
     bool cur_top = false, tie = false;
-    for (int32_t e = e0; e < e1; e += 4) {
+    const int32_t* ptgt = tgt + e0;
+    const int32_t k = (int32_t)(e1 - e0);
+    for (int32_t e = 0; e < k; e += 4) {
         int32_t t[4];
         uint32_t tt[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) t[j] = e + j < e1 ? ptgt[e + j] : -1;
+        for (int j = 0; j < 4; ++j) t[j] = e + j < k ? ptgt[e + j] : -1;
 #pragma unroll
         for (int j = 0; j < 4; ++j) tt[j] = t[j] >= 0 ? topw[t[j]] : 0u;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             if (t[j] < 0) continue;
             if (PLAYER == 0 && t[j] == cur) cur_top = (tt[j] & kG32Top) != 0;
+            tie |= best != sk && !((tt[j] | tbest) & kG32Top) && top_id(tt[j]) == top_id(tbest);
             bool take;
-            if (PLAYER == 1) {
-                tie |= best >= 0 && !((tt[j] | tbest) & kG32Top) && top_id(tt[j]) == top_id(tbest);
-                take = best < 0 || cmp_val(t[j], tt[j], best, tbest, gd32, flags) < 0;
-            } else take = (best == sk ? cmp_sink(tt[j]) : cmp_val(t[j], tt[j], best, tbest, gd32, flags)) > 0;
+            if (PLAYER == 1) take = best < 0 || cmp_val(t[j], tt[j], best, tbest, gd32, flags) < 0;
+            else take = (best == sk ? cmp_sink(tt[j]) : cmp_val(t[j], tt[j], best, tbest, gd32, flags)) > 0;
             if (take) {
                 best = t[j];
                 tbest = tt[j];
@@ -1576,6 +1485,36 @@ __device__ inline bool switch_at(int32_t i, const int32_t* __restrict__ vid,
     const bool sw = best != cur && (PLAYER == 0 ? !cur_top : !(tbest & kG32Top));
     if (sw) strat[v] = best;
     return sw;
+}
+
+// The vertices that a switching pass switched, for k_inc: each warp gathers
+// its own in shared memory and appends kSwBuf - 31 or more of them at a time
+// (one counter step per switched vertex, or per warp round, would serialise a
+// pass that switches millions). Entries beyond cap are only counted.
+constexpr int kSwBuf = 128;
+__device__ inline void list_flush(const int32_t* buf, int32_t have, int32_t* list, int32_t* counter, int32_t cap) {
+    if (!have) return;
+    const int lane = threadIdx.x & 31;
+    int32_t base = 0;
+    if (lane == 0) base = atomicAdd(counter, have);
+    base = __shfl_sync(kFull, base, 0);
+    for (int32_t j = lane; j < have; j += 32)
+        if (base + j < cap) list[base + j] = buf[j];
+    __syncwarp();
+}
+
+// All 32 lanes call this; have (the entries held) stays uniform over the warp.
+__device__ inline void list_push(bool sw, int32_t v, int32_t* buf, int32_t* have, int32_t* list, int32_t* counter,
+                                 int32_t cap) {
+    const unsigned m = __ballot_sync(kFull, sw);
+    if (!m) return;
+    if (sw) buf[*have + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = v;
+    *have += __popc(m);
+    __syncwarp();
+    if (*have > kSwBuf - 32) {
+        list_flush(buf, *have, list, counter, cap);
+        *have = 0;
+    }
 }
 
 // A switch counted into its game (packed games: one atomic per group of
@@ -1592,54 +1531,73 @@ __device__ inline void count_switch(bool sw, int32_t gi, GameState* gst, int32_t
 }
 
 // k_switch_cmp over a player's view: thread i takes the player's i-th vertex.
-// With MARKS (Odd's pass; omark holds one byte per view position, zero padded
-// to a multiple of 16), a pass that is not full evaluates only the marked
-// positions and clears the mark of each unless its decision took a chain
-// comparison; a full pass (the first of a call, or after an SI-Reset:
-// *full_flag != 0) evaluates every vertex and sets each mark to that flag.
+// With MARKS (mark holds one byte per id, zero padded to a multiple of 16),
+// Odd's pass, when it is not full, evaluates only the marked vertices (their
+// edges in off, tgt) and clears the mark of each unless its decision took a
+// chain comparison; a full pass (Even's always; Odd's first of a call, or after
+// an SI-Reset: *full_flag != 0) evaluates the whole view and sets each mark to
+// that flag. One game (inc): the switched vertices are listed for k_inc, and
+// nothing is done for Odd when only Even's pass is due.
 // Full occupancy (32 registers): the evaluations wait on their gathers.
 template <int BS, int PLAYER, bool MARKS, bool BATCH>
 __global__ void __launch_bounds__(BS, 2048 / BS) k_switch_cmp_pl(int32_t np, const int32_t* __restrict__ vid,
                                                       const int32_t* __restrict__ poff,
-                                                      const int32_t* __restrict__ ptgt,
+                                                      const int32_t* __restrict__ ptgt, int32_t n,
+                                                      const int32_t* __restrict__ off32,
+                                                      const int64_t* __restrict__ off64,
+                                                      const int32_t* __restrict__ tgt,
                                                       const uint8_t* __restrict__ flags,
                                                       const uint32_t* __restrict__ gd32,
                                                       const uint32_t* __restrict__ topw,
                                                       const int32_t* __restrict__ vgame,
                                                       const int32_t* __restrict__ gsink, int32_t sink0,
                                                       GameState* gst, int32_t* strat, Counters* cnt,
-                                                      uint8_t* omark, const int32_t* __restrict__ full_flag) {
+                                                      uint8_t* mark, const int32_t* __restrict__ full_flag,
+                                                      const IncState* __restrict__ inc, int32_t* list,
+                                                      int32_t list_cap) {
     if (cnt->err || cnt->deep) return;  // unfinished jumping, or a deep forest (the loop stops)
     if (!BATCH) {  // one game: the whole pass is skipped when the game does not switch this player now
         const GameState st = gst[0];
         if (st.phase != kPhaseActive || (PLAYER == 0 && st.sw_odd != 0)) return;
+        if (PLAYER == 1 && inc && inc->mode == kIncEvenOnly) return;
     }
-    const bool full = !MARKS || *full_flag;
+    const bool full = PLAYER == 0 || !MARKS || *full_flag;
+    __shared__ int32_t swbuf[BATCH ? 1 : BS / 32][BATCH ? 1 : kSwBuf];
+    int32_t* mybuf = BATCH ? nullptr : swbuf[threadIdx.x >> 5];
+    int32_t have = 0;
     int32_t nsw = 0;
+    const int lane = threadIdx.x & 31;
     if (full) {
-        for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < np; i += gridDim.x * blockDim.x) {
-            bool tie;
-            int32_t gi;
-            const bool sw = switch_at<PLAYER, BATCH>(i, vid, poff, ptgt, flags, gd32, topw, vgame, gsink, sink0, gst,
-                                                     strat, &tie, &gi);
-            if (MARKS) omark[i] = tie;
-            count_switch<PLAYER, BATCH>(sw, gi, gst, &nsw);
+        for (int32_t i0 = (blockIdx.x * blockDim.x + threadIdx.x) - lane; i0 < np; i0 += gridDim.x * blockDim.x) {
+            const int32_t i = i0 + lane;
+            bool sw = false;
+            int32_t v = 0;
+            if (i < np) {
+                bool tie;
+                int32_t gi;
+                v = vid[i];
+                sw = switch_at<PLAYER, BATCH>(v, poff[i], poff[i + 1], ptgt, flags, gd32, topw, vgame, gsink, sink0,
+                                              gst, strat, &tie, &gi);
+                if (MARKS) mark[v] = tie ? kMarkTie : 0;
+                count_switch<PLAYER, BATCH>(sw, gi, gst, &nsw);
+            }
+            if (!BATCH && list) list_push(sw, v, mybuf, &have, list, &cnt->n_list, list_cap);
         }
-    } else if (MARKS) {
-        // warps take 512 positions at a time: each lane loads 16 marks, the marked positions are listed in
-        // shared memory (a warp scan of the lanes' counts), and the lanes share the list, so a chunk costs
-        // one 16-byte load per lane plus ceil(marked / 32) evaluation rounds
-        __shared__ int32_t list[BS / 32][512];
-        int32_t* mine = list[threadIdx.x >> 5];
-        const int lane = threadIdx.x & 31;
-        const int32_t nch = (np + 511) >> 9;
+    } else if (MARKS && PLAYER == 1) {
+        // warps take 512 ids at a time: each lane loads 16 marks, the marked ids are listed in shared memory (a
+        // warp scan of the lanes' counts), and the lanes share the list, so a chunk costs one 16-byte load per
+        // lane plus ceil(marked / 32) evaluation rounds
+        __shared__ int32_t found[BS / 32][512];
+        int32_t* mine = found[threadIdx.x >> 5];
+        const int32_t nch = (n + 511) >> 9;
         const int32_t nw = (int32_t)((gridDim.x * blockDim.x) >> 5);
         for (int32_t c = (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); c < nch; c += nw) {
             const int32_t q = (c << 9) + 16 * lane;
             uint4 m = make_uint4(0u, 0u, 0u, 0u);
-            if (q < np) m = *reinterpret_cast<const uint4*>(omark + q);
-            const uint32_t mw[4] = {m.x, m.y, m.z, m.w};
-            const int k = __popc(m.x) + __popc(m.y) + __popc(m.z) + __popc(m.w);  // marks are 0 or 1
+            if (q < n) m = *reinterpret_cast<const uint4*>(mark + q);
+            constexpr uint32_t kTies = 0x01010101u * kMarkTie;
+            const uint32_t mw[4] = {m.x & kTies, m.y & kTies, m.z & kTies, m.w & kTies};
+            const int k = __popc(mw[0]) + __popc(mw[1]) + __popc(mw[2]) + __popc(mw[3]);
             int incl = k;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -1653,18 +1611,26 @@ __global__ void __launch_bounds__(BS, 2048 / BS) k_switch_cmp_pl(int32_t np, con
             for (int b = 0; b < 16; ++b)
                 if ((mw[b >> 2] >> (8 * (b & 3))) & 1u) mine[pos++] = q + b;
             __syncwarp();
-            for (int j = lane; j < total; j += 32) {
-                const int32_t i = mine[j];  // < np: the padding is never marked
-                bool tie;
-                int32_t gi;
-                const bool sw = switch_at<PLAYER, BATCH>(i, vid, poff, ptgt, flags, gd32, topw, vgame, gsink, sink0,
-                                                         gst, strat, &tie, &gi);
-                if (!tie) omark[i] = 0;
-                count_switch<PLAYER, BATCH>(sw, gi, gst, &nsw);
+            for (int j0 = 0; j0 < total; j0 += 32) {
+                bool sw = false;
+                int32_t v = 0;
+                if (j0 + lane < total) {
+                    v = mine[j0 + lane];  // an Odd vertex: the padding is never marked
+                    bool tie;
+                    int32_t gi;
+                    const int64_t e0 = off64 ? off64[v] : (int64_t)off32[v];
+                    const int64_t e1 = off64 ? off64[v + 1] : (int64_t)off32[v + 1];
+                    sw = switch_at<PLAYER, BATCH>(v, e0, e1, tgt, flags, gd32, topw, vgame, gsink, sink0, gst, strat,
+                                                  &tie, &gi);
+                    if (!tie) mark[v] = 0;
+                    count_switch<PLAYER, BATCH>(sw, gi, gst, &nsw);
+                }
+                if (!BATCH && list) list_push(sw, v, mybuf, &have, list, &cnt->n_list, list_cap);
             }
             __syncwarp();
         }
     }
+    if (!BATCH && list) list_flush(mybuf, have, list, &cnt->n_list, list_cap);
     block_add(nsw, &cnt->n_switch);
     if (!BATCH) {  // one game: the block totals are the game's
         __shared__ int32_t tot;
@@ -1737,7 +1703,7 @@ pg_status alloc_scratch(pg_game* g) {
     PG_CUDA_TRY(ctx, A((void**)&g->gscan, sizeof(int64_t) * 3 * (size_t)g->ngames));
     PG_CUDA_TRY(ctx, A((void**)&g->gst, sizeof(GameState) * (size_t)g->ngames));
     PG_CUDA_TRY(ctx, A((void**)&g->gactive, 2 * sizeof(int32_t)));
-    PG_CUDA_TRY(ctx, A((void**)&g->loop_iters, sizeof(int64_t)));
+    PG_CUDA_TRY(ctx, A((void**)&g->loop_iters, 2 * sizeof(int64_t)));
     PG_CUDA_TRY(ctx, A((void**)&g->cnt, sizeof(Counters)));
     PG_CUDA_TRY(ctx, cudaMallocHost((void**)&g->hcnt, sizeof(Counters)));
     g->scan_tmp_bytes = scan_tmp_bytes(n + 2) + 64;
@@ -1914,6 +1880,17 @@ pg_status enqueue_switch(pg_game* g, int player) {
     return PG_OK;
 }
 
+// The Odd marks when the loop compares valuations over the players' views
+// (null otherwise: every Odd vertex is evaluated in every pass).
+uint8_t* omark_of(const pg_game* g) {
+    return g->pl_ok && g->omark && !g->cv && !g->tune.loop_ranks && !g->deep_mode ? g->omark : nullptr;
+}
+
+namespace {
+// The incremental iterations' state when the loop's full iterations prepare them (null otherwise).
+IncState* inc_of(const pg_game* g) { return omark_of(g) && g->emark && inc_applies(g) ? g->inc : nullptr; }
+}  // namespace
+
 pg_status enqueue_bookkeeping(pg_game* g, int64_t cap, bool even_phase) {
     pg_ctx* ctx = g->ctx;
     cudaStream_t s = ctx->stream;
@@ -1921,15 +1898,9 @@ pg_status enqueue_bookkeeping(pg_game* g, int64_t cap, bool even_phase) {
     ctx->launches += 1;
     const unsigned b = (unsigned)std::max<int64_t>(1, std::min<int64_t>(((int64_t)g->ngames + kBlock - 1) / kBlock, 1024));
     k_bookkeep<<<b, kBlock, 0, s>>>(g->ngames, g->gst, cap, even_phase ? 1 : 0, g->reset_tau ? 1 : 0, g->gactive,
-                                    g->cnt);
+                                    g->cnt, inc_of(g));
     PG_CUDA_TRY(ctx, cudaGetLastError());
     return PG_OK;
-}
-
-// The Odd marks when the loop compares valuations over the players' views
-// (null otherwise: every Odd vertex is evaluated in every pass).
-uint8_t* omark_of(const pg_game* g) {
-    return g->pl_ok && g->omark && !g->cv && !g->tune.loop_ranks && !g->deep_mode ? g->omark : nullptr;
 }
 
 pg_status enqueue_reset(pg_game* g) {
@@ -1965,7 +1936,7 @@ pg_status enqueue_valuation_cmp(pg_game* g) {
             default: break;
         }
         walk<<<ilp_grid(n), kBlock, 0, s>>>(n, g->strat, g->flags, g->vgame, g->gsink, g->sink0, g->gd32, g->plist,
-                                            &c->n_pending, g->gst);
+                                            &c->n_pending, g->gst, inc_of(g));
     }
     prof_end(g, KID_WALK, 1);
     {
@@ -1981,8 +1952,8 @@ pg_status enqueue_valuation_cmp(pg_game* g) {
     prof_begin(g, KID_CLASSIFY);
     // the top words live in the chain-weight array, which only a full valuation uses
     k_classify<PG_CHAIN_ILP><<<ilp_grid(n), kBlock, 0, s>>>(n, g->gd32, g->flags, (uint32_t*)g->wgt, g->vgame,
-                                                            g->gst, c, g->tune.deep_cut, g->rv_off, g->rv_src,
-                                                            omark_of(g), g->gactive + 1);
+                                                            g->gst, c, g->tune.deep_cut, g->rv, g->rv_src, omark_of(g),
+                                                     g->gactive + 1, inc_of(g));
     prof_end(g, KID_CLASSIFY, 1);
     PG_CUDA_TRY(ctx, cudaGetLastError());
     return PG_OK;
@@ -2001,14 +1972,18 @@ void launch_switch_cmp_bs(pg_game* g, int player) {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device);
         const int64_t wave = (int64_t)std::max(sms, 1) * (2048 / BS);
         const int64_t b = std::max<int64_t>(1, std::min<int64_t>((np + BS - 1) / BS, wave));
-        uint8_t* om = player == 1 ? omark_of(g) : nullptr;
+        IncState* inc = inc_of(g);
+        uint8_t* om = player == 1 ? omark_of(g) : inc ? g->emark : nullptr;
         const bool batch = g->vgame != nullptr;
-        auto kern = player == 0 ? (batch ? k_switch_cmp_pl<BS, 0, false, true> : k_switch_cmp_pl<BS, 0, false, false>)
+        auto kern = player == 0 ? (batch ? k_switch_cmp_pl<BS, 0, false, true>
+                                   : om  ? k_switch_cmp_pl<BS, 0, true, false>
+                                         : k_switch_cmp_pl<BS, 0, false, false>)
                     : om        ? (batch ? k_switch_cmp_pl<BS, 1, true, true> : k_switch_cmp_pl<BS, 1, true, false>)
                                 : (batch ? k_switch_cmp_pl<BS, 1, false, true> : k_switch_cmp_pl<BS, 1, false, false>);
-        kern<<<(unsigned)b, BS, 0, s>>>((int32_t)np, g->pl_vid[player], g->pl_off[player], g->pl_tgt[player],
-                                        g->flags, g->gd32, topw, g->vgame, g->gsink, g->sink0, g->gst, g->strat,
-                                        g->cnt, om, g->gactive + 1);
+        kern<<<(unsigned)b, BS, 0, s>>>((int32_t)np, g->pl_vid[player], g->pl_off[player], g->pl_tgt[player], g->n,
+                                        g->off, g->off64, g->tgt, g->flags, g->gd32, topw, g->vgame, g->gsink,
+                                        g->sink0, g->gst, g->strat, g->cnt, om, g->gactive + 1, inc,
+                                        inc ? g->plist : nullptr, inc ? inc_max_seeds(g) : 0);
         return;
     }
     const int64_t b = std::max<int64_t>(1, std::min<int64_t>(((int64_t)g->n + BS - 1) / BS, 152LL * 64 * kBlock / BS));
@@ -2069,10 +2044,11 @@ pg_status build_player_split(pg_game* g) {
         if (g->pl_tgt[p]) cudaFreeAsync(g->pl_tgt[p], s);
         g->pl_vid[p] = g->pl_off[p] = g->pl_tgt[p] = nullptr;
     }
-    for (void** q : {(void**)&g->rv_off, (void**)&g->rv_src, (void**)&g->omark}) {
-        if (*q) cudaFreeAsync(*q, s);
-        *q = nullptr;
-    }
+    if (g->vgame)  // a server's layout changed (a loaded game's reverse adjacency stays)
+        for (void** q : {(void**)&g->rv, (void**)&g->rv_src, (void**)&g->omark, (void**)&g->emark}) {
+            if (*q) cudaFreeAsync(*q, s);
+            *q = nullptr;
+        }
     int32_t mp_of[2] = {0, 0};
     // the valuation's scratch is free before a loop: marks in kind and cls, positions in coff, degrees in
     // hugelist
@@ -2118,22 +2094,8 @@ pg_status build_player_split(pg_game* g) {
         PG_CUDA_TRY(ctx, cudaGetLastError());
     }
     ctx->launches += 7;
-    {  // Odd's reverse view, counted in hugelist (free again)
-        const int32_t np = (int32_t)g->pl_n[1];
-        int32_t* cnt = g->hugelist;
-        PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->rv_off, sizeof(int32_t) * ((size_t)n + 1), s));
-        PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->rv_src, sizeof(int32_t) * std::max(mp_of[1], 1), s));
-        const size_t mark_bytes = ((size_t)np + 16) & ~(size_t)15;  // read 16 at a time, the padding zero
-        PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->omark, mark_bytes, s));
-        PG_CUDA_TRY(ctx, cudaMemsetAsync(g->omark, 0, mark_bytes, s));
-        PG_CUDA_TRY(ctx, cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)n, s));
-        k_rv_count<<<grid_for(std::max(mp_of[1], 1)), kBlock, 0, s>>>(np, g->pl_off[1], g->pl_tgt[1], cnt);
-        PG_CUDA_TRY(ctx, exclusive_scan_i32(cnt, g->rv_off, n, nullptr, g->scan_tmp, g->scan_tmp_bytes, s));
-        PG_CUDA_TRY(ctx, cudaMemcpyAsync(cnt, g->rv_off, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s));
-        k_rv_fill<<<grid_for(std::max(np, 1)), kBlock, 0, s>>>(np, g->pl_off[1], g->pl_tgt[1], cnt, g->rv_src);
-        PG_CUDA_TRY(ctx, cudaGetLastError());
-        ctx->launches += 5;
-    }
+    pg_status st = build_reverse(g, mp_of[1]);
+    if (st) return st;
     g->pl_ok = true;
     return PG_OK;
 }

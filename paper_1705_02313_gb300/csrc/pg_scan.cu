@@ -60,6 +60,13 @@ struct LoadI32 {
         }
     }
 };
+struct LoadLow32 {
+    const uint64_t* p;
+    __device__ void operator()(int64_t i0, int64_t n, int64_t v[kIpt]) const {
+#pragma unroll
+        for (int k = 0; k < kIpt; ++k) v[k] = i0 + k < n ? (int64_t)(p[i0 + k] & 0xffffffffull) : 0;
+    }
+};
 struct LoadU8 {
     const uint8_t* p;
     __device__ void operator()(int64_t i0, int64_t n, int64_t v[kIpt]) const {
@@ -158,6 +165,11 @@ size_t scan_tmp_bytes(int64_t n) { return (size_t)((n + kTile - 1) / kTile + 2) 
 cudaError_t exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, int64_t* total_dev, void* tmp,
                                size_t tmp_bytes, cudaStream_t s) {
     return scan_impl(LoadI32{in}, n, out, n, total_dev, tmp, tmp_bytes, s);
+}
+
+cudaError_t exclusive_scan_low32(const uint64_t* in, int32_t* out, int64_t n, void* tmp, size_t tmp_bytes,
+                                 cudaStream_t s) {
+    return scan_impl(LoadLow32{in}, n, out, n, nullptr, tmp, tmp_bytes, s);
 }
 
 cudaError_t exclusive_scan_u8(const uint8_t* in, int32_t* out, int64_t n, void* tmp, size_t tmp_bytes,
