@@ -372,7 +372,7 @@ pg_status enqueue_iteration(pg_game* g, int64_t cap, bool even) {
 // game, the incremental iterations that can follow it.
 pg_status enqueue_body(pg_game* g, int64_t cap, bool even) {
     pg_status st = enqueue_iteration(g, cap, even);
-    if (!st && loop_compares(g) && omark_of(g) && inc_applies(g)) st = enqueue_inc(g, cap, even, false);
+    if (!st && inc_of(g)) st = enqueue_inc(g, cap, even, false);
     return st;
 }
 
@@ -541,6 +541,9 @@ pg_status run_loop(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t limit)
     if (runs_whole(g, tm)) {
         pg_status st = build_reverse(g, 0);
         if (st) return st;
+    } else if (g->cv && !tm.on && g->ctx->graphs && inc_applies(g)) {
+        pg_status st = build_reverse(g, 0);
+        if (st) return st;
     } else if (loop_compares(g) && !g->pl_ok) {
         pg_status st = build_player_split(g);
         if (st) return st;
@@ -553,7 +556,8 @@ pg_status run_loop(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t limit)
         int64_t ran = 0;
         pg_status st = run_loop_once(g, cap, even, tm, limit > 0 ? limit - done : 0, &ran);
         if (st) return st;
-        g->last_cmp = loop_compares(g);
+        // (k_inc keeps the keys of a count-vector game, not its classes and walk lengths)
+        g->last_cmp = loop_compares(g) || (g->cv && g->last_graph && inc_of(g));
         if (g->cv || g->deep_mode || !g->hcnt->deep) return PG_OK;
         g->deep_mode = true;
         st = prepare_deep(g);

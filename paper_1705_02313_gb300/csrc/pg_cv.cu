@@ -19,24 +19,13 @@
 //                  consistent (word, weight) pair)
 //   k_chain_cv     classification and key = sum of segment weights along the g-chain
 //   k_switch_cv    the switching rules of Section 3 and Section 4 on the keys
-#include "pg_internal.cuh"
+#include "pg_device.cuh"
 
 namespace pg {
 namespace {
 
-using i128 = __int128;
-
 constexpr unsigned kFullMask = 0xffffffffu;
 constexpr int kIlpCv = 2;  // walks per thread (2 / 3 / 4 / 6: 129.0 / 133.9 / 136.0 / 168.5 ms per 10M 4-priority solve)
-
-__device__ inline i128 top_key() { return (i128)(~(unsigned __int128)0 >> 1); }
-
-__device__ inline int level_of(const Levels& L, int32_t v) {
-    int l = 0;
-#pragma unroll
-    for (int i = 1; i < kMaxLevels; ++i) l += (i < L.n && v >= L.start[i]) ? 1 : 0;
-    return l;
-}
 
 // The walks count the vertices they pass per level in 7-bit fields of one
 // word (a walk passes at most kWalkCap + 1 < 128 vertices in one kernel) and
@@ -53,12 +42,6 @@ __device__ inline i128 weight_of_counts(const Levels& L, uint64_t c) {
         w += ((L.odd_mask >> l) & 1u) ? -d : d;
     }
     return w;
-}
-
-__device__ inline i128 weight_of(const Levels& L, int32_t v) {
-    const int l = level_of(L, v);
-    const i128 w = (i128)1 << L.shift[l];
-    return ((L.odd_mask >> l) & 1u) ? -w : w;
 }
 
 inline unsigned grid_n(int64_t n) {
@@ -140,7 +123,8 @@ __global__ void __launch_bounds__(kBlock) k_walk_cv(int32_t n, Levels L, const i
                                                     uint64_t* __restrict__ gd, uint64_t* __restrict__ gdB,
                                                     uint32_t* __restrict__ gd32, i128* __restrict__ ws,
                                                     i128* __restrict__ wsB, int32_t* __restrict__ more,
-                                                    Counters* cnt) {
+                                                    Counters* cnt, const IncState* __restrict__ inc) {
+    if (inc && inc->mode == kIncEvenOnly) return;  // the keys are current
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t tile = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; tile * 32 * kIlpCv < n;
@@ -358,7 +342,8 @@ __global__ void __launch_bounds__(kBlock) k_chain_cv(int32_t n, const uint32_t* 
                                                      const int32_t* __restrict__ pri, i128* __restrict__ key,
                                                      uint8_t* __restrict__ kind, uint8_t* __restrict__ cls,
                                                      int32_t* __restrict__ dom, int want_dom, GameState* gst,
-                                                     Counters* cnt) {
+                                                     Counters* cnt, const IncState* __restrict__ inc) {
+    if (inc && inc->mode == kIncEvenOnly) return;  // the keys are current
     if (cnt->err) return;  // unfinished jumping: g-words may point downwards, so no chain walk would end
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -437,46 +422,62 @@ __global__ void __launch_bounds__(kBlock) k_chain_cv(int32_t n, const uint32_t* 
 
 // The switching rules on keys (first minimiser for Odd; the sink first, then
 // the first maximiser for Even; strictly better only), one thread per vertex.
+// inc: the switched vertices are listed for k_inc, Even's pass clears its
+// vertices' queue marks, and Odd's does nothing when only Even's is due.
 template <typename OffT>
 __global__ void __launch_bounds__(kBlock) k_switch_cv(int32_t n, int player, const OffT* __restrict__ off,
                                                       const int32_t* __restrict__ tgt,
                                                       const uint8_t* __restrict__ flags, const i128* __restrict__ key,
-                                                      int32_t sink0, GameState* gst, int32_t* strat, Counters* cnt) {
+                                                      int32_t sink0, GameState* gst, int32_t* strat, Counters* cnt,
+                                                      const IncState* __restrict__ inc, uint8_t* emark, int32_t* list,
+                                                      int32_t list_cap) {
     {
         const GameState st = gst[0];
         if (st.phase != kPhaseActive || (player == 0 && st.sw_odd != 0)) return;
+        if (player == 1 && inc && inc->mode == kIncEvenOnly) return;
     }
+    __shared__ int32_t swbuf[kBlock / 32][kSwBuf];
+    int32_t* mybuf = swbuf[threadIdx.x >> 5];
+    int32_t have = 0;
     int32_t nsw = 0;
-    for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-        const uint8_t f = flags[v];
-        if ((f & kSinkSlot) || (int)(f & kOwnerOdd) != player) continue;
-        const int64_t e0 = off[v], e1 = off[v + 1];
-        const int32_t cur = strat[v];
-        int32_t best = player == 0 ? sink0 : -1;
-        i128 bk = player == 0 ? key[sink0] : 0;
-        const i128 curkey = key[cur];
-        for (int64_t e = e0; e < e1; e += 4) {
-            int32_t t[4];
-            i128 kk[4];
+    const int lane = threadIdx.x & 31;
+    for (int32_t v0 = (blockIdx.x * blockDim.x + threadIdx.x) - lane; v0 < n; v0 += gridDim.x * blockDim.x) {
+        const int32_t v = v0 + lane;
+        const uint8_t f = v < n ? flags[v] : kSinkSlot;
+        bool sw = false;
+        if (!(f & kSinkSlot) && (int)(f & kOwnerOdd) == player) {
+            const int64_t e0 = off[v], e1 = off[v + 1];
+            const int32_t cur = strat[v];
+            int32_t best = player == 0 ? sink0 : -1;
+            i128 bk = player == 0 ? key[sink0] : 0;
+            const i128 curkey = key[cur];
+            for (int64_t e = e0; e < e1; e += 4) {
+                int32_t t[4];
+                i128 kk[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) t[j] = e + j < e1 ? tgt[e + j] : -1;
+                for (int j = 0; j < 4; ++j) t[j] = e + j < e1 ? tgt[e + j] : -1;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) kk[j] = t[j] >= 0 ? key[t[j]] : 0;
+                for (int j = 0; j < 4; ++j) kk[j] = t[j] >= 0 ? key[t[j]] : 0;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                if (t[j] < 0) continue;
-                const bool better = player == 0 ? kk[j] > bk : (best < 0 || kk[j] < bk);
-                if (better) {
-                    best = t[j];
-                    bk = kk[j];
+                for (int j = 0; j < 4; ++j) {
+                    if (t[j] < 0) continue;
+                    const bool better = player == 0 ? kk[j] > bk : (best < 0 || kk[j] < bk);
+                    if (better) {
+                        best = t[j];
+                        bk = kk[j];
+                    }
                 }
             }
+            if (player == 0 ? bk > curkey : bk < curkey) {
+                strat[v] = best;
+                ++nsw;
+                sw = true;
+            }
+            if (player == 0 && inc) emark[v] = 0;
         }
-        if (player == 0 ? bk > curkey : bk < curkey) {
-            strat[v] = best;
-            ++nsw;
-        }
+        if (inc) list_push(sw, v, mybuf, &have, list, &cnt->n_list, list_cap);
     }
+    if (inc) list_flush(mybuf, have, list, &cnt->n_list, list_cap);
     block_add32(nsw, &cnt->n_switch);
     __shared__ int32_t tot;
     if (threadIdx.x == 0) tot = 0;
@@ -639,7 +640,7 @@ pg_status enqueue_valuation_cv(pg_game* g, bool want_dom) {
     PG_CUDA_TRY(ctx, cudaMemsetAsync(c, 0, sizeof(Counters), s));
     prof_begin(g, KID_WALK);
     k_walk_cv<<<grid_ilp(n), kBlock, 0, s>>>(n, g->lev, g->strat, g->flags, g->sink0, g->gd, g->gdB, g->gd32, g->ws,
-                                             g->wsB, g->hugelist, c);
+                                             g->wsB, g->hugelist, c, inc_of(g));
     k_walk_more_cv<<<g->coop_blocks, kBlock, 0, s>>>(g->lev, g->hugelist, g->strat, g->sink0, g->gd, g->gdB, g->gd32,
                                                      g->ws, g->wsB, g->plist, c);
     prof_end(g, KID_WALK, 2);
@@ -654,7 +655,7 @@ pg_status enqueue_valuation_cv(pg_game* g, bool want_dom) {
     }
     prof_begin(g, KID_CHAIN2);
     k_chain_cv<<<grid_ilp(n), kBlock, 0, s>>>(n, g->gd32, g->ws, g->flags, g->pri, g->key128, g->kind, g->cls,
-                                              g->dom, want_dom ? 1 : 0, g->gst, c);
+                                              g->dom, want_dom ? 1 : 0, g->gst, c, inc_of(g));
     prof_end(g, KID_CHAIN2, 1);
     PG_CUDA_TRY(ctx, cudaGetLastError());
     return PG_OK;
@@ -667,7 +668,8 @@ pg_status enqueue_switch_cv(pg_game* g, int player) {
     const int kid = player ? KID_SWITCH_ODD : KID_SWITCH_EVEN;
     prof_begin(g, kid);
     k_switch_cv<int32_t><<<grid_n(g->n), kBlock, 0, s>>>(g->n, player, g->off, g->tgt, g->flags, g->key128, g->sink0,
-                                                        g->gst, g->strat, g->cnt);
+                                                        g->gst, g->strat, g->cnt, inc_of(g), g->emark, g->plist,
+                                                        inc_max_seeds(g));
     prof_end(g, kid, 1);
     PG_CUDA_TRY(ctx, cudaGetLastError());
     return PG_OK;

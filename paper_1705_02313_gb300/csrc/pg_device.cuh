@@ -148,6 +148,55 @@ __device__ inline int cmp_sink(uint32_t tu) {
     return (tu & kTopOdd) ? -1 : 1;
 }
 
+// Count-vector keys (pg_cv.cu): the top key, the level of an id, and the key
+// weight of one vertex.
+using i128 = __int128;
+
+__device__ inline i128 top_key() { return (i128)(~(unsigned __int128)0 >> 1); }
+
+__device__ inline int level_of(const Levels& L, int32_t v) {
+    int l = 0;
+#pragma unroll
+    for (int i = 1; i < kMaxLevels; ++i) l += (i < L.n && v >= L.start[i]) ? 1 : 0;
+    return l;
+}
+
+__device__ inline i128 weight_of(const Levels& L, int32_t v) {
+    const int l = level_of(L, v);
+    const i128 w = (i128)1 << L.shift[l];
+    return ((L.odd_mask >> l) & 1u) ? -w : w;
+}
+
+// The vertices that a switching pass switched, for k_inc: each warp gathers
+// its own in shared memory and appends kSwBuf - 31 or more of them at a time
+// (one counter step per switched vertex, or per warp round, would serialise a
+// pass that switches millions). Entries beyond cap are only counted.
+constexpr int kSwBuf = 128;
+__device__ inline void list_flush(const int32_t* buf, int32_t have, int32_t* list, int32_t* counter, int32_t cap) {
+    if (!have) return;
+    const int lane = threadIdx.x & 31;
+    int32_t base = 0;
+    if (lane == 0) base = atomicAdd(counter, have);
+    base = __shfl_sync(kFull, base, 0);
+    for (int32_t j = lane; j < have; j += 32)
+        if (base + j < cap) list[base + j] = buf[j];
+    __syncwarp();
+}
+
+// All 32 lanes call this; have (the entries held) stays uniform over the warp.
+__device__ inline void list_push(bool sw, int32_t v, int32_t* buf, int32_t* have, int32_t* list, int32_t* counter,
+                                 int32_t cap) {
+    const unsigned m = __ballot_sync(kFull, sw);
+    if (!m) return;
+    if (sw) buf[*have + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = v;
+    *have += __popc(m);
+    __syncwarp();
+    if (*have > kSwBuf - 32) {
+        list_flush(buf, *have, list, counter, cap);
+        *have = 0;
+    }
+}
+
 // The sink slot of v's game.
 __device__ inline int32_t sink_of(int32_t v, const int32_t* vgame, const int32_t* gsink, int32_t sink0) {
     return vgame ? gsink[vgame[v]] : sink0;

@@ -48,6 +48,7 @@ constexpr int kIncEven = 16384;      // Even's queue of a block (beyond it Even'
 constexpr int kIncFanIn = 1024;      // a vertex of A with more predecessors ends the incremental iteration
 constexpr int kIncLevels = 256;      // levels of the closure
 constexpr int kIncRounds = 128;      // rounds of the resolution
+constexpr int kIncWalk = 2048;       // count-vector mode: steps of a play inside A
 constexpr int kIncSteps = 128;       // steps of one resolution round
 constexpr size_t kIncShared = sizeof(int32_t) * (3 * kIncSet + kIncQueue + kIncEven);
 constexpr int32_t kIncBig = 1 << 24;  // (16 blocks' counts sum below 2^31)
@@ -57,6 +58,10 @@ constexpr int32_t kIncBig = 1 << 24;  // (16 blocks' counts sum below 2^31)
 // and 1,025 us from 27.9k; against 62 us on the 1M game, 48 us from 1.3k and
 // 125 us from 4.7k.
 constexpr int kIncSeedShare = 1024, kIncSeeds = 8192;
+// Count-vector games, against 310 us for a full iteration of the 3M-vertex game
+// with 4 priorities: 72 us from 5.8k switched vertices, 126 us from 12.6k
+// (350 us and more from 8-15k when their trees are deep).
+constexpr int kIncSeedShareCv = 256, kIncSeedsCv = 16384;
 // In a launch that runs the whole loop (41k ids): an iteration over all ids
 // takes 17-32 us, an incremental one 13 us (a few switched vertices) to 35 us
 // (a hundred, for the levels of the closure).
@@ -82,6 +87,8 @@ struct IncArgs {
     IncState* st;
     int32_t* gactive;
     int64_t* loop_iters;
+    i128* key;   // count-vector mode: the keys, and the levels they count
+    Levels lev;
     int64_t cap;
     int32_t max_seeds;  // more switched vertices than this take a full iteration
     int32_t whole;      // 1: the launch runs the whole loop, full iterations included (over all ids)
@@ -102,16 +109,17 @@ __device__ inline bool claim_byte(uint8_t* base, int32_t i, uint32_t b) {
 // successors.
 template <int PLAYER>
 __device__ inline bool inc_switch(const IncArgs& a, int32_t v, bool* tie_out) {
-    const int32_t e0 = a.off[v], e1 = a.off[v + 1];
+    const int32_t* tgt = a.tgt + a.off[v];
+    const int32_t deg = a.off[v + 1] - a.off[v];
     const int32_t cur = __ldcg(a.strat + v);
     int32_t best = PLAYER == 0 ? a.sink0 : -1;
     uint32_t tbest = 0;
     bool cur_top = false, tie = false;
-    for (int32_t e = e0; e < e1; e += 4) {
+    for (int32_t e = 0; e < deg; e += 4) {
         int32_t t[4];
         uint32_t tt[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) t[j] = e + j < e1 ? a.tgt[e + j] : -1;
+        for (int j = 0; j < 4; ++j) t[j] = e + j < deg ? tgt[e + j] : -1;
 #pragma unroll
         for (int j = 0; j < 4; ++j) tt[j] = t[j] >= 0 ? __ldcg(a.topw + t[j]) : 0u;
 #pragma unroll
@@ -135,6 +143,109 @@ __device__ inline bool inc_switch(const IncArgs& a, int32_t v, bool* tie_out) {
     return sw;
 }
 
+__device__ inline i128 ld_key(const i128* p) {
+    const longlong2 w = __ldcg(reinterpret_cast<const longlong2*>(p));
+    return (i128)w.y << 64 | (unsigned long long)w.x;
+}
+__device__ inline void st_key(i128* p, i128 k) {
+    __stcg(reinterpret_cast<longlong2*>(p), make_longlong2((long long)k, (long long)(k >> 64)));
+}
+
+// Decision of one vertex on keys (the rules of k_switch_cv).
+template <int PLAYER>
+__device__ inline bool inc_switch_cv(const IncArgs& a, int32_t v) {
+    const int32_t* tgt = a.tgt + a.off[v];
+    const int32_t deg = a.off[v + 1] - a.off[v];
+    const int32_t cur = __ldcg(a.strat + v);
+    const i128 curkey = ld_key(a.key + cur);
+    int32_t best = PLAYER == 0 ? a.sink0 : -1;
+    i128 bk = 0;  // (the sink's key: the empty count vector)
+    for (int32_t e = 0; e < deg; e += 4) {
+        int32_t t[4];
+        i128 k[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) t[j] = e + j < deg ? tgt[e + j] : -1;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) k[j] = t[j] >= 0 ? ld_key(a.key + t[j]) : (i128)0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (t[j] < 0 || !(PLAYER == 0 ? k[j] > bk : (best < 0 || k[j] < bk))) continue;
+            best = t[j];
+            bk = k[j];
+        }
+    }
+    const bool sw = PLAYER == 0 ? bk > curkey : bk < curkey;
+    if (sw) __stcg(a.strat + v, best);
+    return sw;
+}
+
+// Key of a vertex of A (its word is pending): the weights along its play as far
+// as the play stays in A, plus the key of the first vertex outside. A play that
+// stays in A forever ends in a cycle (Brent's method finds it): TOP, and *odd
+// when the cycle's largest vertex is. *cut: the play is longer than kIncWalk.
+__device__ inline i128 inc_key(const IncArgs& a, int32_t v, bool* odd, bool* cut) {
+    i128 acc = weight_of(a.lev, v);
+    int32_t x = g32_ptr(__ldcg(a.gd32 + v)), mark = v;
+    for (int32_t steps = 1, power = 1, lam = 0;; ++steps) {
+        const uint32_t w = __ldcg(a.gd32 + x);
+        if (!g32_pending(w)) {
+            const i128 k = ld_key(a.key + x);
+            return k == top_key() ? k : acc + k;
+        }
+        if (x == mark) break;
+        if (steps >= kIncWalk) {
+            *cut = true;
+            return 0;
+        }
+        if (++lam == power) {
+            mark = x;
+            power *= 2;
+            lam = 0;
+        }
+        acc += weight_of(a.lev, x);
+        x = g32_ptr(w);
+    }
+    int32_t big = x;
+    for (int32_t y = g32_ptr(__ldcg(a.gd32 + x)); y != x; y = g32_ptr(__ldcg(a.gd32 + y))) big = max(big, y);
+    if (a.flags[big] & kPriOdd) *odd = true;
+    return top_key();
+}
+
+// Queues the predecessors of la[i] that want it (all of them if changed, else
+// those with a tie mark) for their player.
+__device__ inline void inc_queue(const IncArgs& a, int32_t e0, int32_t nodd, int32_t deg, bool changed, int32_t* lq,
+                                 int32_t* c_q, int32_t* le, int32_t* c_e) {
+    const int32_t* src = a.rv_src + e0;
+    for (int32_t e = 0; e < deg; e += 4) {
+        int32_t y[4];
+        bool want[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) y[j] = e + j < deg ? src[e + j] : -1;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            want[j] = y[j] >= 0 && (changed || (__ldcg((e + j < nodd ? a.omark : a.emark) + y[j]) & kMarkTie));
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            want[j] = want[j] && claim_byte(e + j < nodd ? a.omark : a.emark, y[j], kMarkQueued);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (!want[j]) continue;
+            if (e + j < nodd) {
+                const int32_t p = atomicAdd(c_q, 1);
+                if (p < kIncQueue) lq[p] = y[j];
+                else __stcg(a.qlist + atomicAdd(&a.st->n_q, 1), y[j]);
+            } else {
+                const int32_t p = atomicAdd(c_e, 1);
+                if (p < kIncEven) le[p] = y[j];
+            }
+        }
+    }
+}
+
+// CV: count-vector mode (repeated priorities). A valuation is a key summed along
+// the play, so the g-words only tell who is in A, and decisions compare keys
+// (no tie marks); full iterations are not run here. 3M vertices, 4 priorities, load and solve: 30.5 -> 15.0 ms.
+template <bool CV>
 __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
     cg::cluster_group cl = cg::this_cluster();
     const int32_t CL = (int32_t)cl.num_blocks(), rank = (int32_t)cl.block_rank(), tid = threadIdx.x;
@@ -146,7 +257,7 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
     int32_t* lq = lc + kIncSet;    // its part of Odd's queue
     int32_t* le = lq + kIncQueue;  //    and of Even's
     __shared__ int2 xb[2][kIncCluster];
-    __shared__ int32_t lvl[3], c_bad, c_left, c_q, c_spill, c_odd, c_s, c_e, c_zero;
+    __shared__ int32_t lvl[3], c_bad, c_left, c_q, c_odd, c_s, c_e, c_zero;
     int par = 0;
     // The sums over the cluster of two counts, final in each block when all its threads call: every block stores
     // its pair in every block's shared memory and sums after the barrier. Two buffers in turn: a block that is
@@ -187,7 +298,7 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
         bool all = fresh || ns > a.max_seeds;
         if (all && !a.whole) break;
         if (tid == 0) {
-            c_bad = c_left = c_q = c_spill = c_odd = 0;
+            c_bad = c_left = c_q = c_odd = 0;
             lvl[1] = 0;
         }
         if (t0 == 0) a.st->n_q = 0;
@@ -212,13 +323,14 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
                 int32_t* next = &lvl[(r + 1) % 3];
                 if (tid == 0) lvl[(r + 2) % 3] = 0;
                 for (int32_t i = lo + tid; i < na; i += kIncThreads) {
-                    const int32_t x = la[i], e0 = ls[i], e1 = e0 + (lc[i] >> 16);
-                    for (int32_t e = e0; e < e1; e += 4) {
+                    const int32_t x = la[i], deg = lc[i] >> 16;
+                    const int32_t* src = a.rv_src + ls[i];
+                    for (int32_t e = 0; e < deg; e += 4) {
                         int32_t y[4], s[4], r1[4];
                         uint32_t w[4];
                         int2 r0[4];
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) y[j] = e + j < e1 ? a.rv_src[e + j] : x;  // (x: not below itself)
+                        for (int j = 0; j < 4; ++j) y[j] = e + j < deg ? src[e + j] : x;  // (x: not below itself)
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             s[j] = __ldcg(a.strat + y[j]);
@@ -265,47 +377,73 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
         }
         // ids [i0, i1) in steps of st are this thread's, or la[i] of them
         const int32_t i0 = all ? t0 : tid, i1 = all ? a.n : na, step = all ? T : kIncThreads;
-        // resolve: words of A turn from jump pointers into g-words; any word read is valid whenever it is read
         bool unresolved = false;
-        for (int32_t r = 0;; ++r) {
-            int32_t left = 0;
-            for (int32_t i = i0; i < i1; i += step) {
-                const int32_t v = all ? i : la[i];
-                const uint32_t w = __ldcg(a.gd32 + v);
-                if (!g32_pending(w)) continue;
-                int32_t x = g32_ptr(w);
-                bool top = false;
-                for (int k = 0; k < kIncSteps && x < v; ++k) {
-                    const uint32_t wx = __ldcg(a.gd32 + x);
-                    if (g32_none(wx) && !g32_pending(wx)) {  // TOP: v's play ends in the same cycle
-                        top = true;
-                        break;
+        if constexpr (CV) {
+            for (int32_t i = tid; i < na; i += kIncThreads) {
+                const int32_t v = la[i];
+                const i128 old = ld_key(a.key + v);
+                bool odd = false, cut = false;
+                const i128 k = inc_key(a, v, &odd, &cut);
+                if (odd) c_odd = 1;
+                if (cut) {
+                    c_left = 1;
+                    continue;
+                }
+                const int32_t nodd = lc[i] & 0xffff;
+                if (k == old) continue;
+                // (a key outside A is never this one: it may change while other plays are walked)
+                st_key(a.key + v, k);
+                inc_queue(a, ls[i], nodd, even_full ? nodd : lc[i] >> 16, true, lq, &c_q, le, &c_e);
+            }
+            unresolved = exchange(&c_left, &c_zero).x != 0;
+            for (int32_t i = tid; i < na; i += kIncThreads) __stcg(a.gd32 + la[i], kG32None);  // no longer in A
+            if (unresolved) {  // Odd's queue is dropped (Even's: its next pass is full)
+                const int32_t nq = min(c_q, kIncQueue), spill = __ldcg(&a.st->n_q);
+                for (int32_t i = tid; i < nq; i += kIncThreads) a.omark[lq[i]] = 0;
+                for (int32_t i = t0; i < spill; i += T) a.omark[__ldcg(a.qlist + i)] = 0;
+            }
+        } else {
+            // resolve: words of A turn from jump pointers into g-words; any word read is valid whenever it is read
+            for (int32_t r = 0;; ++r) {
+                int32_t left = 0;
+                for (int32_t i = i0; i < i1; i += step) {
+                    const int32_t v = all ? i : la[i];
+                    const uint32_t w = __ldcg(a.gd32 + v);
+                    if (!g32_pending(w)) continue;
+                    int32_t x = g32_ptr(w);
+                    bool top = false;
+                    for (int k = 0; k < kIncSteps && x < v; ++k) {
+                        const uint32_t wx = __ldcg(a.gd32 + x);
+                        if (g32_none(wx) && !g32_pending(wx)) {  // TOP: v's play ends in the same cycle
+                            top = true;
+                            break;
+                        }
+                        x = g32_sink(wx) && !g32_pending(wx) ? a.sink0 : g32_ptr(wx);
                     }
-                    x = g32_sink(wx) && !g32_pending(wx) ? a.sink0 : g32_ptr(wx);
+                    uint32_t nw;
+                    if (top) nw = kG32None | (uint32_t)a.sink0;  // (a pointer that no cycle maximum has)
+                    else if (x > v) nw = x == a.sink0 ? g32_sink_word(a.flags[v]) : (uint32_t)x;
+                    else if (x == v) nw = kG32None | (uint32_t)v;
+                    else {
+                        nw = kG32Pend | (uint32_t)x;
+                        left = 1;
+                    }
+                    __stcg(a.gd32 + v, nw);
                 }
-                uint32_t nw;
-                if (top) nw = kG32None | (uint32_t)a.sink0;  // (a pointer that no cycle maximum has)
-                else if (x > v) nw = x == a.sink0 ? g32_sink_word(a.flags[v]) : (uint32_t)x;
-                else if (x == v) nw = kG32None | (uint32_t)v;
-                else {
-                    nw = kG32Pend | (uint32_t)x;
-                    left = 1;
+                if (left) c_left = 1;
+                const int32_t rem = exchange(&c_left, &c_zero).x;
+                if (rem == 0) break;
+                if (r + 1 >= kIncRounds) {
+                    unresolved = true;
+                    break;
                 }
-                __stcg(a.gd32 + v, nw);
+                if (tid == 0) c_left = 0;
+                __syncthreads();
             }
-            if (left) c_left = 1;
-            const int32_t rem = exchange(&c_left, &c_zero).x;
-            if (rem == 0) break;
-            if (r + 1 >= kIncRounds) {
-                unresolved = true;
-                break;
-            }
-            if (tid == 0) c_left = 0;
-            __syncthreads();
         }
         if (unresolved) {
             if (!a.whole) break;  // the full iteration decides
-            if (!all) {           // over all ids once
+            if (!all) {  // over all ids once
                 ns = a.n;
                 __syncthreads();
                 continue;
@@ -317,69 +455,44 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
             ++iters;
             break;
         }
-        // classify (as k_classify)
-        for (int32_t i = i0; i < i1; i += step) {
-            const int32_t v = all ? i : la[i];
-            const uint32_t w0 = __ldcg(a.gd32 + v), old = all ? 0u : __ldcg(a.topw + v);
-            int32_t x = g32_sink(w0) ? v : g32_ptr(w0);
-            bool top = g32_none(w0), odd = g32_sink(w0) && (w0 & 1u);
-            if (top && x == v && (a.flags[v] & kPriOdd)) c_odd = 1;
-            if (!top && !g32_sink(w0)) {
-                for (int32_t len = 1;; ++len) {
-                    if (len > a.deep_cut) {  // a deep forest: the iteration is abandoned
-                        c_bad = 1;
-                        break;
-                    }
-                    const uint32_t wx = __ldcg(a.gd32 + x);
-                    if (wx & kG32Top) {
-                        top = true;
-                        break;
-                    }
-                    if (g32_sink(wx)) {
-                        odd = wx & 1u;
-                        break;
-                    }
-                    const int32_t nx = g32_ptr(wx);
-                    if (nx <= x) break;  // g-chains rise (a guard, never taken)
-                    x = nx;
-                }
-                if (top) __stcg(a.gd32 + v, w0 | kG32Top);
-            }
-            const uint32_t tw = top ? kG32Top : (odd ? kTopOdd : 0u) | (uint32_t)x;
-            if (all) {  // everyone is evaluated: no queues
-                __stcg(a.topw + v, tw);
-                continue;
-            }
-            const bool changed = tw != old;
-            if (changed) __stcg(a.topw + v, tw);
-            const int32_t e0 = ls[i], em = e0 + (lc[i] & 0xffff), e1 = even_full ? em : e0 + (lc[i] >> 16);
-            for (int32_t e = e0; e < e1; e += 4) {
-                int32_t y[4];
-                bool want[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) y[j] = e + j < e1 ? a.rv_src[e + j] : -1;
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    want[j] = y[j] >= 0 && (changed || (__ldcg((e + j < em ? a.omark : a.emark) + y[j]) & kMarkTie));
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    want[j] = want[j] && claim_byte(e + j < em ? a.omark : a.emark, y[j], kMarkQueued);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (!want[j]) continue;
-                    if (e + j < em) {
-                        const int32_t p = atomicAdd(&c_q, 1);
-                        if (p < kIncQueue) {
-                            lq[p] = y[j];
-                        } else {
-                            atomicAdd(&c_spill, 1);
-                            __stcg(a.qlist + atomicAdd(&a.st->n_q, 1), y[j]);
+        if constexpr (!CV) {
+            // classify (as k_classify)
+            for (int32_t i = i0; i < i1; i += step) {
+                const int32_t v = all ? i : la[i];
+                const uint32_t w0 = __ldcg(a.gd32 + v), old = all ? 0u : __ldcg(a.topw + v);
+                int32_t x = g32_sink(w0) ? v : g32_ptr(w0);
+                bool top = g32_none(w0), odd = g32_sink(w0) && (w0 & 1u);
+                if (top && x == v && (a.flags[v] & kPriOdd)) c_odd = 1;
+                if (!top && !g32_sink(w0)) {
+                    for (int32_t len = 1;; ++len) {
+                        if (len > a.deep_cut) {  // a deep forest: the iteration is abandoned
+                            c_bad = 1;
+                            break;
                         }
-                    } else {
-                        const int32_t p = atomicAdd(&c_e, 1);
-                        if (p < kIncEven) le[p] = y[j];
+                        const uint32_t wx = __ldcg(a.gd32 + x);
+                        if (wx & kG32Top) {
+                            top = true;
+                            break;
+                        }
+                        if (g32_sink(wx)) {
+                            odd = wx & 1u;
+                            break;
+                        }
+                        const int32_t nx = g32_ptr(wx);
+                        if (nx <= x) break;  // g-chains rise (a guard, never taken)
+                        x = nx;
                     }
+                    if (top) __stcg(a.gd32 + v, w0 | kG32Top);
                 }
+                const uint32_t tw = top ? kG32Top : (odd ? kTopOdd : 0u) | (uint32_t)x;
+                if (all) {  // everyone is evaluated: no queues
+                    __stcg(a.topw + v, tw);
+                    continue;
+                }
+                const bool changed = tw != old;
+                if (changed) __stcg(a.topw + v, tw);
+                const int32_t nodd = lc[i] & 0xffff;
+                inc_queue(a, ls[i], nodd, even_full ? nodd : lc[i] >> 16, changed, lq, &c_q, le, &c_e);
             }
         }
         if (tid == 0) c_s = 0;
@@ -391,8 +504,8 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
         }
         // Odd's pass; the switched vertices are the next iteration's seeds
         auto odd_vertex = [&](int32_t v) {
-            bool tie;
-            const bool sw = inc_switch<1>(a, v, &tie);
+            bool tie = false;
+            const bool sw = CV ? inc_switch_cv<1>(a, v) : inc_switch<1>(a, v, &tie);
             a.omark[v] = tie ? kMarkTie : 0;
             if (!sw) return;
             const int32_t p = atomicAdd(&c_s, 1);
@@ -422,8 +535,8 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
                 break;
             }
             auto even_vertex = [&](int32_t v) {
-                bool tie;
-                const bool sw = inc_switch<0>(a, v, &tie);
+                bool tie = false;
+                const bool sw = CV ? inc_switch_cv<0>(a, v) : inc_switch<0>(a, v, &tie);
                 a.emark[v] = tie ? kMarkTie : 0;
                 if (!sw) return;
                 const int32_t p = atomicAdd(&c_s, 1);
@@ -525,8 +638,8 @@ __global__ void __launch_bounds__(kBlock) k_rv_fill(int32_t n, const OffT* __res
     for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
         const bool odd = (flags[v] & kOwnerOdd) != 0;
         if (odd_only && !odd) continue;
-        const OffT e1 = off[v + 1];
-        for (OffT e = off[v]; e < e1; e += 4) {  // four cursor steps in flight
+        const int64_t e1 = off[v + 1];
+        for (int64_t e = off[v]; e < e1; e += 4) {  // four cursor steps in flight
             int32_t t[4], p[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) t[j] = e + j < e1 ? tgt[e + j] : -1;
@@ -542,12 +655,16 @@ __global__ void __launch_bounds__(kBlock) k_rv_fill(int32_t n, const OffT* __res
 
 }  // namespace
 
-bool inc_applies(const pg_game* g) { return !g->vgame && g->ngames == 1 && g->off != nullptr && !g->cv; }
+bool inc_applies(const pg_game* g) { return !g->vgame && g->ngames == 1 && g->off != nullptr; }
 
 pg_status build_reverse(pg_game* g, int64_t odd_edges) {
-    if (g->rv) return PG_OK;
+    if (g->rv_ok) return PG_OK;
     pg_ctx* ctx = g->ctx;
     cudaStream_t s = ctx->stream;
+    for (void** q : {(void**)&g->rv, (void**)&g->rv_src, (void**)&g->omark, (void**)&g->emark}) {
+        if (*q) cudaFreeAsync(*q, s);
+        *q = nullptr;
+    }
     const int32_t n = g->n;
     // packed games take no incremental iterations: their lists hold Odd's edges only (the marks of k_classify)
     const int odd_only = inc_applies(g) ? 0 : 1;
@@ -587,14 +704,18 @@ pg_status build_reverse(pg_game* g, int64_t odd_edges) {
     });
     PG_CUDA_TRY(ctx, cudaGetLastError());
     ctx->launches += 4;
+    g->rv_ok = true;
     return PG_OK;
 }
 
-int32_t inc_max_seeds(const pg_game* g) { return std::max(1, std::min(g->n / kIncSeedShare, kIncSeeds)); }
+int32_t inc_max_seeds(const pg_game* g) {
+    return g->cv ? std::max(1, std::min(g->n / kIncSeedShareCv, kIncSeedsCv))
+                 : std::max(1, std::min(g->n / kIncSeedShare, kIncSeeds));
+}
 
-static int inc_cluster_for(int want) {
-    cudaFuncSetAttribute(k_inc, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_inc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kIncShared);
+static int inc_cluster_for(void (*kern)(IncArgs), int want) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kIncShared);
     for (int c = want; c > 1; c >>= 1) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(c);
@@ -607,7 +728,7 @@ static int inc_cluster_for(int want) {
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int k = 0;
-        if (cudaOccupancyMaxActiveClusters(&k, k_inc, &cfg) == cudaSuccess && k > 0) return c;
+        if (cudaOccupancyMaxActiveClusters(&k, kern, &cfg) == cudaSuccess && k > 0) return c;
         cudaGetLastError();
     }
     return 1;
@@ -636,6 +757,8 @@ pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole) {
     a.st = g->inc;
     a.gactive = g->gactive;
     a.loop_iters = g->loop_iters;
+    a.key = g->key128;
+    a.lev = g->lev;
     a.cap = cap;
     a.whole = whole ? 1 : 0;
     a.even = even ? 1 : 0;
@@ -645,7 +768,8 @@ pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole) {
     int want = kIncCluster;
     if (whole)
         while (want > 1 && (int64_t)want * kIncThreads / 2 >= g->n) want >>= 1;
-    if (!g->inc_cluster) g->inc_cluster = inc_cluster_for(kIncCluster);
+    auto kern = g->cv ? k_inc<true> : k_inc<false>;
+    if (!g->inc_cluster) g->inc_cluster = inc_cluster_for(kern, kIncCluster);
     const int c = std::min(want, g->inc_cluster);
     a.max_seeds = std::min(whole ? std::max(1, g->n / kIncWholeShare) : inc_max_seeds(g), c * (kIncSet / 2));
     cudaLaunchConfig_t cfg = {};
@@ -659,7 +783,7 @@ pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole) {
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    PG_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, k_inc, a));
+    PG_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, kern, a));
     ctx->launches += 1;
     return PG_OK;
 }

@@ -299,6 +299,7 @@ struct pg_game {
     int32_t* rv_src = nullptr;
     uint8_t* omark = nullptr;
     uint8_t* emark = nullptr;
+    bool rv_ok = false;           // the four above are complete
     pg::IncState* inc = nullptr;  // incremental iterations (pg_inc.cu; single games)
     int inc_cluster = 0;          // blocks of their cluster (0: not yet asked)
     // ruling-set ranks (pg_deep.cu), for games whose g-forest is deep
@@ -426,6 +427,7 @@ pg_status build_player_split(pg_game* g);
 // use (odd_edges: the edges of Odd's vertices, for packed games), one launch of k_inc. whole: the launch is
 // the entire loop; otherwise it follows a full iteration whose passes listed at most inc_max_seeds switches.
 bool inc_applies(const pg_game* g);
+IncState* inc_of(const pg_game* g);  // the state, when the loop's full iterations prepare incremental ones, or null
 pg_status build_reverse(pg_game* g, int64_t odd_edges);
 int32_t inc_max_seeds(const pg_game* g);
 pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole);

@@ -1487,36 +1487,6 @@ __device__ inline bool switch_at(int32_t v, int64_t e0, int64_t e1, const int32_
     return sw;
 }
 
-// The vertices that a switching pass switched, for k_inc: each warp gathers
-// its own in shared memory and appends kSwBuf - 31 or more of them at a time
-// (one counter step per switched vertex, or per warp round, would serialise a
-// pass that switches millions). Entries beyond cap are only counted.
-constexpr int kSwBuf = 128;
-__device__ inline void list_flush(const int32_t* buf, int32_t have, int32_t* list, int32_t* counter, int32_t cap) {
-    if (!have) return;
-    const int lane = threadIdx.x & 31;
-    int32_t base = 0;
-    if (lane == 0) base = atomicAdd(counter, have);
-    base = __shfl_sync(kFull, base, 0);
-    for (int32_t j = lane; j < have; j += 32)
-        if (base + j < cap) list[base + j] = buf[j];
-    __syncwarp();
-}
-
-// All 32 lanes call this; have (the entries held) stays uniform over the warp.
-__device__ inline void list_push(bool sw, int32_t v, int32_t* buf, int32_t* have, int32_t* list, int32_t* counter,
-                                 int32_t cap) {
-    const unsigned m = __ballot_sync(kFull, sw);
-    if (!m) return;
-    if (sw) buf[*have + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = v;
-    *have += __popc(m);
-    __syncwarp();
-    if (*have > kSwBuf - 32) {
-        list_flush(buf, *have, list, counter, cap);
-        *have = 0;
-    }
-}
-
 // A switch counted into its game (packed games: one atomic per group of
 // lanes of the same game; one game: the block total at the end).
 template <int PLAYER, bool BATCH>
@@ -1886,10 +1856,9 @@ uint8_t* omark_of(const pg_game* g) {
     return g->pl_ok && g->omark && !g->cv && !g->tune.loop_ranks && !g->deep_mode ? g->omark : nullptr;
 }
 
-namespace {
-// The incremental iterations' state when the loop's full iterations prepare them (null otherwise).
-IncState* inc_of(const pg_game* g) { return omark_of(g) && g->emark && inc_applies(g) ? g->inc : nullptr; }
-}  // namespace
+IncState* inc_of(const pg_game* g) {
+    return g->rv_ok && g->inc && inc_applies(g) && (g->cv || omark_of(g)) ? g->inc : nullptr;
+}
 
 pg_status enqueue_bookkeeping(pg_game* g, int64_t cap, bool even_phase) {
     pg_ctx* ctx = g->ctx;
@@ -2044,11 +2013,7 @@ pg_status build_player_split(pg_game* g) {
         if (g->pl_tgt[p]) cudaFreeAsync(g->pl_tgt[p], s);
         g->pl_vid[p] = g->pl_off[p] = g->pl_tgt[p] = nullptr;
     }
-    if (g->vgame)  // a server's layout changed (a loaded game's reverse adjacency stays)
-        for (void** q : {(void**)&g->rv, (void**)&g->rv_src, (void**)&g->omark, (void**)&g->emark}) {
-            if (*q) cudaFreeAsync(*q, s);
-            *q = nullptr;
-        }
+    if (g->vgame) g->rv_ok = false;  // a server's layout changed (a loaded game's reverse adjacency stays)
     int32_t mp_of[2] = {0, 0};
     // the valuation's scratch is free before a loop: marks in kind and cls, positions in coff, degrees in
     // hugelist

@@ -5,7 +5,7 @@ repeated edges and self-loops."""
 import numpy as np
 import pytest
 
-from oracle import o2
+from oracle import o2, o3
 from paper_1705_02313_gb300 import gen
 from paper_1705_02313_gb300.gen import Game
 
@@ -69,3 +69,22 @@ def test_many_predecessors(pg, ctx, n, hubs, share):
 @pytest.mark.parametrize("n", [700, 30000, 100003])
 def test_reset(pg, ctx, n):
     check(pg, ctx, gen.native_random_game(n, 2, 5, seed=n), reset=True)
+
+
+@pytest.mark.parametrize("levels", [2, 4])
+@pytest.mark.parametrize("n,hubs,share", [(900, 1, 0.0), (20000, 3, 0.3), (150001, 50, 0.0), (150001, 4000, 0.4)])
+def test_few_priorities(pg, ctx, n, hubs, share, levels):
+    g = hub_game(n, hubs, share, n + hubs)
+    g.pri[:] = g.pri % levels
+    _, _, want = o3.solve_game(g.n, g.offsets, g.targets, g.owner, g.pri)
+    game = pg.pg_load_csr(ctx, g.n, g.m, *g.arrays())
+    try:
+        d = pg.pg_game_levels(game).size
+        out = dict(win=np.empty(n, np.uint8), val_class=np.empty(n, np.int8), val_counts=np.empty(n * d, np.int32),
+                   **{k: np.empty(n, np.int32) for k in ("sigma", "tau", "val_depth")})
+        for _ in range(2):
+            assert pg.pg_solve(ctx, game, **out) == (want["major"], want["inner"])
+            for k in out:
+                assert np.array_equal(out[k].reshape(np.asarray(want[k]).shape), np.asarray(want[k])), k
+    finally:
+        pg.pg_game_free(game)
