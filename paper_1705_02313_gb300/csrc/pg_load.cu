@@ -323,6 +323,187 @@ __global__ void k_maps(int32_t n0, int32_t k, const int32_t* nid, int32_t* nid0,
     }
 }
 
+// ---------------------------------------------------------------------------
+// Many games in one load (load_union): the input vertices of all games are
+// numbered through (game g's from vb[g]), their edges too (from eb[g]), and the
+// trap computation runs once on the union, whose components it leaves apart.
+// Vertex x's id in the packed layout is its rank among all G' priorities
+// ordered by (game, priority), plus one sink slot per earlier game.
+struct UnionGame {
+    int32_t vb, eb;  // first vertex and edge
+    int32_t db;      // first dummy
+    int32_t words;   // first word of the game's priority bitmap
+};
+
+// The game of every vertex, edges as vertices of the union, validation as in
+// k_validate with the error bits and the largest priority per game.
+__global__ void k_union_prepare(int32_t n, int32_t ng, const UnionGame* __restrict__ G,
+                                const int32_t* __restrict__ off, const int32_t* __restrict__ tgt,
+                                const uint8_t* __restrict__ own, const int32_t* __restrict__ pri,
+                                int32_t* __restrict__ vg, int32_t* __restrict__ uoff, int32_t* __restrict__ utgt,
+                                int32_t* gerr, int32_t* gmax) {
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) - lane; b < n; b += stride) {
+        const int64_t v = b + lane;
+        int32_t g = -1, err = 0, p = -1;
+        if (v < n) {
+            int32_t lo = 0, hi = ng;  // the last game that starts at or before v
+            while (hi - lo > 1) {
+                const int32_t mid = (lo + hi) >> 1;
+                if (G[mid].vb <= v) lo = mid;
+                else hi = mid;
+            }
+            g = lo;
+            vg[v] = g;
+            const int32_t v0 = G[g].vb, e0 = G[g].eb, nv = G[g + 1].vb - v0, ne = G[g + 1].eb - e0;
+            const int32_t a = off[v + g], c = off[v + g + 1];  // (one more offset than vertices per game)
+            const bool ok = a >= 0 && a < c && c <= ne;
+            if (!ok || (v == v0 && a != 0) || (v == v0 + nv - 1 && c != ne)) err |= kEOff;
+            if (own[v] > 1) err |= kEOwn;
+            p = pri[v];
+            if (p < 0) err |= kEPri;
+            uoff[v] = e0 + a;
+            if (v == n - 1) uoff[n] = G[ng].eb;
+            for (int32_t e = a; ok && e < c; ++e) {
+                const int32_t t = tgt[(int64_t)e0 + e];
+                if (t < 0 || t >= nv) err |= kETgt;
+                utgt[(int64_t)e0 + e] = v0 + t;
+            }
+        }
+        // one atomic of each kind per warp and game
+        const unsigned peers = __match_any_sync(0xffffffffu, g);
+        const int32_t err_all = __reduce_or_sync(peers, err), p_all = __reduce_max_sync(peers, p);
+        if (g >= 0 && lane == __ffs(peers) - 1) {
+            if (err_all) atomicOr(gerr + g, err_all);
+            if (p_all > *(volatile int32_t*)(gmax + g)) atomicMax(gmax + g, p_all);
+        }
+    }
+}
+
+__global__ void k_union_dummies(int32_t n, int32_t ng, UnionGame* __restrict__ G, const uint8_t* __restrict__ isW,
+                                const int32_t* __restrict__ widx, const int32_t* __restrict__ vg,
+                                int32_t* __restrict__ dsrc) {
+    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v <= n; v += (int64_t)gridDim.x * blockDim.x) {
+        if (v == n) G[ng].db = widx[n];
+        else {
+            if (v == G[vg[v]].vb) G[vg[v]].db = widx[v];
+            if (isW[v]) dsrc[widx[v]] = (int32_t)v;
+        }
+    }
+}
+
+// Game and bitmap position of G' vertex x (originals, then the dummies, as
+// dummy d guards vertex dsrc[d]): an original's priority is raised by twice its
+// game's dummies, the game's j-th dummy has 2j.
+__device__ inline int32_t union_prio(int64_t x, int32_t n, const UnionGame* __restrict__ G,
+                                     const int32_t* __restrict__ vg, const int32_t* __restrict__ pri,
+                                     const int32_t* __restrict__ dsrc, int32_t* g) {
+    if (x < n) {
+        *g = vg[x];
+        return pri[x] + 2 * (G[*g + 1].db - G[*g].db);
+    }
+    *g = vg[dsrc[x - n]];
+    return 2 * ((int32_t)(x - n) - G[*g].db);
+}
+
+// Marks the priorities (as k_mark_priorities, a bitmap per game).
+__global__ void k_union_mark(int64_t np, int32_t n, const UnionGame* __restrict__ G, const int32_t* __restrict__ vg,
+                             const int32_t* __restrict__ pri, const int32_t* __restrict__ dsrc, uint32_t* bits,
+                             int32_t* dup) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < np; x += stride) {
+        int32_t g;
+        const int32_t p = union_prio(x, n, G, vg, pri, dsrc, &g);
+        const uint32_t bit = 1u << (p & 31);
+        if (atomicOr(bits + (int64_t)G[g].words + (p >> 5), bit) & bit) *dup = 1;
+    }
+}
+
+__global__ void k_union_rank(int64_t np, int32_t n, const UnionGame* __restrict__ G, const int32_t* __restrict__ vg,
+                             const int32_t* __restrict__ pri, const int32_t* __restrict__ dsrc,
+                             const uint32_t* __restrict__ bits, const int32_t* __restrict__ wprefix,
+                             int32_t* __restrict__ nid0, int32_t* __restrict__ dnid, int32_t* __restrict__ gid) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < np; x += stride) {
+        int32_t g;
+        const int32_t p = union_prio(x, n, G, vg, pri, dsrc, &g);
+        const int64_t w = (int64_t)G[g].words + (p >> 5);
+        const int32_t id = wprefix[w] + __popc(bits[w] & ((1u << (p & 31)) - 1u)) + g;
+        if (x < n) nid0[x] = id;
+        else dnid[x - n] = id;
+        gid[id] = (int32_t)x;
+    }
+}
+
+// Per vertex of the union, what the rows in relabelled order read of it (as
+// k_pack_vertices, with its game in w above the two bits), and its id as the
+// target of an edge from U.
+__global__ void k_union_pack(int32_t n, const UnionGame* __restrict__ G, const int32_t* __restrict__ vg,
+                             const int32_t* __restrict__ uoff, const uint8_t* __restrict__ own,
+                             const int32_t* __restrict__ pri, const uint8_t* __restrict__ inU,
+                             const uint8_t* __restrict__ isW, const int32_t* __restrict__ widx,
+                             const int32_t* __restrict__ nid0, const int32_t* __restrict__ dnid,
+                             int4* __restrict__ rec, int32_t* __restrict__ nidu) {
+    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t e0 = uoff[v], g = vg[v];
+        rec[v] = make_int4(e0, uoff[v + 1] - e0, pri[v] + 2 * (G[g + 1].db - G[g].db),
+                           g << 2 | (inU[v] ? 2 : 0) | (own[v] ? 1 : 0));
+        nidu[v] = isW[v] ? dnid[widx[v]] : nid0[v];
+    }
+}
+
+__global__ void k_union_degree(int64_t nid, int32_t n, const int4* __restrict__ rec, const int32_t* __restrict__ gid,
+                               int32_t* __restrict__ deg) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nid; i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t src = gid[i];
+        deg[i] = src < 0 ? 0 : src < n ? rec[src].y : 1;  // a sink slot has no edges
+    }
+}
+
+__global__ void k_union_rows(int64_t nid, int32_t n, const UnionGame* __restrict__ G, const int4* __restrict__ rec,
+                             const int32_t* __restrict__ utgt, const int32_t* __restrict__ nid0,
+                             const int32_t* __restrict__ nidu, const int32_t* __restrict__ dsrc,
+                             const int32_t* __restrict__ gid, const int32_t* __restrict__ roff,
+                             int32_t* __restrict__ rtgt, uint8_t* __restrict__ rflags, int32_t* __restrict__ rpri,
+                             int32_t* __restrict__ orig_of, int32_t* __restrict__ vgame,
+                             int32_t* __restrict__ dummy_of, int32_t* __restrict__ gsink,
+                             int32_t* __restrict__ strat) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nid; i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t src = gid[i];
+        const int32_t base = roff[i];
+        if (src < 0) {  // the sink slot after its game's vertices
+            const int32_t prev = gid[i - 1];
+            const int32_t g = rec[prev < n ? prev : dsrc[prev - n]].w >> 2;
+            rflags[i] = kSinkSlot;
+            rpri[i] = -1;
+            orig_of[i] = -1;
+            vgame[i] = g;
+            gsink[g] = (int32_t)i;
+            strat[i] = (int32_t)i;
+            continue;
+        }
+        const int32_t w = src < n ? src : dsrc[src - n];
+        const int4 r = rec[w];
+        const int32_t g = r.w >> 2;
+        int32_t p;
+        if (src < n) {
+            p = r.z;
+            const int32_t* map = (r.w & 2) ? nidu : nid0;
+            for (int32_t j = 0; j < r.y; ++j) rtgt[base + j] = map[utgt[r.x + j]];
+            rflags[i] = (uint8_t)(((r.w & 1) ? kOwnerOdd : 0) | ((p & 1) ? kPriOdd : 0));
+        } else {
+            p = 2 * (src - n - G[g].db);
+            rtgt[base] = nid0[w];
+            rflags[i] = 0;  // dummies are Even, their priorities too
+            dummy_of[src - n] = w - G[g].vb;
+        }
+        rpri[i] = p;
+        orig_of[i] = w - G[g].vb;
+        vgame[i] = g;
+    }
+}
+
 // The game's own arrays, stream-ordered on the load stream from the game
 // pool (no global allocation lock between concurrent loads); the load
 // synchronises its stream before returning, so they are valid on every stream
@@ -352,6 +533,74 @@ struct Temps {
 };
 
 }  // namespace
+
+// Odd's Even-free trap (Section 3's preprocessing): U and W as flags, the
+// position of each vertex of W among them (widx, its total at widx[n]), and the
+// counters that hold the peeling's error bits.
+struct Trap {
+    uint8_t *inU, *isW;
+    int32_t* widx;
+    Counters* pc;
+};
+
+static pg_status find_trap(pg_ctx* ctx, Temps& T, int32_t n, int64_t m, const int32_t* off, const int32_t* tgt,
+                           const uint8_t* own, Trap* out) {
+    cudaStream_t s = ctx->stream;
+    // reverse adjacency for the trap computation
+    int32_t *indeg, *roff, *radj, *fill, *cnt, *fa, *fb, *widx;
+    uint8_t *inU, *isW;
+    LoadScalars* sc;
+    PG_CUDA_TRY(ctx, T.get(&sc, 1));
+    PG_CUDA_TRY(ctx, cudaMemsetAsync(sc, 0, sizeof(LoadScalars), s));
+    size_t stb = scan_tmp_bytes((int64_t)n + 2) + 64;
+    void* stmp;
+    PG_CUDA_TRY(ctx, T.get((char**)&stmp, (int64_t)stb));
+    PG_CUDA_TRY(ctx, T.get(&indeg, n));
+    PG_CUDA_TRY(ctx, T.get(&roff, (int64_t)n + 1));
+    PG_CUDA_TRY(ctx, T.get(&radj, m));
+    PG_CUDA_TRY(ctx, T.get(&fill, (int64_t)n + 1));
+    PG_CUDA_TRY(ctx, cudaMemsetAsync(indeg, 0, sizeof(int32_t) * (size_t)n, s));
+    ++ctx->launches;
+    k_indegree<<<nblocks(n), kBlock, 0, s>>>(n, off, tgt, own, indeg);
+    ctx->launches += 3;
+    PG_CUDA_TRY(ctx, exclusive_scan_i32(indeg, roff, n, nullptr, stmp, stb, s));
+    PG_CUDA_TRY(ctx, cudaMemcpyAsync(fill, roff, sizeof(int32_t) * ((size_t)n + 1), cudaMemcpyDeviceToDevice, s));
+    ++ctx->launches;
+    k_reverse_scatter<<<nblocks(n), kBlock, 0, s>>>(n, off, tgt, own, fill, radj);
+
+    // U: greatest fixpoint by peeling
+    PG_CUDA_TRY(ctx, T.get(&cnt, n));
+    PG_CUDA_TRY(ctx, T.get(&fa, n));
+    PG_CUDA_TRY(ctx, T.get(&fb, n));
+    PG_CUDA_TRY(ctx, T.get(&inU, n));
+    Counters* pc;  // the peeling rounds' frontier counts and grid barrier
+    PG_CUDA_TRY(ctx, T.get(&pc, 1));
+    PG_CUDA_TRY(ctx, cudaMemsetAsync(pc, 0, sizeof(Counters), s));
+    ++ctx->launches;
+    k_trap_init<<<nblocks(n), kBlock, 0, s>>>(n, off, tgt, own, inU, cnt, fa, sc);
+    ++ctx->launches;
+    k_trap_peel_dfs<<<nblocks(n), kBlock, 0, s>>>(fa, sc, roff, radj, own, inU, cnt, fb, pc);
+    {  // the overflow list (in fb), if any, in rounds
+        int sms = 0, per = 0;
+        PG_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
+        PG_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_trap_peel_coop, kBlock, 0));
+        int blocks = std::max(1, sms * std::max(1, std::min(per, 4)));
+        int32_t max_rounds = n + 1;
+        void* args[] = {(void*)&roff, (void*)&radj, (void*)&own, (void*)&inU, (void*)&cnt,
+                        (void*)&fb,   (void*)&fa,   (void*)&pc,  (void*)&max_rounds};
+        ++ctx->launches;
+        PG_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((void*)k_trap_peel_coop, blocks, kBlock, args, 0, s));
+    }
+    PG_CUDA_TRY(ctx, T.get(&isW, n));
+    PG_CUDA_TRY(ctx, T.get(&widx, (int64_t)n + 1));
+    PG_CUDA_TRY(ctx, cudaMemsetAsync(isW, 0, (size_t)n, s));
+    ++ctx->launches;
+    k_mark_w<<<nblocks(n), kBlock, 0, s>>>(n, off, tgt, inU, isW);
+    ctx->launches += 3;
+    PG_CUDA_TRY(ctx, exclusive_scan_u8(isW, widx, n, stmp, stb, s));
+    *out = {inU, isW, widx, pc};
+    return PG_OK;
+}
 
 // Vertices whose priorities are checked for repeats before the load chooses its
 // mode: games with few distinct priorities repeat them within the first few
@@ -416,55 +665,14 @@ pg_status load_game_pass(pg_ctx* ctx, int32_t n, int64_t m, const int32_t* off_i
         cv = (h.err & kEDup) != 0;
     }
 
-    // reverse adjacency for the trap computation
-    int32_t *indeg, *roff, *radj, *fill, *cnt, *fa, *fb, *widx;
-    uint8_t *inU, *isW;
-    size_t stb = scan_tmp_bytes((int64_t)n + 2) + 64;
-    void* stmp;
-    PG_CUDA_TRY(ctx, T.get((char**)&stmp, (int64_t)stb));
-    PG_CUDA_TRY(ctx, T.get(&indeg, n));
-    PG_CUDA_TRY(ctx, T.get(&roff, (int64_t)n + 1));
-    PG_CUDA_TRY(ctx, T.get(&radj, m));
-    PG_CUDA_TRY(ctx, T.get(&fill, (int64_t)n + 1));
-    PG_CUDA_TRY(ctx, cudaMemsetAsync(indeg, 0, sizeof(int32_t) * (size_t)n, s));
-    ++ctx->launches;
-    k_indegree<<<nblocks(n), kBlock, 0, s>>>(n, off, tgt, own, indeg);
-    ctx->launches += 3;
-    PG_CUDA_TRY(ctx, exclusive_scan_i32(indeg, roff, n, nullptr, stmp, stb, s));
-    PG_CUDA_TRY(ctx, cudaMemcpyAsync(fill, roff, sizeof(int32_t) * ((size_t)n + 1), cudaMemcpyDeviceToDevice, s));
-    ++ctx->launches;
-    k_reverse_scatter<<<nblocks(n), kBlock, 0, s>>>(n, off, tgt, own, fill, radj);
-
-    // U: greatest fixpoint by peeling
-    PG_CUDA_TRY(ctx, T.get(&cnt, n));
-    PG_CUDA_TRY(ctx, T.get(&fa, n));
-    PG_CUDA_TRY(ctx, T.get(&fb, n));
-    PG_CUDA_TRY(ctx, T.get(&inU, n));
-    Counters* pc;  // the peeling rounds' frontier counts and grid barrier
-    PG_CUDA_TRY(ctx, T.get(&pc, 1));
-    PG_CUDA_TRY(ctx, cudaMemsetAsync(pc, 0, sizeof(Counters), s));
-    ++ctx->launches;
-    k_trap_init<<<nblocks(n), kBlock, 0, s>>>(n, off, tgt, own, inU, cnt, fa, sc);
-    ++ctx->launches;
-    k_trap_peel_dfs<<<nblocks(n), kBlock, 0, s>>>(fa, sc, roff, radj, own, inU, cnt, fb, pc);
-    {  // the overflow list (in fb), if any, in rounds
-        int sms = 0, per = 0;
-        PG_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
-        PG_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_trap_peel_coop, kBlock, 0));
-        int blocks = std::max(1, sms * std::max(1, std::min(per, 4)));
-        int32_t max_rounds = n + 1;
-        void* args[] = {(void*)&roff, (void*)&radj, (void*)&own, (void*)&inU, (void*)&cnt,
-                        (void*)&fb,   (void*)&fa,   (void*)&pc,  (void*)&max_rounds};
-        ++ctx->launches;
-        PG_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((void*)k_trap_peel_coop, blocks, kBlock, args, 0, s));
+    Trap trap;
+    {
+        pg_status st = find_trap(ctx, T, n, m, off, tgt, own, &trap);
+        if (st) return st;
     }
-    PG_CUDA_TRY(ctx, T.get(&isW, n));
-    PG_CUDA_TRY(ctx, T.get(&widx, (int64_t)n + 1));
-    PG_CUDA_TRY(ctx, cudaMemsetAsync(isW, 0, (size_t)n, s));
-    ++ctx->launches;
-    k_mark_w<<<nblocks(n), kBlock, 0, s>>>(n, off, tgt, inU, isW);
-    ctx->launches += 3;
-    PG_CUDA_TRY(ctx, exclusive_scan_u8(isW, widx, n, stmp, stb, s));
+    uint8_t *inU = trap.inU, *isW = trap.isW;
+    int32_t* widx = trap.widx;
+    Counters* pc = trap.pc;
     int32_t k = 0, peel_err = 0;
     PG_CUDA_TRY(ctx, cudaMemcpyAsync(&k, widx + n, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     PG_CUDA_TRY(ctx, cudaMemcpyAsync(&peel_err, &pc->err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
@@ -650,6 +858,161 @@ pg_status load_game(pg_ctx* ctx, int32_t n, int64_t m, const int32_t* off_in, co
     pg_status st = load_game_pass(ctx, n, m, off_in, tgt_in, own_in, pri_in, mem_kind, out, with_scratch, false, &again);
     if (st != PG_OK || !again) return st;
     return load_game_pass(ctx, n, m, off_in, tgt_in, own_in, pri_in, mem_kind, out, with_scratch, true, &again);
+}
+
+// One chunk of a batch: games c0 .. c0 + ng of the batch's packed inputs, loaded
+// together (the results are those of load_game and pack_games per game). *general
+// is set, and nothing returned, when some game needs the general path: an input
+// it refuses, repeated or very sparse priorities, sizes at the limits of int32.
+pg_status load_union(pg_ctx* ctx, int32_t ng, const int64_t* vb, const int64_t* eb, const int32_t* off_in,
+                     const int32_t* tgt_in, const uint8_t* own_in, const int32_t* pri_in, int32_t mem_kind,
+                     pg_game** out, bool* general) {
+    *out = nullptr;
+    *general = true;
+    const int64_t N = vb[ng] - vb[0], M = eb[ng] - eb[0];
+    if (N >= (1 << 28) || M + N > INT32_MAX - 1) return PG_OK;
+    for (int32_t i = 0; i < ng; ++i)
+        if (eb[i + 1] - eb[i] < vb[i + 1] - vb[i]) return PG_OK;
+    const int32_t n = (int32_t)N;
+    cudaStream_t s = ctx->stream;
+    Temps T(ctx, s);
+    std::vector<UnionGame> G(ng + 1);
+    for (int32_t i = 0; i <= ng; ++i) G[i] = {(int32_t)(vb[i] - vb[0]), (int32_t)(eb[i] - eb[0]), 0, 0};
+    UnionGame* dG;
+    int32_t *vg, *uoff, *utgt, *gstat;
+    PG_CUDA_TRY(ctx, T.get(&dG, ng + 1));
+    PG_CUDA_TRY(ctx, T.get(&vg, N));
+    PG_CUDA_TRY(ctx, T.get(&uoff, N + 1));
+    PG_CUDA_TRY(ctx, T.get(&utgt, M));
+    PG_CUDA_TRY(ctx, T.get(&gstat, 2 * (int64_t)ng + 1));  // per game: error bits; largest priority; a repeat
+    const int32_t *off = off_in + vb[0], *tgt = tgt_in + eb[0], *pri = pri_in + vb[0];
+    const uint8_t* own = own_in + vb[0];
+    if (mem_kind == PG_MEM_HOST) {
+        int32_t *o, *t, *p;
+        uint8_t* w;
+        PG_CUDA_TRY(ctx, T.get(&o, N + ng));
+        PG_CUDA_TRY(ctx, T.get(&t, M));
+        PG_CUDA_TRY(ctx, T.get(&w, N));
+        PG_CUDA_TRY(ctx, T.get(&p, N));
+        PG_CUDA_TRY(ctx, cudaMemcpyAsync(o, off, sizeof(int32_t) * (size_t)(N + ng), cudaMemcpyHostToDevice, s));
+        PG_CUDA_TRY(ctx, cudaMemcpyAsync(t, tgt, sizeof(int32_t) * (size_t)M, cudaMemcpyHostToDevice, s));
+        PG_CUDA_TRY(ctx, cudaMemcpyAsync(w, own, (size_t)N, cudaMemcpyHostToDevice, s));
+        PG_CUDA_TRY(ctx, cudaMemcpyAsync(p, pri, sizeof(int32_t) * (size_t)N, cudaMemcpyHostToDevice, s));
+        off = o;
+        tgt = t;
+        own = w;
+        pri = p;
+    }
+    PG_CUDA_TRY(ctx, cudaMemcpyAsync(dG, G.data(), sizeof(UnionGame) * (size_t)(ng + 1), cudaMemcpyHostToDevice, s));
+    PG_CUDA_TRY(ctx, cudaMemsetAsync(gstat, 0, sizeof(int32_t) * (size_t)(2 * (int64_t)ng + 1), s));
+    k_union_prepare<<<nblocks(n), kBlock, 0, s>>>(n, ng, dG, off, tgt, own, pri, vg, uoff, utgt, gstat, gstat + ng);
+    PG_CUDA_TRY(ctx, cudaGetLastError());
+    std::vector<int32_t> hstat(2 * (size_t)ng);
+    PG_CUDA_TRY(ctx, cudaMemcpyAsync(hstat.data(), gstat, sizeof(int32_t) * hstat.size(), cudaMemcpyDeviceToHost, s));
+    PG_CUDA_TRY(ctx, cudaStreamSynchronize(s));
+    for (int32_t i = 0; i < ng; ++i)
+        if (hstat[i]) return PG_OK;
+
+    // Odd's trap on the union (as load_game_pass)
+    Trap trap;
+    pg_status st = find_trap(ctx, T, n, M, uoff, utgt, own, &trap);
+    if (st) return st;
+    int32_t* dsrc;
+    PG_CUDA_TRY(ctx, T.get(&dsrc, N));
+    k_union_dummies<<<nblocks(N + 1), kBlock, 0, s>>>(n, ng, dG, trap.isW, trap.widx, vg, dsrc);
+    PG_CUDA_TRY(ctx, cudaGetLastError());
+    int32_t peel_err = 0;
+    PG_CUDA_TRY(ctx, cudaMemcpyAsync(&peel_err, &trap.pc->err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    PG_CUDA_TRY(ctx, cudaMemcpyAsync(G.data(), dG, sizeof(UnionGame) * G.size(), cudaMemcpyDeviceToHost, s));
+    PG_CUDA_TRY(ctx, cudaStreamSynchronize(s));
+    if (peel_err) return PG_OK;
+    const int64_t K = G[ng].db, NP = N + K, ids = NP + ng;
+    if (ids >= (1 << 29) - 1 || M + K > INT32_MAX - 1) return PG_OK;
+    int64_t words = 0;
+    for (int32_t i = 0; i < ng; ++i) {
+        const int64_t top = (int64_t)hstat[ng + i] + 2 * (int64_t)(G[i + 1].db - G[i].db);
+        if (top > INT32_MAX - 1) return PG_OK;
+        G[i].words = (int32_t)words;
+        words += (top >> 5) + 1;
+        if (words > NP + 64 * (int64_t)ng) return PG_OK;  // sparse priorities: at most a word per vertex here
+    }
+
+    pg_game* g = new pg_game();
+    g->ctx = ctx;
+    g->device = ctx->device;
+    g->ngames = ng;
+    g->n0 = N;
+    g->m0 = M;
+    g->k = (int32_t)K;
+    g->n = (int32_t)ids;
+    g->m = M + K;
+    auto bail = [&](cudaError_t e, const char* where) {
+        free_game(g);
+        return cuda_fail(ctx, e, where);
+    };
+#define LU_TRY(expr)                                   \
+    do {                                               \
+        cudaError_t _e = (expr);                       \
+        if (_e != cudaSuccess) return bail(_e, #expr); \
+    } while (0)
+    LU_TRY(dalloc(ctx, &g->off, ids + 1, s));
+    LU_TRY(dalloc(ctx, &g->tgt, M + K, s));
+    LU_TRY(dalloc(ctx, &g->flags, ids, s));
+    LU_TRY(dalloc(ctx, &g->pri, ids, s));
+    LU_TRY(dalloc(ctx, &g->nid0, N, s));
+    LU_TRY(dalloc(ctx, &g->orig_of, ids, s));
+    LU_TRY(dalloc(ctx, &g->dnid, K, s));
+    LU_TRY(dalloc(ctx, &g->dummy_of, K, s));
+    LU_TRY(dalloc(ctx, &g->vgame, ids, s));
+    LU_TRY(dalloc(ctx, &g->strat, ids, s));
+    LU_TRY(dalloc(ctx, &g->gsink, ng, s));
+    uint32_t* bits;
+    int32_t *wprefix, *gid, *deg, *nidu;
+    int4* rec;
+    void* stmp;
+    const size_t stb = scan_tmp_bytes(std::max<int64_t>(words, ids) + 2) + 64;
+    LU_TRY(T.get(&bits, words));
+    LU_TRY(T.get(&wprefix, words + 1));
+    LU_TRY(T.get(&gid, ids));
+    LU_TRY(T.get(&deg, ids));
+    LU_TRY(T.get(&nidu, N));
+    LU_TRY(T.get(&rec, N));
+    LU_TRY(T.get((char**)&stmp, (int64_t)stb));
+    LU_TRY(cudaMemcpyAsync(dG, G.data(), sizeof(UnionGame) * G.size(), cudaMemcpyHostToDevice, s));
+    LU_TRY(cudaMemsetAsync(bits, 0, sizeof(uint32_t) * (size_t)words, s));
+    int32_t* dup = gstat + 2 * (int64_t)ng;
+    k_union_mark<<<nblocks(NP), kBlock, 0, s>>>(NP, n, dG, vg, pri, dsrc, bits, dup);
+    int32_t hdup = 0;
+    LU_TRY(cudaMemcpyAsync(&hdup, dup, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    LU_TRY(cudaStreamSynchronize(s));
+    if (hdup) {  // two vertices of one rank: the general path says which game
+        free_game(g);
+        return PG_OK;
+    }
+    LU_TRY(exclusive_popc_scan(bits, wprefix, words, stmp, stb, s));
+    LU_TRY(cudaMemsetAsync(gid, 0xff, sizeof(int32_t) * (size_t)ids, s));  // what no vertex takes is a sink slot
+    k_union_rank<<<nblocks(NP), kBlock, 0, s>>>(NP, n, dG, vg, pri, dsrc, bits, wprefix, g->nid0, g->dnid, gid);
+    k_union_pack<<<nblocks(n), kBlock, 0, s>>>(n, dG, vg, uoff, own, pri, trap.inU, trap.isW, trap.widx, g->nid0,
+                                               g->dnid, rec, nidu);
+    k_union_degree<<<nblocks(ids), kBlock, 0, s>>>(ids, n, rec, gid, deg);
+    LU_TRY(exclusive_scan_i32(deg, g->off, ids, nullptr, stmp, stb, s));
+    k_union_rows<<<nblocks(ids), kBlock, 0, s>>>(ids, n, dG, rec, utgt, g->nid0, nidu, dsrc, gid, g->off, g->tgt,
+                                                 g->flags, g->pri, g->orig_of, g->vgame, g->dummy_of, g->gsink,
+                                                 g->strat);
+    LU_TRY(cudaGetLastError());
+    LU_TRY(cudaMemcpyAsync(&g->sink0, g->gsink, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    LU_TRY(cudaStreamSynchronize(s));
+#undef LU_TRY
+    ctx->launches += 13;
+    g->h_base0.resize(ng + 1);
+    g->h_dbase.resize(ng + 1);
+    for (int32_t i = 0; i <= ng; ++i) {
+        g->h_base0[i] = G[i].vb;
+        g->h_dbase[i] = G[i].db;
+    }
+    *general = false;
+    *out = g;
+    return PG_OK;
 }
 
 }  // namespace pg
