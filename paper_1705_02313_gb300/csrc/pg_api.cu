@@ -86,12 +86,12 @@ void free_game(pg_game* g) {
     if (!g) return;
     void* ptrs[] = {g->off,  g->off64,   g->vgame, g->gsink, g->gst,   g->gactive, g->gscan,
                     g->tgt,     g->flags, g->pri,   g->nid0,  g->orig_of, g->dnid,    g->dummy_of,
-                    g->strat, g->gd,     g->gd32,  g->kind,  g->plist, g->slot,  g->ccnt,  g->coff,    g->cl_ks,   g->sz,
-                    g->sinkval, g->wgt,  g->oddsz, g->key,   g->cls,   g->depth,   g->dom,     g->hugelist,
+                    g->strat, g->gd,     g->gd32,  g->kind,  g->ccnt,  g->coff,    g->cl_ks,   g->sz,
+                    g->wgt,  g->oddsz, g->key,   g->cls,   g->depth,   g->dom,
                     g->tiles, g->tsum,   g->cnt,    g->scan_tmp, g->stage, g->loop_iters, g->ws, g->wsB, g->gdB, g->key128,
                     g->d_anc, g->d_sc, g->d_podd, g->d_peven, g->d_oddL, g->d_evenL, g->d_nxt, g->d_wt, g->d_loc,
                     g->d_own, g->d_rid, g->d_rl, g->d_val, g->d_rnx, g->pl_vid[0], g->pl_vid[1], g->pl_off[0],
-                    g->pl_off[1], g->pl_tgt[0], g->pl_tgt[1], g->rv, g->rv_src, g->omark, g->emark, g->inc};
+                    g->pl_off[1], g->pl_tgt[0], g->pl_tgt[1], g->rv, g->rv_src, g->omark, g->emark, g->inc, g->quad};
     int prev = -1;
     const bool switched =
         cudaGetDevice(&prev) == cudaSuccess && prev != g->device && cudaSetDevice(g->device) == cudaSuccess;
@@ -116,8 +116,6 @@ inline unsigned grid_of(int64_t n) {
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>(b, 152 * 64));
 }
 
-// Sets g->strat from a profile given in original ids (NULL arrays take the
-// defaults: Even and dummies to the sink, Odd to its first edge).
 __device__ inline int32_t sink_id(int32_t i, const int32_t* vgame, const int32_t* gsink, int32_t sink0) {
     return vgame ? gsink[vgame[i]] : sink0;
 }
@@ -136,45 +134,47 @@ __global__ void k_default_profile(int32_t n, const OffT* __restrict__ off, const
     }
 }
 
+// A profile given in original ids, for one game. In relabelled order, so that a
+// vertex's edges and its entry of strat are read and written in order and only
+// two reads per vertex are random, its successor's original id and that one's id
+// (in the caller's order all but the successor were: 4M random game 138 us, 10M
+// chain 465 us). The dummies, whose priorities are the lowest, have the first k
+// ids; the edges of a vertex lead to t or, redirected, to t's dummy.
 template <typename OffT>
-__global__ void k_apply_profile(int64_t n0, int32_t k, const int32_t* __restrict__ nid0,
+__global__ void k_apply_profile(int32_t n, int32_t n0, int32_t k, const int32_t* __restrict__ nid0,
                                 const OffT* __restrict__ off, const int32_t* __restrict__ tgt,
                                 const uint8_t* __restrict__ flags, const int32_t* __restrict__ orig_of,
-                                const int32_t* __restrict__ dnid, const int32_t* __restrict__ vgame,
-                                const int32_t* __restrict__ gsink, int32_t sink0, const int32_t* sigma,
-                                const int32_t* tau, const int8_t* dsig, int32_t* strat, int32_t* err) {
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n0 + (int64_t)k;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        if (v >= n0) {
-            int32_t d = dnid[v - n0];
-            strat[d] = (dsig && dsig[v - n0]) ? tgt[off[d]] : sink_id(d, vgame, gsink, sink0);
+                                int32_t sink0, const int32_t* __restrict__ sigma, const int32_t* __restrict__ tau,
+                                const int8_t* __restrict__ dsig, int32_t* __restrict__ strat, int32_t* err) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        if (i == sink0) continue;
+        if (i < k) {
+            strat[i] = (dsig && dsig[i]) ? tgt[off[i]] : sink0;
             continue;
         }
-        int32_t i = nid0[v];
-        const int32_t n = sink_id(i, vgame, gsink, sink0);
-        bool odd = (flags[i] & kOwnerOdd) != 0;
+        const bool odd = (flags[i] & kOwnerOdd) != 0;
         const int32_t* src = odd ? tau : sigma;
+        const int64_t e0 = off[i], e1 = off[i + 1];
         if (!src) {
-            strat[i] = odd ? tgt[off[i]] : n;
+            strat[i] = odd ? tgt[e0] : sink0;
             continue;
         }
-        int32_t t = src[v];
+        const int32_t t = src[orig_of[i]];
         if (!odd && t == -1) {
-            strat[i] = n;
+            strat[i] = sink0;
             continue;
         }
+        const int32_t want = t >= 0 && t < n0 ? nid0[t] : -1;
         int32_t pick = -1;
-        for (OffT e = off[i]; e < off[i + 1]; ++e)
-            if (orig_of[tgt[e]] == t) {
-                pick = tgt[e];
-                break;
-            }
+        for (int64_t e = e0; e < e1 && pick < 0 && want >= 0; ++e) {
+            const int32_t x = tgt[e];
+            if (x == want || (x < k && orig_of[x] == t)) pick = x;
+        }
         if (pick < 0) {
             atomicOr(err, 1);
-            strat[i] = odd ? tgt[off[i]] : n;
-        } else {
-            strat[i] = pick;
+            pick = odd ? tgt[e0] : sink0;
         }
+        strat[i] = pick;
     }
 }
 
@@ -190,32 +190,56 @@ struct OutPtrs {
     int8_t* dsig;
 };
 
-__global__ void k_results(int64_t n0, int32_t k, const int32_t* __restrict__ nid0,
-                          const int32_t* __restrict__ dnid, const uint8_t* __restrict__ flags,
+// What the outputs read of each id, packed in relabelled order: x = its
+// successor's original vertex (-1: the sink), y = depth, z = rank of a finite
+// vertex or dominant priority of a TOP one, w = bit 0: finite, bit 1: Odd's.
+// Arrays that no output needs are null.
+constexpr int32_t kRecFin = 1, kRecOdd = 2;
+__global__ void k_records(int32_t lo, int32_t hi, const uint8_t* __restrict__ flags,
                           const int32_t* __restrict__ strat, const uint8_t* __restrict__ cls,
                           const int32_t* __restrict__ depth, const int32_t* __restrict__ key,
                           const int32_t* __restrict__ orig_of, const int32_t* __restrict__ dom,
                           const int32_t* __restrict__ vgame, const int32_t* __restrict__ gsink, int32_t sink0,
-                          OutPtrs o) {
+                          int4* __restrict__ rec) {
+    for (int64_t i = lo + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < hi;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const uint8_t f = flags[i];
+        if (f & kSinkSlot) continue;
+        const bool fin = cls[i] == kFin;
+        int4 r = make_int4(-1, -1, 0, (fin ? kRecFin : 0) | ((f & kOwnerOdd) ? kRecOdd : 0));
+        if (strat) {
+            const int32_t s = strat[i];
+            if (s != sink_id((int32_t)i, vgame, gsink, sink0)) r.x = orig_of[s];
+        }
+        if (depth && fin) r.y = depth[i];
+        if (fin ? key != nullptr : dom != nullptr) r.z = fin ? key[i] : dom[i];
+        rec[i] = r;
+    }
+}
+
+// The outputs in the caller's order, from one 16-byte record per vertex: read
+// field by field they took seven random reads (10M random game 470 us).
+__global__ void k_results(int64_t n0, int32_t k, const int32_t* __restrict__ nid0,
+                          const int32_t* __restrict__ dnid, const int32_t* __restrict__ strat,
+                          const int4* __restrict__ rec, const int32_t* __restrict__ vgame,
+                          const int32_t* __restrict__ gsink, int32_t sink0, OutPtrs o) {
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n0 + (int64_t)k;
          v += (int64_t)gridDim.x * blockDim.x) {
         if (v >= n0) {
+            if (!o.dsig) return;
             const int32_t d = dnid[v - n0];
-            if (o.dsig) o.dsig[v - n0] = strat[d] != sink_id(d, vgame, gsink, sink0);
+            o.dsig[v - n0] = strat[d] != sink_id(d, vgame, gsink, sink0);
             continue;
         }
-        int32_t i = nid0[v];
-        const int32_t n = sink_id(i, vgame, gsink, sink0);
-        bool fin = cls[i] == kFin;
-        bool odd = (flags[i] & kOwnerOdd) != 0;
-        int32_t s = strat[i];
+        const int4 r = rec[nid0[v]];
+        const bool fin = (r.w & kRecFin) != 0, odd = (r.w & kRecOdd) != 0;
         if (o.win) o.win[v] = fin ? 1 : 0;
-        if (o.sigma) o.sigma[v] = odd ? -1 : (s == n ? -1 : orig_of[s]);
-        if (o.tau) o.tau[v] = odd ? orig_of[s] : -1;
+        if (o.sigma) o.sigma[v] = odd ? -1 : r.x;
+        if (o.tau) o.tau[v] = odd ? r.x : -1;
         if (o.vclass) o.vclass[v] = fin ? 0 : 1;
-        if (o.vdepth) o.vdepth[v] = fin ? depth[i] : -1;
-        if (o.vrank) o.vrank[v] = o.cv ? -1 : (fin ? key[i] : INT32_MAX);
-        if (o.vdom) o.vdom[v] = dom[i];
+        if (o.vdepth) o.vdepth[v] = fin ? r.y : -1;
+        if (o.vrank) o.vrank[v] = o.cv ? -1 : (fin ? r.z : INT32_MAX);
+        if (o.vdom) o.vdom[v] = fin ? -1 : r.z;
     }
 }
 
@@ -262,9 +286,12 @@ pg_status write_outputs(pg_game* g, int32_t mem_kind, uint8_t* win, int32_t* sig
         pg_status st = enqueue_depth(g);
         if (st) return st;
     }
-    ctx->launches += 1;
-    k_results<<<grid_of((int64_t)g->n0 + g->k), kBlock, 0, s>>>(g->n0, g->k, g->nid0, g->dnid, g->flags, g->strat,
-                                                                g->cls, g->depth, g->key, g->orig_of, g->dom,
+    const int32_t hi = g->rec_hi ? g->rec_hi : g->n;
+    ctx->launches += 2;
+    k_records<<<grid_of(hi - g->rec_lo), kBlock, 0, s>>>(
+        g->rec_lo, hi, g->flags, sigma || tau ? g->strat : nullptr, g->cls, vdepth ? g->depth : nullptr,
+        vrank && !g->cv ? g->key : nullptr, g->orig_of, vdom ? g->dom : nullptr, g->vgame, g->gsink, g->sink0, g->rec);
+    k_results<<<grid_of((int64_t)g->n0 + g->k), kBlock, 0, s>>>(g->n0, g->k, g->nid0, g->dnid, g->strat, g->rec,
                                                                 g->vgame, g->gsink, g->sink0, o);
     PG_CUDA_TRY(ctx, cudaGetLastError());
     if (mem_kind == PG_MEM_HOST) {
@@ -327,13 +354,13 @@ pg_status apply_profile(pg_game* g, const int32_t* sigma, const int32_t* tau, co
     if (e == cudaSuccess) {
         ctx->launches += 1;
         if (g->off64)
-            k_apply_profile<int64_t><<<grid_of((int64_t)g->n0 + g->k), kBlock, 0, s>>>(
-                g->n0, g->k, g->nid0, g->off64, g->tgt, g->flags, g->orig_of, g->dnid, g->vgame, g->gsink, g->sink0, ds,
-                dt, dd, g->strat, err);
+            k_apply_profile<int64_t><<<grid_of(g->n), kBlock, 0, s>>>(g->n, (int32_t)g->n0, g->k, g->nid0, g->off64,
+                                                                      g->tgt, g->flags, g->orig_of, g->sink0, ds, dt,
+                                                                      dd, g->strat, err);
         else
-            k_apply_profile<int32_t><<<grid_of((int64_t)g->n0 + g->k), kBlock, 0, s>>>(
-                g->n0, g->k, g->nid0, g->off, g->tgt, g->flags, g->orig_of, g->dnid, g->vgame, g->gsink, g->sink0, ds,
-                dt, dd, g->strat, err);
+            k_apply_profile<int32_t><<<grid_of(g->n), kBlock, 0, s>>>(g->n, (int32_t)g->n0, g->k, g->nid0, g->off,
+                                                                      g->tgt, g->flags, g->orig_of, g->sink0, ds, dt,
+                                                                      dd, g->strat, err);
         e = cudaMemcpyAsync(ctx->pinned, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -538,13 +565,13 @@ pg_status run_loop_once(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t l
 // game continues from the same profile with the ruling-set ranks (for the
 // rest of this call), so the trajectory is unchanged.
 pg_status run_loop(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t limit) {
-    if (runs_whole(g, tm)) {
+    g->depth_ok = false;
+    if (runs_whole(g, tm) || (g->cv && !tm.on && g->ctx->graphs && inc_applies(g))) {
         pg_status st = build_reverse(g, 0);
-        if (st) return st;
-    } else if (g->cv && !tm.on && g->ctx->graphs && inc_applies(g)) {
-        pg_status st = build_reverse(g, 0);
-        if (st) return st;
-    } else if (loop_compares(g) && !g->pl_ok) {
+        if (st == PG_ENOMEM) g->no_inc = true;  // the loop without incremental iterations
+        else if (st) return st;
+    }
+    if (!runs_whole(g, tm) && loop_compares(g) && !g->pl_ok) {
         pg_status st = build_player_split(g);
         if (st) return st;
     }
@@ -879,11 +906,12 @@ pg_status pg_best_response(pg_game* g, const int32_t* sigma, const int8_t* dummy
     if (st) return st;
     tm.mark(2);
     g->t_total = tm.since(3, 2);
-    st = write_outputs(g, mem_kind, nullptr, nullptr, tau_inout, nullptr, nullptr, nullptr, nullptr, nullptr);
+    const bool apart = !out || out->mem_kind != mem_kind;  // else the strategy comes with the valuation
+    if (apart) st = write_outputs(g, mem_kind, nullptr, nullptr, tau_inout, nullptr, nullptr, nullptr, nullptr, nullptr);
     if (st) return st;
     if (out) {
-        st = write_outputs(g, out->mem_kind, nullptr, nullptr, nullptr, out->val_class, out->val_depth,
-                           out->val_rank, nullptr, nullptr);
+        st = write_outputs(g, out->mem_kind, nullptr, nullptr, apart ? nullptr : tau_inout, out->val_class,
+                           out->val_depth, out->val_rank, nullptr, nullptr);
         if (!st && g->cv && out->val_counts) st = write_counts(g, out->mem_kind, out->val_counts);
         if (st) return st;
         if (out->dom) {

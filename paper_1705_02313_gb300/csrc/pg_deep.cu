@@ -759,7 +759,7 @@ pg_status enqueue_valuation_deep(pg_game* g, bool want_dom) {
                                            g->gsink, g->sink0, g->key, g->depth, c);
     prof_end(g, KID_DEEP, 20);
     PG_CUDA_TRY(ctx, cudaGetLastError());
-    g->val_deep = true;
+    g->val_deep = g->depth_ok = true;
     return PG_OK;
 }
 

@@ -655,16 +655,34 @@ __global__ void __launch_bounds__(kBlock) k_rv_fill(int32_t n, const OffT* __res
 
 }  // namespace
 
-bool inc_applies(const pg_game* g) { return !g->vgame && g->ngames == 1 && g->off != nullptr; }
+bool inc_applies(const pg_game* g) { return !g->vgame && g->ngames == 1 && g->off != nullptr && !g->no_inc; }
+
+static void drop_reverse(pg_game* g) {
+    g->rv_ok = false;
+    for (void** q : {(void**)&g->rv, (void**)&g->rv_src, (void**)&g->omark, (void**)&g->emark}) {
+        if (*q) cudaFreeAsync(*q, g->ctx->stream);
+        *q = nullptr;
+    }
+}
+
+static pg_status make_reverse(pg_game* g, int64_t odd_edges);
 
 pg_status build_reverse(pg_game* g, int64_t odd_edges) {
     if (g->rv_ok) return PG_OK;
+    drop_reverse(g);
+    pg_status st = make_reverse(g, odd_edges);
+    if (!st) {
+        g->rv_ok = true;
+        return PG_OK;
+    }
+    drop_reverse(g);
+    if (st == PG_ENOMEM) cudaGetLastError();
+    return st;
+}
+
+static pg_status make_reverse(pg_game* g, int64_t odd_edges) {
     pg_ctx* ctx = g->ctx;
     cudaStream_t s = ctx->stream;
-    for (void** q : {(void**)&g->rv, (void**)&g->rv_src, (void**)&g->omark, (void**)&g->emark}) {
-        if (*q) cudaFreeAsync(*q, s);
-        *q = nullptr;
-    }
     const int32_t n = g->n;
     // packed games take no incremental iterations: their lists hold Odd's edges only (the marks of k_classify)
     const int odd_only = inc_applies(g) ? 0 : 1;
@@ -704,7 +722,6 @@ pg_status build_reverse(pg_game* g, int64_t odd_edges) {
     });
     PG_CUDA_TRY(ctx, cudaGetLastError());
     ctx->launches += 4;
-    g->rv_ok = true;
     return PG_OK;
 }
 

@@ -274,6 +274,9 @@ struct pg_game {
     int coop_blocks = 0;         // co-resident blocks for the cooperative kernels
     int chain1_blocks = 0;       // k_chain1 blocks resident at once (0: one block per 8 tiles)
     void* stage = nullptr;       // staging for host outputs
+    int32_t* quad = nullptr;     // [4 n] plist, slot, sinkval and hugelist; rec while outputs are written
+    int4* rec = nullptr;         // [n] what the outputs read of each id (write_outputs)
+    int32_t rec_lo = 0, rec_hi = 0;  // the ids whose outputs are written (0, 0: all)
     int64_t* loop_iters = nullptr;  // [2] iterations and loop bodies run by the device-side loop
     // instantiated loop graphs: [0] inner loop only, [1] both players; built for loop_cap[i]
     cudaGraphExec_t loop_exec[2] = {nullptr, nullptr};
@@ -300,11 +303,13 @@ struct pg_game {
     uint8_t* omark = nullptr;
     uint8_t* emark = nullptr;
     bool rv_ok = false;           // the four above are complete
+    bool no_inc = false;          // there is no memory for Even's lists: no incremental iterations
     pg::IncState* inc = nullptr;  // incremental iterations (pg_inc.cu; single games)
     int inc_cluster = 0;          // blocks of their cluster (0: not yet asked)
     // ruling-set ranks (pg_deep.cu), for games whose g-forest is deep
     bool deep_mode = false;      // every valuation of the current call takes the ruling-set path
-    bool val_deep = false;       // the last valuation took it (its depths are written; no depth pass)
+    bool val_deep = false;       // the last valuation took it
+    bool depth_ok = false;       // the last valuation wrote the depths (no depth pass)
     int32_t* d_anc = nullptr;    // [n] root of each vertex's g-chain
     uint8_t* d_sc = nullptr;     // [2n] the sink's odd and even children (flags for the compactions)
     int32_t* d_podd = nullptr;   // [n+1] positions of the sink's odd children
@@ -411,9 +416,9 @@ void prof_end(pg_game* g, int id, int nlaunch);
 void prof_collect(pg_game* g);  // after a stream synchronisation
 // Resets the between-valuation invariants of the scratch arrays (once per call).
 pg_status reset_scratch(pg_game* g);
-// Enqueues one valuation of g->strat: cls, depth, key (and dom when want_dom). No host synchronisation.
-pg_status enqueue_valuation(pg_game* g, bool want_dom);
-// Enqueues the depth pass (outputs only; after a valuation).
+// Enqueues one valuation of g->strat: cls, key (depth and dom when asked for). No host synchronisation.
+pg_status enqueue_valuation(pg_game* g, bool want_dom, bool with_depth = false);
+// Enqueues the depth pass (outputs only; after a valuation) unless the valuation wrote the depths.
 pg_status enqueue_depth(pg_game* g);
 // Enqueues one switching pass for player (0 Even, 1 Odd) using g->key. No host synchronisation.
 pg_status enqueue_switch(pg_game* g, int player);

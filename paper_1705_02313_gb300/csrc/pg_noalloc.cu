@@ -203,8 +203,7 @@ extern "C" pg_status pg_valuate_static(int32_t n, const int32_t* succ, const uin
     if (cudaGetLastError() != cudaSuccess) return PG_ECUDA;
 
     st = reset_scratch(&g);  // the buffer keeps the previous call's contents
-    if (st == PG_OK) st = enqueue_valuation(&g, false);
-    if (st == PG_OK) st = enqueue_depth(&g);
+    if (st == PG_OK) st = enqueue_valuation(&g, false, true);
     if (st != PG_OK) return st;
     k_static_results<<<(unsigned)std::min<int64_t>(((int64_t)n + kBlock - 1) / kBlock, 4096), kBlock, 0, s>>>(
         n, g.cls, g.depth, g.key, val_class, val_depth, val_rank);

@@ -297,6 +297,8 @@ pg_status collect(pg_server* sv, size_t i, Done* d) {
     view.n0 = n0;
     view.k = k;
     view.stage = sv->stage;
+    for (size_t j = 0; j < i; ++j) view.rec_lo += sv->res[j].g->n;  // its ids
+    view.rec_hi = view.rec_lo + sv->res[i].g->n;
     d->n = (int32_t)n0;
     d->k = k;
     d->win.resize(n0);
