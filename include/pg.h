@@ -367,8 +367,8 @@ pg_status pg_best_response_bf(pg_game *game, const int32_t *sigma, const int8_t 
  * error. No message is recorded.
  *
  * Set-up: every call looks up the fixed array's device address on the current
- * device (a lookup, no allocation); the first call on a device also computes
- * the cooperative launch size and keeps it. All calls share the array and it
+ * device (a lookup, no allocation); the first call on a device also asks for
+ * the size of its cluster launches and keeps it. All calls share the array and it
  * keeps the last call's contents (each call clears what must start at zero),
  * so calls that overlap on the GPU, from any thread or stream, race:
  * serialise them. */

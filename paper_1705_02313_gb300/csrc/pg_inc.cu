@@ -730,26 +730,7 @@ int32_t inc_max_seeds(const pg_game* g) {
                  : std::max(1, std::min(g->n / kIncSeedShare, kIncSeeds));
 }
 
-static int inc_cluster_for(void (*kern)(IncArgs), int want) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kIncShared);
-    for (int c = want; c > 1; c >>= 1) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(c);
-        cfg.blockDim = dim3(kIncThreads);
-        cfg.dynamicSmemBytes = kIncShared;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = c;
-        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        int k = 0;
-        if (cudaOccupancyMaxActiveClusters(&k, kern, &cfg) == cudaSuccess && k > 0) return c;
-        cudaGetLastError();
-    }
-    return 1;
-}
+static std::atomic<int> g_inc_cluster[2][kClusterDevices];
 
 pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole) {
     pg_ctx* ctx = g->ctx;
@@ -786,8 +767,8 @@ pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole) {
     if (whole)
         while (want > 1 && (int64_t)want * kIncThreads / 2 >= g->n) want >>= 1;
     auto kern = g->cv ? k_inc<true> : k_inc<false>;
-    if (!g->inc_cluster) g->inc_cluster = inc_cluster_for(kern, kIncCluster);
-    const int c = std::min(want, g->inc_cluster);
+    const int c = std::min(want, cluster_blocks((const void*)kern, kIncThreads, kIncShared, kIncCluster, g->device,
+                                                g_inc_cluster[g->cv ? 1 : 0]));
     a.max_seeds = std::min(whole ? std::max(1, g->n / kIncWholeShare) : inc_max_seeds(g), c * (kIncSet / 2));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(c);

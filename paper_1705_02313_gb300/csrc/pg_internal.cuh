@@ -12,6 +12,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -26,6 +27,8 @@ constexpr int kJumpFollow = 32;       // resolved vertices a pointer-jumping rou
 constexpr int kJumpRoundsDeep = 4096; // extra pointer-jumping rounds allowed on the ruling-set path
 constexpr int kHugeChildren = 4096;   // a parent with more children is ranked by an id-ordered scan instead
 constexpr int kCoopTile = 4096;       // elements per tile of the id-ordered scans
+constexpr int kClusterDevices = 64;   // devices whose cluster sizes are remembered
+constexpr int32_t kSmallIds = (1 << 18) + 1;  // a game of up to this many ids is valuated by one cluster (pg_small.cu)
 // Count-vector mode (repeated priorities): at most kMaxLevels distinct
 // priorities; a count vector is one signed 128-bit key with one digit per
 // level (Levels::shift), each wide enough that its signed count stays below
@@ -78,6 +81,7 @@ struct Counters {
     int32_t n_huge;      // parents ranked by the id-ordered scan
     int32_t n_big;       // parents ranked by one block each
     int32_t n_switch;    // switched vertices in the last switching pass (all games)
+    int32_t bad;         // successors out of range (pg_valuate_static)
     int32_t n_list;      // vertices switched since the valuation, listed for k_inc as far as it takes them
     int32_t err;         // device-side error bits (kErr*)
     int32_t sink_rank;   // rank of game 0's sink (its empty valuation)
@@ -271,6 +275,11 @@ struct pg_game {
     pg::Counters* hcnt = nullptr;// pinned host copy
     void* scan_tmp = nullptr;    // children-count scan scratch
     size_t scan_tmp_bytes = 0;
+    // pg_valuate_static: the caller's successors and parities, which the valuation copies and checks first
+    const int32_t* in_succ = nullptr;
+    const uint8_t* in_odd = nullptr;
+    int8_t* out_class = nullptr;  // and its outputs, which the valuation writes
+    int32_t *out_depth = nullptr, *out_rank = nullptr;
     int coop_blocks = 0;         // co-resident blocks for the cooperative kernels
     int chain1_blocks = 0;       // k_chain1 blocks resident at once (0: one block per 8 tiles)
     void* stage = nullptr;       // staging for host outputs
@@ -305,7 +314,6 @@ struct pg_game {
     bool rv_ok = false;           // the four above are complete
     bool no_inc = false;          // there is no memory for Even's lists: no incremental iterations
     pg::IncState* inc = nullptr;  // incremental iterations (pg_inc.cu; single games)
-    int inc_cluster = 0;          // blocks of their cluster (0: not yet asked)
     // ruling-set ranks (pg_deep.cu), for games whose g-forest is deep
     bool deep_mode = false;      // every valuation of the current call takes the ruling-set path
     bool val_deep = false;       // the last valuation took it
@@ -440,6 +448,10 @@ IncState* inc_of(const pg_game* g);  // the state, when the loop's full iteratio
 pg_status build_reverse(pg_game* g, int64_t odd_edges);
 int32_t inc_max_seeds(const pg_game* g);
 pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole);
+// The valuation of a small game, depths included, in one launch (pg_small.cu; the counters are clear).
+pg_status enqueue_val_small(pg_game* g, bool want_dom);
+// The largest cluster of at most want blocks that the device runs for kern (asked once per device: cache).
+int cluster_blocks(const void* kern, int threads, size_t shared, int want, int device, std::atomic<int>* cache);
 // K1 alone (counters cleared, nearest-greater walks and pointer jumping with walk lengths).
 pg_status enqueue_k1(pg_game* g);
 // The valuation through the ruling-set ranks of an Euler tour (pg_deep.cu): cls, depth, key, dom.

@@ -1686,7 +1686,7 @@ pg_status alloc_scratch(pg_game* g) {
     PG_CUDA_TRY(ctx, A((void**)&g->depth, sizeof(int32_t) * n));
     PG_CUDA_TRY(ctx, A((void**)&g->dom, sizeof(int32_t) * n));
     g->ntiles = std::max<int64_t>(1, (n + kCoopTile - 1) / kCoopTile);
-    PG_CUDA_TRY(ctx, A((void**)&g->tiles, sizeof(int64_t) * (2 * g->ntiles + 2)));
+    PG_CUDA_TRY(ctx, A((void**)&g->tiles, sizeof(int64_t) * std::max<int64_t>(2 * g->ntiles + 2, 256)));
     PG_CUDA_TRY(ctx, A((void**)&g->tsum, sizeof(int64_t) * (2 * g->ntiles + 2)));
     PG_CUDA_TRY(ctx, A((void**)&g->gscan, sizeof(int64_t) * 3 * (size_t)g->ngames));
     PG_CUDA_TRY(ctx, A((void**)&g->gst, sizeof(GameState) * (size_t)g->ngames));
@@ -1796,6 +1796,17 @@ pg_status enqueue_valuation(pg_game* g, bool want_dom, bool with_depth) {
     int32_t n = g->n;
     Counters* c = g->cnt;
     const unsigned grid = grid_for(n);
+    // one game whose sink slot is its last id
+    const bool single = g->ngames == 1 && !g->vgame && g->sink0 == n - 1;
+    const bool small = single && n <= kSmallIds && !ctx->timing;
+    if (small) {
+        PG_CUDA_TRY(ctx, cudaMemsetAsync(c, 0, sizeof(Counters), s));
+        pg_status st = enqueue_val_small(g, want_dom);
+        if (st) return st;
+        ctx->launches += 1;
+        g->depth_ok = true;
+        return PG_OK;
+    }
     // K1: walks here are short but for a few, one pass of kWalkCap steps straight into the jumping list
     pg_status st1 = enqueue_k1(g);
     if (st1) return st1;
@@ -1821,11 +1832,10 @@ pg_status enqueue_valuation(pg_game* g, bool want_dom, bool with_depth) {
     prof_begin(g, KID_SINKSCAN);
     {
         int64_t ntiles = g->ntiles;
-        void* args[] = {(void*)&n,        (void*)&g->gd32,   (void*)&g->sz,  (void*)&g->kind,  (void*)&g->hugelist,
-                        (void*)&g->tiles, (void*)&ntiles,    (void*)&g->wgt, (void*)&g->oddsz, (void*)&c};
+        void* args[] = {(void*)&n,        (void*)&g->gd32, (void*)&g->sz,  (void*)&g->kind,  (void*)&g->hugelist,
+                        (void*)&g->tiles, (void*)&ntiles,  (void*)&g->wgt, (void*)&g->oddsz, (void*)&c};
         PG_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((void*)k_idscan_coop, g->coop_blocks, kBlock, args, 0, s));
-        // one game whose sink slot is its last id: the tile scan ranks the sink itself
-        const bool single = g->ngames == 1 && !g->vgame && g->sink0 == n - 1;
+        // (a single game's tile scan ranks the sink itself)
         k_tiles_scan<<<1, kTileScanThreads, 0, s>>>(g->tsum, g->tiles, g->ntiles, single ? g->sink0 : -1, g->gscan,
                                                     g->key, c);
         if (!single) {
@@ -1842,8 +1852,8 @@ pg_status enqueue_valuation(pg_game* g, bool want_dom, bool with_depth) {
         k_chain2<false><<<ilp_grid(n), kBlock, 0, s>>>(n, g->gd32, g->gd, g->kind, g->wgt, g->oddsz, g->key, g->depth,
                                                        c);
     prof_end(g, KID_CHAIN2, 1);
-    PG_CUDA_TRY(ctx, cudaGetLastError());
     g->depth_ok = with_depth;
+    PG_CUDA_TRY(ctx, cudaGetLastError());
     return PG_OK;
 }
 
