@@ -241,6 +241,35 @@ __device__ bool grid_sync(Counters* c) {
     return ok != 0;
 }
 
+// Exclusive scan of one 64-bit value per thread of a 1024-thread block; *total:
+// the block's sum.
+__device__ inline uint64_t block_scan_1024(uint64_t v, uint64_t* total) {
+    __shared__ uint64_t wsum[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint64_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t y = __shfl_up_sync(kFull, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[wid] = x;
+    __syncthreads();
+    if (wid == 0) {
+        uint64_t w = wsum[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint64_t y = __shfl_up_sync(kFull, w, o);
+            if (lane >= o) w += y;
+        }
+        wsum[lane] = w;
+    }
+    __syncthreads();
+    const uint64_t before = (wid ? wsum[wid - 1] : 0) + x - v;
+    *total = wsum[32 - 1];
+    __syncthreads();
+    return before;
+}
+
 // ---------------------------------------------------------------------------
 // Pointer-chasing passes give each thread kIlp vertices, v + 32 j for
 // j < kIlp within a warp tile of 32 kIlp vertices: per-vertex reads and writes

@@ -28,6 +28,7 @@ constexpr int kJumpRoundsDeep = 4096; // extra pointer-jumping rounds allowed on
 constexpr int kHugeChildren = 4096;   // a parent with more children is ranked by an id-ordered scan instead
 constexpr int kCoopTile = 4096;       // elements per tile of the id-ordered scans
 constexpr int kClusterDevices = 64;   // devices whose cluster sizes are remembered
+constexpr int32_t kLoadSmall = 1 << 22;  // a game of up to this many vertices is loaded in one launch (pg_load_small.cu)
 constexpr int32_t kSmallIds = (1 << 18) + 1;  // a game of up to this many ids is valuated by one cluster (pg_small.cu)
 // Count-vector mode (repeated priorities): at most kMaxLevels distinct
 // priorities; a count vector is one signed 128-bit key with one digit per
@@ -365,6 +366,9 @@ pg_status load_game(pg_ctx* ctx, int32_t n, int64_t m, const int32_t* off, const
 pg_status load_union(pg_ctx* ctx, int32_t ngames, const int64_t* vb, const int64_t* eb, const int32_t* off,
                      const int32_t* tgt, const uint8_t* own, const int32_t* pri, int32_t mem_kind, pg_game** out,
                      bool* general);
+// A small game loaded in one launch, without scratch (pg_load_small.cu); *general: load_game's passes must load it.
+pg_status load_small(pg_ctx* ctx, int32_t n, int64_t m, const int32_t* off, const int32_t* tgt, const uint8_t* own,
+                     const int32_t* pri, int32_t mem_kind, pg_game** out, bool* general);
 pg_status alloc_scratch(pg_game* g);
 // Event timing of a call's phases (active when the context's timing is on).
 struct Timer {

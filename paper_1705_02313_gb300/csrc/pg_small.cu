@@ -69,34 +69,6 @@ __device__ inline void small_hot_add(int32_t x, int32_t* tkey, int32_t* tcnt, in
     atomicAdd(sz + x, 1);
 }
 
-// Exclusive scan of one 64-bit value per thread; *total: the block's sum.
-__device__ inline uint64_t small_scan(uint64_t v, uint64_t* total) {
-    __shared__ uint64_t wsum[kSmallThreads / 32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint64_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint64_t y = __shfl_up_sync(kFull, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) wsum[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        uint64_t w = wsum[lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint64_t y = __shfl_up_sync(kFull, w, o);
-            if (lane >= o) w += y;
-        }
-        wsum[lane] = w;
-    }
-    __syncthreads();
-    const uint64_t before = (wid ? wsum[wid - 1] : 0) + x - v;
-    *total = wsum[kSmallThreads / 32 - 1];
-    __syncthreads();
-    return before;
-}
-
 // What id v adds to the packed sums, once sizes and children counts are final.
 __device__ inline uint64_t small_sums(const SmallArgs& a, int32_t v, uint8_t kd) {
     uint64_t s = (uint64_t)__ldcg(a.ccnt + v);
@@ -286,14 +258,14 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_val_small(SmallArgs a) {
     const int32_t lo = min(n, rank * per), hi = min(n, lo + per);
     uint64_t sum = 0, total;
     for (int32_t v = lo + tid; v < hi; v += kSmallThreads) sum += small_sums(a, v, __ldcg(a.kind + v));
-    small_scan(sum, &total);
+    block_scan_1024(sum, &total);
     if (tid == 0) __stcg((unsigned long long*)a.tiles + rank, (unsigned long long)total);
     if (!sync()) return;
     __shared__ uint64_t s_run;
     uint64_t all;
     {
         const uint64_t x = tid < CL ? __ldcg((unsigned long long*)a.tiles + tid) : 0;
-        const uint64_t before = small_scan(x, &all);
+        const uint64_t before = block_scan_1024(x, &all);
         if (tid == rank) s_run = before;
         __syncthreads();
     }
@@ -309,7 +281,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_val_small(SmallArgs a) {
         const int32_t v = b + tid;
         const uint8_t kd = v < hi ? __ldcg(a.kind + v) : 0;
         const uint64_t own = v < hi ? small_sums(a, v, kd) : 0;
-        const uint64_t at = run + small_scan(own, &total);
+        const uint64_t at = run + block_scan_1024(own, &total);
         run += total;
         if (v >= hi) continue;
         __stcg(a.coff + v, (int32_t)(at & kSumMask));
@@ -398,10 +370,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_val_small(SmallArgs a) {
         for (int base = 0; base < k; base += kSmallThreads) {
             const int i = base + tid;
             const int2 e = i < k ? sk[i] : make_int2(0, 0);
-            const uint64_t at = before + small_scan(i < k ? (uint64_t)e.y : 0, &part);
+            const uint64_t at = before + block_scan_1024(i < k ? (uint64_t)e.y : 0, &part);
             before += part;
             if (i < k) a.wgt[e.x >= 0 ? e.x : -e.x - 1] = (int32_t)at + (e.x >= 0 ? 1 : 0);
-            small_scan(i < k && e.x < 0 ? (uint64_t)e.y : 0, &part);
+            block_scan_1024(i < k && e.x < 0 ? (uint64_t)e.y : 0, &part);
             odd_all += part;
         }
         if (tid == 0) a.oddsz[p] = (int32_t)odd_all;
@@ -417,10 +389,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_val_small(SmallArgs a) {
         };
         sum = 0;
         for (int32_t v = lo + tid; v < hi; v += kSmallThreads) sum += size_of(v);
-        small_scan(sum, &total);
+        block_scan_1024(sum, &total);
         if (tid == 0) __stcg((unsigned long long*)a.tiles + rank, (unsigned long long)total);
         if (!sync()) return;
-        const uint64_t bx = small_scan(tid < CL ? __ldcg((unsigned long long*)a.tiles + tid) : 0, &all);
+        const uint64_t bx = block_scan_1024(tid < CL ? __ldcg((unsigned long long*)a.tiles + tid) : 0, &all);
         if (tid == rank) s_run = bx;
         __syncthreads();
         run = s_run;
@@ -428,7 +400,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_val_small(SmallArgs a) {
         for (int32_t b = lo; b < hi; b += kSmallThreads) {
             const int32_t v = b + tid;
             const uint64_t own = v < hi ? size_of(v) : 0;
-            const uint64_t at = run + small_scan(own, &total);
+            const uint64_t at = run + block_scan_1024(own, &total);
             run += total;
             const int32_t se = (int32_t)((own >> kSumBits) & kSumMask), so = (int32_t)(own >> (2 * kSumBits));
             if (se) a.wgt[v] = 1 + podd + (int32_t)((at >> kSumBits) & kSumMask);
