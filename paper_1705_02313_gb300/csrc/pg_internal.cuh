@@ -76,6 +76,8 @@ constexpr uint8_t kKindSinkChild = 2;  // nearest greater ancestor is the sink
 struct Counters {
     int32_t n_pending;   // walks that ran out of steps (length of the pending list)
     int32_t n_walk2;     // walks continued by the second walk pass
+    int32_t leveled;     // the valuation may take pg_level.cuh's bodies
+    int32_t n_roots;     // vertices whose nearest greater vertex is the sink, or who have none (as the walk found them)
     int32_t left[3];     // pending vertices left after a jump round (three rotating counters)
     int32_t n_fin;       // finite vertices
     int32_t n_odd;       // vertices reaching an odd cycle (all games)

@@ -44,6 +44,7 @@
 #include <string.h>
 
 #include "pg_device.cuh"
+#include "pg_level.cuh"
 
 // Vertices per thread of the loop's two chain passes (k_walk_cmp, k_classify).
 #ifndef PG_CHAIN_ILP
@@ -75,8 +76,11 @@ __global__ void __launch_bounds__(kBlock) k_walk(int32_t n, const int32_t* __res
                                                  const int32_t* __restrict__ gsink, int32_t sink0,
                                                  uint64_t* __restrict__ gd, uint32_t* __restrict__ gd32,
                                                  int32_t* __restrict__ more, int32_t* __restrict__ sz,
-                                                 int32_t* __restrict__ oddsz, Counters* cnt, int32_t* more_count) {
+                                                 int32_t* __restrict__ oddsz, Counters* cnt, int32_t* more_count,
+                                                 int leveled) {
     const int lane = threadIdx.x & 31;
+    int32_t roots = 0;
+    if (leveled && blockIdx.x == 0 && threadIdx.x == 0) cnt->leveled = 1;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t tile = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; warp_tile_base(tile) < n;
          tile += nwarps) {
@@ -115,6 +119,7 @@ __global__ void __launch_bounds__(kBlock) k_walk(int32_t n, const int32_t* __res
             if (v[j] < n) {
                 const uint64_t w = slotid[j] ? gd_pack(true, false, 0, v[j], true)  // a sink slot: inert
                                              : walk_word(v[j], x[j], d[j], vgame, gsink, sink0, &pend);
+                roots += gd_resolved(w) && (gd_none(w) || gd_sink(w));
                 gd[v[j]] = w;
                 gd32[v[j]] = g32_of(w);
                 sz[v[j]] = 0;  // zeros for this valuation's size and odd-total accumulation
@@ -124,6 +129,7 @@ __global__ void __launch_bounds__(kBlock) k_walk(int32_t n, const int32_t* __res
             if (pend) more[slot] = v[j];
         }
     }
+    block_add(roots, &cnt->n_roots);
 }
 
 // Pointer jumping over smaller vertices for the walks that ran out of steps,
@@ -136,7 +142,11 @@ __global__ void __launch_bounds__(kBlock) k_walk(int32_t n, const int32_t* __res
 __global__ void __launch_bounds__(kBlock) k_jump_coop(const int32_t* __restrict__ plist, uint64_t* gd,
                                                       uint32_t* gd32, const int32_t* __restrict__ vgame,
                                                       const int32_t* __restrict__ gsink, int32_t sink0, Counters* cnt,
-                                                      int32_t cap, int cap_deep) {
+                                                      int32_t cap, int cap_deep, int32_t n, uint64_t* word,
+                                                      uint64_t* sum) {
+    if (word && lv_applies(cnt, n))
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+            word[i] = sum[i] = 0;
     const int32_t np = cnt->n_pending;
     if (np == 0) return;
     for (int32_t r = 0;; ++r) {
@@ -372,8 +382,12 @@ __global__ void __launch_bounds__(kBlock, 5) k_chain1(int32_t n, const uint32_t*
                                                    uint8_t* __restrict__ kind, uint8_t* __restrict__ cls,
                                                    int32_t* __restrict__ dom, int want_dom,
                                                    const int32_t* __restrict__ vgame, GameState* gst, Counters* cnt,
-                                                   int32_t deep_cut) {
+                                                   int32_t deep_cut, uint64_t* word) {
     if (cnt->err || cnt->deep) return;  // unfinished jumping: g-words may point downwards, no chain walk would end
+    if (lv_applies(cnt, n)) {
+        lv_classify<kIlpChain1>(n, gd32, flags, pri, ccnt, slot, kind, cls, dom, want_dom, word, gst, cnt, deep_cut);
+        return;
+    }
     __shared__ int32_t tkey[kHotSlots], tcnt[kHotSlots];
     for (int i = threadIdx.x; i < kHotSlots; i += blockDim.x) {
         tkey[i] = -1;
@@ -890,8 +904,12 @@ __global__ void __launch_bounds__(kBlock) k_sink_apply(int32_t n, const int32_t*
                                                        const int64_t* __restrict__ tiles,
                                                        const int32_t* __restrict__ vgame,
                                                        const int64_t* __restrict__ gscan, int32_t* __restrict__ wgt,
-                                                       const Counters* cnt) {
+                                                       const Counters* cnt, uint64_t* word) {
     if (cnt->deep) return;
+    if (lv_applies(cnt, n)) {  // (for k_chain2)
+        const int64_t lo = (int64_t)blockIdx.x * kCoopTile;
+        for (int64_t i = lo + threadIdx.x; i < lo + kCoopTile && i < n; i += blockDim.x) word[i] = 0;
+    }
     const int64_t i0 = (int64_t)blockIdx.x * kCoopTile + (int64_t)threadIdx.x * kCIpt;
     int32_t v[kCIpt];
     load8(sinkval, n, i0, v);
@@ -1013,8 +1031,13 @@ __global__ void __launch_bounds__(kBlock) k_chain2(int32_t n, const uint32_t* __
                                                    const uint64_t* __restrict__ gd,
                                                    const uint8_t* __restrict__ kind, const int32_t* __restrict__ wgt,
                                                    const int32_t* __restrict__ oddsz, int32_t* __restrict__ key,
-                                                   int32_t* __restrict__ depth, const Counters* cnt) {
+                                                   int32_t* __restrict__ depth, const Counters* cnt,
+                                                   uint64_t* word) {
     if (cnt->err || cnt->deep) return;  // unfinished jumping or a deep forest: no chain walk
+    if (lv_applies(cnt, n)) {
+        lv_ranks<DEPTH, 2>(n, gd32, gd, kind, wgt, oddsz, key, depth, word);
+        return;
+    }
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t tile = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; warp_tile_base(tile) < n;
@@ -1738,8 +1761,7 @@ pg_status reset_scratch(pg_game* g) {
     g->tune = tune_for(ctx, g->n);
     cudaStream_t s = ctx->stream;
     const int64_t n = g->n;
-    PG_CUDA_TRY(ctx, cudaMemsetAsync(g->sz, 0, sizeof(int32_t) * n, s));
-    PG_CUDA_TRY(ctx, cudaMemsetAsync(g->oddsz, 0, sizeof(int32_t) * n, s));
+    // (the walks of a valuation clear its sizes and odd totals)
     PG_CUDA_TRY(ctx, cudaMemsetAsync(g->ccnt, 0, sizeof(int32_t) * (n + 1), s));
     PG_CUDA_TRY(ctx, cudaMemsetAsync(g->tsum, 0, sizeof(int64_t) * (2 * g->ntiles + 2), s));
     return reset_games(g);
@@ -1750,6 +1772,14 @@ pg_status reset_games(pg_game* g) {
     PG_CUDA_TRY(ctx, cudaMemsetAsync(g->gst, 0, sizeof(GameState) * (size_t)g->ngames, ctx->stream));
     return PG_OK;
 }
+
+// Forests with few roots (pg_level.cuh): the games whose valuations may take its bodies, and the arrays that are free
+// then: the children segments, and two of the four arrays that k_scatter and k_siblings write.
+namespace {
+bool levels_apply(const pg_game* g) { return !g->vgame && g->n > kSmallIds && g->tune.deep_cut < kLvMaxCut; }
+uint64_t* lv_word(const pg_game* g) { return (uint64_t*)g->cl_ks; }
+uint64_t* lv_sum(const pg_game* g) { return (uint64_t*)g->sinkval; }
+}  // namespace
 
 pg_status enqueue_k1(pg_game* g) {
     pg_ctx* ctx = g->ctx;
@@ -1767,7 +1797,8 @@ pg_status enqueue_k1(pg_game* g) {
             default: break;
         }
         walk<<<ilp_grid(n), kBlock, 0, s>>>(n, g->strat, g->flags, g->vgame, g->gsink, g->sink0, g->gd, g->gd32,
-                                            g->plist, g->sz, g->oddsz, c, &c->n_pending);
+                                            g->plist, g->sz, g->oddsz, c, &c->n_pending,
+                                            levels_apply(g) ? 1 : 0);
     }
     prof_end(g, KID_WALK, 1);
     {
@@ -1776,8 +1807,11 @@ pg_status enqueue_k1(pg_game* g) {
         // on the ruling-set path the rounds may run much longer (long increasing runs below pending walks)
         int cap_deep = (ctx->deep_fallback && !g->deep_mode) ? 1 : 0;
         if (g->deep_mode) cap += kJumpRoundsDeep;
+        uint64_t* word = levels_apply(g) ? lv_word(g) : nullptr;
+        uint64_t* sum = lv_sum(g);
         void* args[] = {(void*)&g->plist, (void*)&g->gd,    (void*)&g->gd32, (void*)&g->vgame,
-                        (void*)&g->gsink, (void*)&g->sink0, (void*)&c,       (void*)&cap, (void*)&cap_deep};
+                        (void*)&g->gsink, (void*)&g->sink0, (void*)&c,       (void*)&cap, (void*)&cap_deep,
+                        (void*)&n,        (void*)&word,     (void*)&sum};
         prof_begin(g, KID_JUMP);
         PG_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((void*)k_jump_coop, g->coop_blocks, kBlock, args, 0, s));
         prof_end(g, KID_JUMP, 1);
@@ -1810,14 +1844,16 @@ pg_status enqueue_valuation(pg_game* g, bool want_dom, bool with_depth) {
     // K1: walks here are short but for a few, one pass of kWalkCap steps straight into the jumping list
     pg_status st1 = enqueue_k1(g);
     if (st1) return st1;
+    const bool levels = levels_apply(g);
     prof_begin(g, KID_CHAIN1);
     // one wave of resident blocks for a single game; packed games (batches, servers) keep one block per 8 tiles,
     // which measured faster there (4,096-game batch: 5.95 s of loop against 6.52 s)
     const unsigned c1grid =
         (g->chain1_blocks > 0 && !g->vgame) ? std::min(ilp_grid(n), (unsigned)g->chain1_blocks) : ilp_grid(n);
     k_chain1<<<c1grid, kBlock, 0, s>>>(n, g->gd32, g->flags, g->pri, g->sz, g->ccnt, g->slot, g->kind, g->cls,
-                                       g->dom, want_dom ? 1 : 0, g->vgame, g->gst, c, g->tune.deep_cut);
-    prof_end(g, KID_CHAIN1, 1);
+                                       g->dom, want_dom ? 1 : 0, g->vgame, g->gst, c, g->tune.deep_cut, lv_word(g));
+    if (levels) k_lv_sizes<<<grid, kBlock, 0, s>>>(n, g->gd32, g->kind, g->ccnt, g->sz, lv_sum(g), c);
+    prof_end(g, KID_CHAIN1, levels ? 2 : 1);
     prof_begin(g, KID_CSCAN);
     PG_CUDA_TRY(ctx, exclusive_scan_i32(g->ccnt, g->coff, (int64_t)n + 1, nullptr, g->scan_tmp, g->scan_tmp_bytes, s));
     prof_end(g, KID_CSCAN, 3);
@@ -1842,15 +1878,17 @@ pg_status enqueue_valuation(pg_game* g, bool want_dom, bool with_depth) {
             const unsigned gp = (unsigned)std::max<int64_t>(1, std::min<int64_t>(((int64_t)g->ngames + 7) / 8, 4096));
             k_game_prefix<<<gp, kBlock, 0, s>>>(n, g->ngames, g->gsink, g->sinkval, g->tiles, g->gscan, g->key, c);
         }
-        k_sink_apply<<<(unsigned)g->ntiles, kBlock, 0, s>>>(n, g->sinkval, g->tiles, g->vgame, g->gscan, g->wgt, c);
+        k_sink_apply<<<(unsigned)g->ntiles, kBlock, 0, s>>>(n, g->sinkval, g->tiles, g->vgame, g->gscan, g->wgt, c,
+                                                            lv_word(g));
         prof_end(g, KID_SINKSCAN, single ? 3 : 4);
     }
     prof_begin(g, KID_CHAIN2);
     if (with_depth)
-        k_chain2<true><<<ilp_grid(n), kBlock, 0, s>>>(n, g->gd32, g->gd, g->kind, g->wgt, g->oddsz, g->key, g->depth, c);
+        k_chain2<true><<<ilp_grid(n), kBlock, 0, s>>>(n, g->gd32, g->gd, g->kind, g->wgt, g->oddsz, g->key, g->depth, c,
+                                                      lv_word(g));
     else
         k_chain2<false><<<ilp_grid(n), kBlock, 0, s>>>(n, g->gd32, g->gd, g->kind, g->wgt, g->oddsz, g->key, g->depth,
-                                                       c);
+                                                       c, lv_word(g));
     prof_end(g, KID_CHAIN2, 1);
     g->depth_ok = with_depth;
     PG_CUDA_TRY(ctx, cudaGetLastError());
