@@ -566,6 +566,14 @@ pg_status run_loop_once(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t l
 // rest of this call), so the trajectory is unchanged.
 pg_status run_loop(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t limit) {
     g->depth_ok = false;
+    int div = 1, blocks = 1;
+    if (even && limit <= 0 && !tm.on && g->ctx->graphs && games_apply(g, &div, &blocks)) {
+        bool done = false;
+        pg_status st = run_games(g, cap, div, blocks, &done);
+        if (st) return st;
+        g->last_cmp = g->last_graph = true;
+        if (done) return PG_OK;
+    }
     if (runs_whole(g, tm) || (g->cv && !tm.on && g->ctx->graphs && inc_applies(g))) {
         pg_status st = build_reverse(g, 0);
         if (st == PG_ENOMEM) g->no_inc = true;  // the loop without incremental iterations

@@ -455,7 +455,8 @@ pg_status batch_solve(pg_ctx* ctx, int32_t ngames, const int64_t* vb, const int6
     }
     if (out->dummy_base)
         for (int32_t i = 0; i <= ngames; ++i) out->dummy_base[i] = g->h_dbase[i];
-    out->iterations = g->t_vals;
+    out->iterations = 0;  // (the games' loops need not run in step)
+    for (const GameState& q : gs) out->iterations = std::max<int64_t>(out->iterations, q.inner);
     st = write_outputs(g, out->mem_kind, out->win, out->sigma, out->tau, out->val_class, out->val_depth,
                        out->val_rank, nullptr, out->dummy_sigma);
     if (st) return st;

@@ -50,7 +50,9 @@ constexpr int kIncLevels = 256;      // levels of the closure
 constexpr int kIncRounds = 128;      // rounds of the resolution
 constexpr int kIncWalk = 2048;       // count-vector mode: steps of a play inside A
 constexpr int kIncSteps = 128;       // steps of one resolution round
-constexpr size_t kIncShared = sizeof(int32_t) * (3 * kIncSet + kIncQueue + kIncEven);
+// A block has kIncThreads / div threads and that share of the lists.
+constexpr size_t inc_shared(int div) { return sizeof(int32_t) * (3 * kIncSet + kIncQueue + kIncEven) / div; }
+constexpr size_t kIncShared = inc_shared(1);
 constexpr int32_t kIncBig = 1 << 24;  // (16 blocks' counts sum below 2^31)
 // A full iteration follows a pass that switched more vertices than this. Large
 // games: against 270 us for a full iteration of the 10M random game, an
@@ -66,6 +68,22 @@ constexpr int kIncSeedShareCv = 256, kIncSeedsCv = 16384;
 // takes 17-32 us, an incremental one 13 us (a few switched vertices) to 35 us
 // (a hundred, for the levels of the closure).
 constexpr int kIncWholeShare = 512;
+
+// Packed games (GAMES): a cluster for each game runs the game's whole loop over
+// its range of ids, all games at once. Against the lockstep loop, whose
+// iterations take 50 us at least, as many as the slowest game needs: 608 games
+// of 500 vertices 2.6 -> 0.8 ms, of 2,000 vertices 3.9 -> 2.4; 100 of 9,000
+// (12k ids) 3.9 -> 2.7; 19 and 9 of 20,000 (8 and 16 blocks each) 3.5 -> 2.6 and
+// 3.1 -> 2.1. An SM moves a sector or two per clock and the loop reads its words
+// at random, so this holds while an SM has few ids: 150 games of 12,000 (16k
+// ids) take 5.8 ms against 5.7, 152 of 100,000 44 against 30. The route is taken
+// when every game can run at once with at most kIncBlockIds ids for an SM.
+constexpr int kIncSmallDiv = 4;              // blocks of a quarter of the threads, four to an SM
+constexpr int32_t kIncBlockIds = 12288;      // (a block of 1,024 threads; a quarter for the small ones)
+// A full iteration follows a pass that switched more than this part of a packed
+// game: a 32nd, 64th, 200th: 2.3, 2.5, 2.7 ms (608 games of 2,000), 2.5, 2.3,
+// 2.3 ms (9 games of 20,000).
+constexpr int kIncGameShare = 64;
 
 struct IncArgs {
     int32_t n;       // ids, the sink slot included
@@ -84,7 +102,9 @@ struct IncArgs {
     int32_t* qlist;        // [n] Odd's queue beyond the blocks' own
     GameState* gst;
     Counters* cnt;
-    IncState* st;
+    IncState* st;          // (GAMES: one per game)
+    const int2* games;     // GAMES: first id and index of each cluster's game,
+    const int32_t* gsink;  //    and the games' sinks
     int32_t* gactive;
     int64_t* loop_iters;
     i128* key;   // count-vector mode: the keys, and the levels they count
@@ -213,6 +233,7 @@ __device__ inline i128 inc_key(const IncArgs& a, int32_t v, bool* odd, bool* cut
 
 // Queues the predecessors of la[i] that want it (all of them if changed, else
 // those with a tie mark) for their player.
+template <int DIV>
 __device__ inline void inc_queue(const IncArgs& a, int32_t e0, int32_t nodd, int32_t deg, bool changed, int32_t* lq,
                                  int32_t* c_q, int32_t* le, int32_t* c_e) {
     const int32_t* src = a.rv_src + e0;
@@ -232,11 +253,11 @@ __device__ inline void inc_queue(const IncArgs& a, int32_t e0, int32_t nodd, int
             if (!want[j]) continue;
             if (e + j < nodd) {
                 const int32_t p = atomicAdd(c_q, 1);
-                if (p < kIncQueue) lq[p] = y[j];
+                if (p < kIncQueue / DIV) lq[p] = y[j];
                 else __stcg(a.qlist + atomicAdd(&a.st->n_q, 1), y[j]);
             } else {
                 const int32_t p = atomicAdd(c_e, 1);
-                if (p < kIncEven) le[p] = y[j];
+                if (p < kIncEven / DIV) le[p] = y[j];
             }
         }
     }
@@ -245,17 +266,30 @@ __device__ inline void inc_queue(const IncArgs& a, int32_t e0, int32_t nodd, int
 // CV: count-vector mode (repeated priorities). A valuation is a key summed along
 // the play, so the g-words only tell who is in A, and decisions compare keys
 // (no tie marks); full iterations are not run here. 3M vertices, 4 priorities, load and solve: 30.5 -> 15.0 ms.
-template <bool CV>
-__global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
+template <bool CV, int DIV, bool GAMES>
+__global__ void __launch_bounds__(kIncThreads / DIV, DIV) k_inc(IncArgs a) {
+    constexpr int TH = kIncThreads / DIV, SET = kIncSet / DIV, QUEUE = kIncQueue / DIV, EVEN = kIncEven / DIV;
     cg::cluster_group cl = cg::this_cluster();
     const int32_t CL = (int32_t)cl.num_blocks(), rank = (int32_t)cl.block_rank(), tid = threadIdx.x;
-    const int32_t T = CL * kIncThreads, t0 = rank * kIncThreads + tid;
+    const int32_t T = CL * TH, t0 = rank * TH + tid;
+    int32_t lo0 = 0;  // the first id
+    if constexpr (GAMES) {
+        const int2 game = a.games[blockIdx.x / CL];
+        lo0 = game.x;
+        a.sink0 = a.gsink[game.y];
+        a.n = a.sink0 + 1;
+        a.max_seeds = min(max(1, (a.n - lo0) / kIncGameShare), CL * (SET / 2));
+        a.gst += game.y;
+        a.st += game.y;
+        a.qlist += lo0;
+    }
+    const auto whole = [&] { return GAMES || a.whole; };
     extern __shared__ int32_t dyn[];
     int32_t* la = dyn;             // this block's part of A: vertex,
-    int32_t* ls = la + kIncSet;    //    start of its predecessors,
-    int32_t* lc = ls + kIncSet;    //    their number << 16 | Odd's among them
-    int32_t* lq = lc + kIncSet;    // its part of Odd's queue
-    int32_t* le = lq + kIncQueue;  //    and of Even's
+    int32_t* ls = la + SET;    //    start of its predecessors,
+    int32_t* lc = ls + SET;    //    their number << 16 | Odd's among them
+    int32_t* lq = lc + SET;    // its part of Odd's queue
+    int32_t* le = lq + QUEUE;  //    and of Even's
     __shared__ int2 xb[2][kIncCluster];
     __shared__ int32_t lvl[3], c_bad, c_left, c_q, c_odd, c_s, c_e, c_zero;
     int par = 0;
@@ -280,15 +314,15 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
     gs.phase = __ldcg(&a.gst->phase);
     gs.inner = __ldcg(&a.gst->inner);
     gs.major = __ldcg(&a.gst->major);
-    const bool dead = __ldcg(&a.cnt->err) || __ldcg(&a.cnt->deep) || gs.phase != kPhaseActive;
+    const bool dead = (!GAMES && (__ldcg(&a.cnt->err) || __ldcg(&a.cnt->deep))) || gs.phase != kPhaseActive;
     // every Odd vertex is evaluated (the first iteration, or after an SI-Reset: gactive[1], set by k_bookkeep)
-    bool fresh = a.whole || __ldcg(a.gactive + 1);
-    bool even_full = a.whole || __ldcg(&a.st->even_full);
+    bool fresh = whole() || __ldcg(a.gactive + 1);
+    bool even_full = whole() || __ldcg(&a.st->even_full);
     int32_t ns = fresh ? 0 : __ldcg(&a.cnt->n_list);  // switched vertices, all blocks
     // nothing to do here (the state stays as k_bookkeep left it: a full iteration is next)
-    if (dead || (!a.whole && (fresh || ns > a.max_seeds))) return;
+    if (dead || (!whole() && (fresh || ns > a.max_seeds))) return;
     int32_t nsl = ns > rank ? (ns - rank + CL - 1) / CL : 0;  // this block's, in la
-    for (int32_t i = tid; i < nsl; i += kIncThreads) la[i] = __ldcg(a.alist + rank + i * CL);
+    for (int32_t i = tid; i < nsl; i += TH) la[i] = __ldcg(a.alist + rank + i * CL);
     if (tid == 0) c_e = c_zero = 0;
     int32_t mode = kIncFull;
     int64_t iters = 0;
@@ -296,7 +330,7 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
     cl.sync();
     while (!done) {
         bool all = fresh || ns > a.max_seeds;
-        if (all && !a.whole) break;
+        if (all && !whole()) break;
         if (tid == 0) {
             c_bad = c_left = c_q = c_odd = 0;
             lvl[1] = 0;
@@ -305,7 +339,7 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
         __syncthreads();
         int32_t na = nsl;
         if (!all) {
-            for (int32_t i = tid; i < nsl; i += kIncThreads) {
+            for (int32_t i = tid; i < nsl; i += TH) {
                 const int32_t v = la[i];
                 const int2 r = a.rv[v];
                 const int32_t k = a.rv[v + 1].x - r.x;
@@ -322,7 +356,7 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
             for (int32_t r = 0; !bad && lo < na; ++r) {
                 int32_t* next = &lvl[(r + 1) % 3];
                 if (tid == 0) lvl[(r + 2) % 3] = 0;
-                for (int32_t i = lo + tid; i < na; i += kIncThreads) {
+                for (int32_t i = lo + tid; i < na; i += TH) {
                     const int32_t x = la[i], deg = lc[i] >> 16;
                     const int32_t* src = a.rv_src + ls[i];
                     for (int32_t e = 0; e < deg; e += 4) {
@@ -348,7 +382,7 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
                             if (!in) continue;
                             __stcg(a.gd32 + y[j], kG32Pend | (uint32_t)x);
                             const int32_t p = na + atomicAdd(next, 1), k = r1[j] - r0[j].x;
-                            if (p >= kIncSet || k > kIncFanIn) {
+                            if (p >= SET || k > kIncFanIn) {
                                 atomicOr(next, kIncBig);
                                 continue;
                             }
@@ -366,20 +400,20 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
             }
             if (bad && tid == 0) c_bad = 1;
             all = exchange(&c_bad, &c_zero).x != 0;
-            if (all && !a.whole) break;
+            if (all && !whole()) break;
         }
         if (all) {
             even_full = true;
             if (tid == 0) c_bad = 0;
-            for (int32_t v = t0; v < a.n; v += T)
+            for (int32_t v = lo0 + t0; v < a.n; v += T)
                 __stcg(a.gd32 + v, v == a.sink0 ? kG32Sink : kG32Pend | (uint32_t)__ldcg(a.strat + v));
             cl.sync();
         }
         // ids [i0, i1) in steps of st are this thread's, or la[i] of them
-        const int32_t i0 = all ? t0 : tid, i1 = all ? a.n : na, step = all ? T : kIncThreads;
+        const int32_t i0 = all ? lo0 + t0 : tid, i1 = all ? a.n : na, step = all ? T : TH;
         bool unresolved = false;
         if constexpr (CV) {
-            for (int32_t i = tid; i < na; i += kIncThreads) {
+            for (int32_t i = tid; i < na; i += TH) {
                 const int32_t v = la[i];
                 const i128 old = ld_key(a.key + v);
                 bool odd = false, cut = false;
@@ -393,13 +427,13 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
                 if (k == old) continue;
                 // (a key outside A is never this one: it may change while other plays are walked)
                 st_key(a.key + v, k);
-                inc_queue(a, ls[i], nodd, even_full ? nodd : lc[i] >> 16, true, lq, &c_q, le, &c_e);
+                inc_queue<DIV>(a, ls[i], nodd, even_full ? nodd : lc[i] >> 16, true, lq, &c_q, le, &c_e);
             }
             unresolved = exchange(&c_left, &c_zero).x != 0;
-            for (int32_t i = tid; i < na; i += kIncThreads) __stcg(a.gd32 + la[i], kG32None);  // no longer in A
+            for (int32_t i = tid; i < na; i += TH) __stcg(a.gd32 + la[i], kG32None);  // no longer in A
             if (unresolved) {  // Odd's queue is dropped (Even's: its next pass is full)
-                const int32_t nq = min(c_q, kIncQueue), spill = __ldcg(&a.st->n_q);
-                for (int32_t i = tid; i < nq; i += kIncThreads) a.omark[lq[i]] = 0;
+                const int32_t nq = min(c_q, QUEUE), spill = __ldcg(&a.st->n_q);
+                for (int32_t i = tid; i < nq; i += TH) a.omark[lq[i]] = 0;
                 for (int32_t i = t0; i < spill; i += T) a.omark[__ldcg(a.qlist + i)] = 0;
             }
         } else {
@@ -442,13 +476,13 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
             }
         }
         if (unresolved) {
-            if (!a.whole) break;  // the full iteration decides
+            if (!whole()) break;  // the full iteration decides
             if (!all) {  // over all ids once
                 ns = a.n;
                 __syncthreads();
                 continue;
             }
-            if (t0 == 0) {
+            if (!GAMES && t0 == 0) {  // (a packed game stays active)
                 if (a.deep_fallback) a.cnt->deep = 1;
                 else atomicOr(&a.cnt->err, kErrJumpRounds);
             }
@@ -492,13 +526,13 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
                 const bool changed = tw != old;
                 if (changed) __stcg(a.topw + v, tw);
                 const int32_t nodd = lc[i] & 0xffff;
-                inc_queue(a, ls[i], nodd, even_full ? nodd : lc[i] >> 16, changed, lq, &c_q, le, &c_e);
+                inc_queue<DIV>(a, ls[i], nodd, even_full ? nodd : lc[i] >> 16, changed, lq, &c_q, le, &c_e);
             }
         }
         if (tid == 0) c_s = 0;
         const int2 bad_odd = exchange(&c_bad, &c_odd);
         if (bad_odd.x) {  // the iteration is abandoned
-            if (t0 == 0) a.cnt->deep = 1;
+            if (!GAMES && t0 == 0) a.cnt->deep = 1;
             ++iters;
             break;
         }
@@ -509,27 +543,27 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
             a.omark[v] = tie ? kMarkTie : 0;
             if (!sw) return;
             const int32_t p = atomicAdd(&c_s, 1);
-            if (p < kIncSet) la[p] = v;
+            if (p < SET) la[p] = v;
         };
         if (all) {
-            for (int32_t v = t0; v < a.n; v += T)
+            for (int32_t v = lo0 + t0; v < a.n; v += T)
                 if ((a.flags[v] & (kOwnerOdd | kSinkSlot)) == kOwnerOdd) odd_vertex(v);
         } else {
-            const int32_t nq = min(c_q, kIncQueue), spill = __ldcg(&a.st->n_q);
-            for (int32_t i = tid; i < nq; i += kIncThreads) odd_vertex(lq[i]);
+            const int32_t nq = min(c_q, QUEUE), spill = __ldcg(&a.st->n_q);
+            for (int32_t i = tid; i < nq; i += TH) odd_vertex(lq[i]);
             for (int32_t i = t0; i < spill; i += T) odd_vertex(__ldcg(a.qlist + i));
         }
         // (a block that switched more than it can hold makes the next iteration a full one)
         __syncthreads();
-        if (tid == 0 && c_s > kIncSet) c_s = kIncBig;
-        if (tid == 0) c_bad = c_e > kIncEven;
+        if (tid == 0 && c_s > SET) c_s = kIncBig;
+        if (tid == 0) c_bad = c_e > EVEN;
         const int2 odd_sum = exchange(&c_s, &c_bad);
         ns = odd_sum.x;
         nsl = c_s;
         even_full |= odd_sum.y != 0;
         int32_t nse = 0;
         if (ns == 0 && a.even) {
-            if (!a.whole && (even_full || a.reset)) {  // Even's pass over its view; it counts this iteration
+            if (!whole() && (even_full || a.reset)) {  // Even's pass over its view; it counts this iteration
                 mode = kIncEvenOnly;
                 if (t0 == 0 && bad_odd.y) a.gst->nodd = 1;
                 break;
@@ -540,16 +574,16 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
                 a.emark[v] = tie ? kMarkTie : 0;
                 if (!sw) return;
                 const int32_t p = atomicAdd(&c_s, 1);
-                if (p < kIncSet) la[p] = v;
+                if (p < SET) la[p] = v;
             };
             if (even_full) {
-                for (int32_t v = t0; v < a.n; v += T)
+                for (int32_t v = lo0 + t0; v < a.n; v += T)
                     if (!(a.flags[v] & (kOwnerOdd | kSinkSlot))) even_vertex(v);
             } else {
-                for (int32_t i = tid; i < c_e; i += kIncThreads) even_vertex(le[i]);
+                for (int32_t i = tid; i < c_e; i += TH) even_vertex(le[i]);
             }
             __syncthreads();
-            if (tid == 0 && c_s > kIncSet) c_s = kIncBig;
+            if (tid == 0 && c_s > SET) c_s = kIncBig;
             nse = exchange(&c_s, &c_zero).x;
             nsl = c_s;
             even_full = false;
@@ -567,7 +601,7 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
                 ++gs.major;
                 ns = nse;
                 if (a.reset) {  // Odd restarts from its first edges
-                    for (int32_t v = t0; v < a.n; v += T)
+                    for (int32_t v = lo0 + t0; v < a.n; v += T)
                         if ((a.flags[v] & (kOwnerOdd | kSinkSlot)) == kOwnerOdd) __stcg(a.strat + v, a.tgt[a.off[v]]);
                     fresh = true;
                     cl.sync();
@@ -583,6 +617,7 @@ __global__ void __launch_bounds__(kIncThreads, 1) k_inc(IncArgs a) {
         a.gst->inner = gs.inner;
         a.gst->major = gs.major;
         a.gst->sw_odd = a.gst->sw_even = a.gst->reset = 0;
+        if (GAMES) return;
         a.gactive[0] = gs.phase == kPhaseActive;
         a.st->mode = mode;
         a.st->even_full = even_full;
@@ -685,7 +720,7 @@ static pg_status make_reverse(pg_game* g, int64_t odd_edges) {
     cudaStream_t s = ctx->stream;
     const int32_t n = g->n;
     // packed games take no incremental iterations: their lists hold Odd's edges only (the marks of k_classify)
-    const int odd_only = inc_applies(g) ? 0 : 1;
+    const int odd_only = inc_applies(g) || g->by_game ? 0 : 1;
     const size_t edges = (size_t)(odd_only ? odd_edges : g->m), mark_bytes = ((size_t)n + 16) & ~(size_t)15;
     PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->rv, sizeof(int2) * ((size_t)n + 1), s));
     PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->rv_src, sizeof(int32_t) * std::max<size_t>(edges, 1), s));
@@ -694,7 +729,7 @@ static pg_status make_reverse(pg_game* g, int64_t odd_edges) {
     if (!odd_only) {
         PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->emark, mark_bytes, s));
         PG_CUDA_TRY(ctx, cudaMemsetAsync(g->emark, 0, mark_bytes, s));
-        if (!g->inc) PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->inc, sizeof(IncState), s));
+        if (!g->inc && !g->by_game) PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->inc, sizeof(IncState), s));
     }
     // the valuation's scratch is free before a loop: degrees and cursors in gd, the scan's output in hugelist/coff
     unsigned long long* deg = (unsigned long long*)g->gd;
@@ -732,8 +767,7 @@ int32_t inc_max_seeds(const pg_game* g) {
 
 static std::atomic<int> g_inc_cluster[2][kClusterDevices];
 
-pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole) {
-    pg_ctx* ctx = g->ctx;
+static IncArgs inc_args(const pg_game* g, int64_t cap, bool even) {
     IncArgs a = {};
     a.n = g->n;
     a.sink0 = g->sink0;
@@ -758,31 +792,97 @@ pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole) {
     a.key = g->key128;
     a.lev = g->lev;
     a.cap = cap;
-    a.whole = whole ? 1 : 0;
     a.even = even ? 1 : 0;
     a.reset = even && g->reset_tau ? 1 : 0;
     a.deep_cut = g->tune.deep_cut;
-    a.deep_fallback = ctx->deep_fallback ? 1 : 0;
-    int want = kIncCluster;
-    if (whole)
-        while (want > 1 && (int64_t)want * kIncThreads / 2 >= g->n) want >>= 1;
-    auto kern = g->cv ? k_inc<true> : k_inc<false>;
-    const int c = std::min(want, cluster_blocks((const void*)kern, kIncThreads, kIncShared, kIncCluster, g->device,
-                                                g_inc_cluster[g->cv ? 1 : 0]));
-    a.max_seeds = std::min(whole ? std::max(1, g->n / kIncWholeShare) : inc_max_seeds(g), c * (kIncSet / 2));
+    a.deep_fallback = g->ctx->deep_fallback ? 1 : 0;
+    return a;
+}
+
+static cudaError_t inc_launch(void (*kern)(IncArgs), int clusters, int c, int div, const IncArgs& a, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(c);
-    cfg.blockDim = dim3(kIncThreads);
-    cfg.dynamicSmemBytes = kIncShared;
-    cfg.stream = ctx->stream;
+    cfg.gridDim = dim3((unsigned)clusters * c);
+    cfg.blockDim = dim3(kIncThreads / div);
+    cfg.dynamicSmemBytes = inc_shared(div);
+    cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = c;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    PG_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, kern, a));
+    return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole) {
+    pg_ctx* ctx = g->ctx;
+    IncArgs a = inc_args(g, cap, even);
+    a.whole = whole ? 1 : 0;
+    int want = kIncCluster;
+    if (whole)
+        while (want > 1 && (int64_t)want * kIncThreads / 2 >= g->n) want >>= 1;
+    auto kern = g->cv ? k_inc<true, 1, false> : k_inc<false, 1, false>;
+    const int c = std::min(want, cluster_blocks((const void*)kern, kIncThreads, kIncShared, kIncCluster, g->device,
+                                                g_inc_cluster[g->cv ? 1 : 0]));
+    a.max_seeds = std::min(whole ? std::max(1, g->n / kIncWholeShare) : inc_max_seeds(g), c * (kIncSet / 2));
+    PG_CUDA_TRY(ctx, inc_launch(kern, 1, c, 1, a, ctx->stream));
     ctx->launches += 1;
+    return PG_OK;
+}
+
+static std::atomic<int> g_game_cluster[2][kClusterDevices];
+
+bool games_apply(const pg_game* g, int* div, int* blocks) {
+    const int64_t ng = g->ngames;
+    if (!g->vgame || g->cv || !g->off || g->tune.loop_ranks || g->deep_mode || (int64_t)g->h_base0.size() != ng + 1 ||
+        (int64_t)g->h_dbase.size() != ng + 1)
+        return false;
+    int64_t most = 0;  // ids of the largest game
+    for (int32_t i = 0; i < ng; ++i)
+        most = std::max<int64_t>(most, g->h_base0[i + 1] - g->h_base0[i] + g->h_dbase[i + 1] - g->h_dbase[i] + 1);
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device) != cudaSuccess) return false;
+    *blocks = 0;
+    for (int d : {1, kIncSmallDiv}) {
+        if (ng > (int64_t)sms * d) continue;
+        auto kern = d == 1 ? k_inc<false, 1, true> : k_inc<false, kIncSmallDiv, true>;
+        const int largest = cluster_blocks((const void*)kern, kIncThreads / d, inc_shared(d), kIncCluster, g->device,
+                                           g_game_cluster[d == 1 ? 0 : 1]);
+        int64_t c = 1;  // as many blocks for each game as the device has room for and the game has use for
+        while (2 * c <= largest && 2 * c * ng <= (int64_t)sms * d && c * (kIncThreads / d) < most) c *= 2;
+        if (most > c * (kIncBlockIds / d) || (*blocks && c * *div <= *blocks * (int64_t)d)) continue;
+        *div = d;
+        *blocks = (int)c;
+    }
+    return *blocks > 0;
+}
+
+pg_status run_games(pg_game* g, int64_t cap, int div, int blocks, bool* done) {
+    pg_ctx* ctx = g->ctx;
+    cudaStream_t s = ctx->stream;
+    *done = false;
+    g->by_game = true;
+    g->rv_ok = false;
+    pg_status st = build_reverse(g, 0);
+    g->by_game = false;
+    if (st) return st == PG_ENOMEM ? PG_OK : st;
+    g->rv_ok = false;  // (the lockstep loop keeps Odd's lists only)
+    const int32_t ng = g->ngames;
+    std::vector<int2> games(ng);
+    for (int32_t i = 0; i < ng; ++i) games[i] = make_int2((int32_t)(g->h_base0[i] + g->h_dbase[i] + i), i);
+    int2* list = (int2*)g->slot;  // (scratch that is free during a loop; a game has two ids at least)
+    PG_CUDA_TRY(ctx, cudaMemcpyAsync(list, games.data(), sizeof(int2) * ng, cudaMemcpyHostToDevice, s));
+    IncArgs a = inc_args(g, cap, true);
+    a.st = (IncState*)g->cl_ks;  // (for the queues' lengths)
+    a.gsink = g->gsink;
+    a.games = list;
+    PG_CUDA_TRY(ctx, inc_launch(div == 1 ? k_inc<false, 1, true> : k_inc<false, kIncSmallDiv, true>, ng, blocks, div, a, s));
+    ctx->launches += 1;
+    std::vector<GameState> gs(ng);
+    PG_CUDA_TRY(ctx, cudaMemcpyAsync(gs.data(), g->gst, sizeof(GameState) * ng, cudaMemcpyDeviceToHost, s));
+    PG_CUDA_TRY(ctx, cudaStreamSynchronize(s));
+    *done = true;
+    for (const GameState& x : gs) *done = *done && x.phase != kPhaseActive;
     return PG_OK;
 }
 

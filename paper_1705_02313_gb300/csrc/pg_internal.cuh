@@ -315,6 +315,7 @@ struct pg_game {
     uint8_t* omark = nullptr;
     uint8_t* emark = nullptr;
     bool rv_ok = false;           // the four above are complete
+    bool by_game = false;         // run_games: the lists hold every edge
     bool no_inc = false;          // there is no memory for Even's lists: no incremental iterations
     pg::IncState* inc = nullptr;  // incremental iterations (pg_inc.cu; single games)
     // ruling-set ranks (pg_deep.cu), for games whose g-forest is deep
@@ -450,6 +451,10 @@ pg_status build_player_split(pg_game* g);
 // use (odd_edges: the edges of Odd's vertices, for packed games), one launch of k_inc. whole: the launch is
 // the entire loop; otherwise it follows a full iteration whose passes listed at most inc_max_seeds switches.
 bool inc_applies(const pg_game* g);
+// Packed games that can all run at once run their loops in a cluster per game (pg_inc.cu: blocks of 1,024 / div
+// threads); *done: every game has ended (the lockstep loop takes the rest: deep forests).
+bool games_apply(const pg_game* g, int* div, int* blocks);
+pg_status run_games(pg_game* g, int64_t cap, int div, int blocks, bool* done);
 IncState* inc_of(const pg_game* g);  // the state, when the loop's full iterations prepare incremental ones, or null
 pg_status build_reverse(pg_game* g, int64_t odd_edges);
 int32_t inc_max_seeds(const pg_game* g);
