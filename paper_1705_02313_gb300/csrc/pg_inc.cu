@@ -73,13 +73,13 @@ constexpr int kIncWholeShare = 512;
 // its range of ids, all games at once. Against the lockstep loop, whose
 // iterations take 50 us at least, as many as the slowest game needs: 608 games
 // of 500 vertices 2.6 -> 0.8 ms, of 2,000 vertices 3.9 -> 2.4; 100 of 9,000
-// (12k ids) 3.9 -> 2.7; 19 and 9 of 20,000 (8 and 16 blocks each) 3.5 -> 2.6 and
-// 3.1 -> 2.1. An SM moves a sector or two per clock and the loop reads its words
+// (12k ids) 3.9 -> 2.7; 19 and 9 of 20,000 (several blocks each) 3.5 -> 2.0 and
+// 3.1 -> 1.6. An SM moves a sector or two per clock and the loop reads its words
 // at random, so this holds while an SM has few ids: 150 games of 12,000 (16k
 // ids) take 5.8 ms against 5.7, 152 of 100,000 44 against 30. The route is taken
 // when every game can run at once with at most kIncBlockIds ids for an SM.
 constexpr int kIncSmallDiv = 4;              // blocks of a quarter of the threads, four to an SM
-constexpr int32_t kIncBlockIds = 12288;      // (a block of 1,024 threads; a quarter for the small ones)
+constexpr int32_t kIncBlockIds = 12800;      // (a block of 1,024 threads; a quarter for the small ones)
 // A full iteration follows a pass that switched more than this part of a packed
 // game: a 32nd, 64th, 200th: 2.3, 2.5, 2.7 ms (608 games of 2,000), 2.5, 2.3,
 // 2.3 ms (9 games of 20,000).
@@ -799,20 +799,21 @@ static IncArgs inc_args(const pg_game* g, int64_t cap, bool even) {
     return a;
 }
 
-static cudaError_t inc_launch(void (*kern)(IncArgs), int clusters, int c, int div, const IncArgs& a, cudaStream_t s) {
+struct IncLaunch {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)clusters * c);
-    cfg.blockDim = dim3(kIncThreads / div);
-    cfg.dynamicSmemBytes = inc_shared(div);
-    cfg.stream = s;
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = c;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, a);
-}
+    IncLaunch(int clusters, int c, int div, cudaStream_t s) {
+        cfg.gridDim = dim3((unsigned)clusters * c);
+        cfg.blockDim = dim3(kIncThreads / div);
+        cfg.dynamicSmemBytes = inc_shared(div);
+        cfg.stream = s;
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = c;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+    }
+};
 
 pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole) {
     pg_ctx* ctx = g->ctx;
@@ -825,7 +826,8 @@ pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole) {
     const int c = std::min(want, cluster_blocks((const void*)kern, kIncThreads, kIncShared, kIncCluster, g->device,
                                                 g_inc_cluster[g->cv ? 1 : 0]));
     a.max_seeds = std::min(whole ? std::max(1, g->n / kIncWholeShare) : inc_max_seeds(g), c * (kIncSet / 2));
-    PG_CUDA_TRY(ctx, inc_launch(kern, 1, c, 1, a, ctx->stream));
+    IncLaunch l(1, c, 1, ctx->stream);
+    PG_CUDA_TRY(ctx, cudaLaunchKernelEx(&l.cfg, kern, a));
     ctx->launches += 1;
     return PG_OK;
 }
@@ -848,11 +850,17 @@ bool games_apply(const pg_game* g, int* div, int* blocks) {
         auto kern = d == 1 ? k_inc<false, 1, true> : k_inc<false, kIncSmallDiv, true>;
         const int largest = cluster_blocks((const void*)kern, kIncThreads / d, inc_shared(d), kIncCluster, g->device,
                                            g_game_cluster[d == 1 ? 0 : 1]);
-        int64_t c = 1;  // as many blocks for each game as the device has room for and the game has use for
+        // as many blocks for each game as the device has room for and the game has use for
+        int c = 1;
         while (2 * c <= largest && 2 * c * ng <= (int64_t)sms * d && c * (kIncThreads / d) < most) c *= 2;
-        if (most > c * (kIncBlockIds / d) || (*blocks && c * *div <= *blocks * (int64_t)d)) continue;
+        for (int fit = 0; c > 1; c /= 2) {  // (a cluster's blocks share a part of the device: fewer of them may fit)
+            IncLaunch l((int)ng, c, d, nullptr);
+            if (cudaOccupancyMaxActiveClusters(&fit, kern, &l.cfg) == cudaSuccess && fit >= ng) break;
+            cudaGetLastError();
+        }
+        if (most > (int64_t)c * (kIncBlockIds / d) || (*blocks && c * *div <= *blocks * d)) continue;
         *div = d;
-        *blocks = (int)c;
+        *blocks = c;
     }
     return *blocks > 0;
 }
@@ -876,7 +884,8 @@ pg_status run_games(pg_game* g, int64_t cap, int div, int blocks, bool* done) {
     a.st = (IncState*)g->cl_ks;  // (for the queues' lengths)
     a.gsink = g->gsink;
     a.games = list;
-    PG_CUDA_TRY(ctx, inc_launch(div == 1 ? k_inc<false, 1, true> : k_inc<false, kIncSmallDiv, true>, ng, blocks, div, a, s));
+    IncLaunch l(ng, blocks, div, s);
+    PG_CUDA_TRY(ctx, cudaLaunchKernelEx(&l.cfg, div == 1 ? k_inc<false, 1, true> : k_inc<false, kIncSmallDiv, true>, a));
     ctx->launches += 1;
     std::vector<GameState> gs(ng);
     PG_CUDA_TRY(ctx, cudaMemcpyAsync(gs.data(), g->gst, sizeof(GameState) * ng, cudaMemcpyDeviceToHost, s));
