@@ -97,8 +97,8 @@ void free_game(pg_game* g) {
         cudaGetDevice(&prev) == cudaSuccess && prev != g->device && cudaSetDevice(g->device) == cudaSuccess;
     cudaDeviceSynchronize();
     for (void* p : ptrs)
-        if (p) cudaFreeAsync(p, 0);
-    if (g->hcnt) cudaFreeHost(g->hcnt);
+        if (p && !((char*)p >= g->slab && (char*)p < g->slab + g->slab_bytes)) cudaFreeAsync(p, 0);
+    if (g->slab) cudaFreeAsync(g->slab, 0);
     for (auto& x : g->loop_exec)
         if (x) cudaGraphExecDestroy(x);
     for (auto& e : g->ev)
@@ -642,7 +642,7 @@ pg_status pg_ctx_create(pg_ctx** out, int device) {
     if (cudaSetDevice(device) != cudaSuccess) return PG_ECUDA;
     pg_ctx* c = new pg_ctx();
     c->device = device;
-    if (cudaMallocHost((void**)&c->pinned, 64) != cudaSuccess) {
+    if (cudaMallocHost((void**)&c->pinned, 64 + sizeof(Counters)) != cudaSuccess) {
         delete c;
         return PG_ENOMEM;
     }

@@ -29,6 +29,7 @@ constexpr int kHugeChildren = 4096;   // a parent with more children is ranked b
 constexpr int kCoopTile = 4096;       // elements per tile of the id-ordered scans
 constexpr int kClusterDevices = 64;   // devices whose cluster sizes are remembered
 constexpr int32_t kLoadSmall = 1 << 22;  // a game of up to this many vertices is loaded in one launch (pg_load_small.cu)
+constexpr int32_t kSlabIds = 1 << 20;  // a game of up to this many ids has its scratch in one allocation
 constexpr int32_t kSmallIds = (1 << 18) + 1;  // a game of up to this many ids is valuated by one cluster (pg_small.cu)
 // Count-vector mode (repeated priorities): at most kMaxLevels distinct
 // priorities; a count vector is one signed 128-bit key with one digit per
@@ -275,7 +276,10 @@ struct pg_game {
     int64_t ntiles = 0;
     int64_t* gscan = nullptr;    // [3 * ngames] per game: even and odd prefix at its first id, odd prefix at its sink
     pg::Counters* cnt = nullptr; // device counters
-    pg::Counters* hcnt = nullptr;// pinned host copy
+    pg::Counters* hcnt = nullptr; // host copy (hcnt_copy, or a static valuation's own)
+    pg::Counters hcnt_copy = {};
+    char* slab = nullptr;         // the scratch of a small game (alloc_scratch)
+    size_t slab_bytes = 0;
     void* scan_tmp = nullptr;    // children-count scan scratch
     size_t scan_tmp_bytes = 0;
     // pg_valuate_static: the caller's successors and parities, which the valuation copies and checks first
@@ -374,10 +378,13 @@ pg_status load_small(pg_ctx* ctx, int32_t n, int64_t m, const int32_t* off, cons
                      const int32_t* pri, int32_t mem_kind, pg_game** out, bool* general);
 pg_status alloc_scratch(pg_game* g);
 // Event timing of a call's phases (active when the context's timing is on).
+void make_events(pg_game* g);
+
 struct Timer {
     pg_game* g;
     bool on;
     explicit Timer(pg_game* gg) : g(gg), on(gg->ctx->timing) {
+        if (on) make_events(g);  // (36 events, created when timing is first on)
         g->t_total = g->t_val = g->t_switch = 0;
         g->t_vals = 0;
     }

@@ -1657,6 +1657,13 @@ const char* const kKernelNames[KID_COUNT] = {"walk",     "jump",      "chain1", 
                                               "siblings", "sink_scan", "chain2", "switch_odd", "switch_even",
                                               "classify", "ruling_set"};
 
+void make_events(pg_game* g) {
+    for (auto& e : g->ev)
+        if (!e) cudaEventCreate(&e);
+    for (auto& e : g->kev)
+        if (!e) cudaEventCreate(&e);
+}
+
 void prof_begin(pg_game* g, int id) {
     if (g->ctx->timing) cudaEventRecord(g->kev[2 * id], g->ctx->stream);
 }
@@ -1685,40 +1692,68 @@ void prof_collect(pg_game* g) {
 pg_status alloc_scratch(pg_game* g) {
     pg_ctx* ctx = g->ctx;
     const int64_t n = g->n;
-    auto A = [&](void** p, size_t bytes) { return dev_alloc(ctx, p, bytes, ctx->stream); };
-    PG_CUDA_TRY(ctx, A((void**)&g->gd, sizeof(uint64_t) * n));
-    PG_CUDA_TRY(ctx, A((void**)&g->gd32, sizeof(uint32_t) * n));
-    PG_CUDA_TRY(ctx, A((void**)&g->kind, n));
-    {  // four arrays that only a valuation or a loop uses, in one: afterwards the outputs' records take their place
-        const int64_t n4 = (n + 63) & ~(int64_t)63;
-        PG_CUDA_TRY(ctx, A((void**)&g->quad, 4 * sizeof(int32_t) * n4));
-        g->plist = g->quad;
-        g->slot = g->quad + n4;
-        g->sinkval = g->quad + 2 * n4;
-        g->hugelist = g->quad + 3 * n4;
-        g->rec = (int4*)g->quad;
+    // The arrays of a game of up to kSlabIds ids lie in one allocation: an allocation and its release cost 2 us on the
+    // host, and there are 22 arrays (1k vertices, load and solve: 873 -> 829 us, events and the pinned block included). Larger games take one each, which
+    // the pool serves from whatever it holds in pieces.
+    size_t at = 0;
+    bool place = false;  // the first pass of a slab only counts
+    const bool slab = n <= kSlabIds;
+    auto A = [&](void** p, size_t bytes) {
+        if (!slab) return dev_alloc(ctx, p, bytes, ctx->stream);
+        if (place) *p = g->slab + at;
+        at += (bytes + 255) & ~(size_t)255;
+        return cudaSuccess;
+    };
+    auto arrays = [&]() -> cudaError_t {
+#define PG_A(x)                                  \
+    do {                                         \
+        cudaError_t e_ = (x);                    \
+        if (e_ != cudaSuccess) return e_;        \
+    } while (0)
+        PG_A(A((void**)&g->gd, sizeof(uint64_t) * n));
+        PG_A(A((void**)&g->gd32, sizeof(uint32_t) * n));
+        PG_A(A((void**)&g->kind, n));
+        {  // four arrays that only a valuation or a loop uses, in one: afterwards the outputs' records take their place
+            const int64_t n4 = (n + 63) & ~(int64_t)63;
+            PG_A(A((void**)&g->quad, 4 * sizeof(int32_t) * n4));
+            g->plist = g->quad;
+            g->slot = g->quad + n4;
+            g->sinkval = g->quad + 2 * n4;
+            g->hugelist = g->quad + 3 * n4;
+            g->rec = (int4*)g->quad;
+        }
+        PG_A(A((void**)&g->ccnt, sizeof(int32_t) * (n + 1)));
+        PG_A(A((void**)&g->coff, sizeof(int32_t) * (n + 2)));
+        PG_A(A((void**)&g->cl_ks, sizeof(int2) * n));
+        PG_A(A((void**)&g->sz, sizeof(int32_t) * n));
+        PG_A(A((void**)&g->wgt, sizeof(int32_t) * n));
+        PG_A(A((void**)&g->oddsz, sizeof(int32_t) * n));
+        PG_A(A((void**)&g->key, sizeof(int32_t) * n));
+        PG_A(A((void**)&g->cls, n));
+        PG_A(A((void**)&g->depth, sizeof(int32_t) * n));
+        PG_A(A((void**)&g->dom, sizeof(int32_t) * n));
+        g->ntiles = std::max<int64_t>(1, (n + kCoopTile - 1) / kCoopTile);
+        PG_A(A((void**)&g->tiles, sizeof(int64_t) * std::max<int64_t>(2 * g->ntiles + 2, 256)));
+        PG_A(A((void**)&g->tsum, sizeof(int64_t) * (2 * g->ntiles + 2)));
+        PG_A(A((void**)&g->gscan, sizeof(int64_t) * 3 * (size_t)g->ngames));
+        PG_A(A((void**)&g->gst, sizeof(GameState) * (size_t)g->ngames));
+        PG_A(A((void**)&g->gactive, 2 * sizeof(int32_t)));
+        PG_A(A((void**)&g->loop_iters, 2 * sizeof(int64_t)));
+        PG_A(A((void**)&g->cnt, sizeof(Counters)));
+        g->hcnt = &g->hcnt_copy;
+        g->scan_tmp_bytes = scan_tmp_bytes(n + 2) + 64;
+        PG_A(A(&g->scan_tmp, g->scan_tmp_bytes));
+#undef PG_A
+        return cudaSuccess;
+    };
+    if (slab) {
+        arrays();
+        PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->slab, at, ctx->stream));
+        g->slab_bytes = at;
+        at = 0;
+        place = true;
     }
-    PG_CUDA_TRY(ctx, A((void**)&g->ccnt, sizeof(int32_t) * (n + 1)));
-    PG_CUDA_TRY(ctx, A((void**)&g->coff, sizeof(int32_t) * (n + 2)));
-    PG_CUDA_TRY(ctx, A((void**)&g->cl_ks, sizeof(int2) * n));
-    PG_CUDA_TRY(ctx, A((void**)&g->sz, sizeof(int32_t) * n));
-    PG_CUDA_TRY(ctx, A((void**)&g->wgt, sizeof(int32_t) * n));
-    PG_CUDA_TRY(ctx, A((void**)&g->oddsz, sizeof(int32_t) * n));
-    PG_CUDA_TRY(ctx, A((void**)&g->key, sizeof(int32_t) * n));
-    PG_CUDA_TRY(ctx, A((void**)&g->cls, n));
-    PG_CUDA_TRY(ctx, A((void**)&g->depth, sizeof(int32_t) * n));
-    PG_CUDA_TRY(ctx, A((void**)&g->dom, sizeof(int32_t) * n));
-    g->ntiles = std::max<int64_t>(1, (n + kCoopTile - 1) / kCoopTile);
-    PG_CUDA_TRY(ctx, A((void**)&g->tiles, sizeof(int64_t) * std::max<int64_t>(2 * g->ntiles + 2, 256)));
-    PG_CUDA_TRY(ctx, A((void**)&g->tsum, sizeof(int64_t) * (2 * g->ntiles + 2)));
-    PG_CUDA_TRY(ctx, A((void**)&g->gscan, sizeof(int64_t) * 3 * (size_t)g->ngames));
-    PG_CUDA_TRY(ctx, A((void**)&g->gst, sizeof(GameState) * (size_t)g->ngames));
-    PG_CUDA_TRY(ctx, A((void**)&g->gactive, 2 * sizeof(int32_t)));
-    PG_CUDA_TRY(ctx, A((void**)&g->loop_iters, 2 * sizeof(int64_t)));
-    PG_CUDA_TRY(ctx, A((void**)&g->cnt, sizeof(Counters)));
-    PG_CUDA_TRY(ctx, cudaMallocHost((void**)&g->hcnt, sizeof(Counters)));
-    g->scan_tmp_bytes = scan_tmp_bytes(n + 2) + 64;
-    PG_CUDA_TRY(ctx, A(&g->scan_tmp, g->scan_tmp_bytes));
+    PG_CUDA_TRY(ctx, arrays());
     pg_status st = coop_blocks_for(ctx, &g->coop_blocks);
     if (st) return st;
     st = chain1_blocks_for(ctx, &g->chain1_blocks);
@@ -1727,12 +1762,16 @@ pg_status alloc_scratch(pg_game* g) {
         pg_status st2 = alloc_cv(g);
         if (st2) return st2;
     }
-    for (int i = 0; i < 4; ++i) PG_CUDA_TRY(ctx, cudaEventCreate(&g->ev[i]));
-    for (int i = 0; i < 2 * KID_COUNT; ++i) PG_CUDA_TRY(ctx, cudaEventCreate(&g->kev[i]));
+    if (ctx->timing) make_events(g);
     return reset_scratch(g);
 }
 
+// (both depend on the device alone, asked once: 4 us of a load)
+static std::atomic<int> g_coop_blocks[kClusterDevices], g_chain1_blocks[kClusterDevices];
+
 pg_status coop_blocks_for(pg_ctx* ctx, int* out) {
+    const bool cached = ctx->device >= 0 && ctx->device < kClusterDevices;
+    if (cached && (*out = g_coop_blocks[ctx->device].load())) return PG_OK;
     int sms = 0, a = 0, b = 0;
     PG_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
     PG_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_jump_coop, kBlock, 0));
@@ -1740,6 +1779,7 @@ pg_status coop_blocks_for(pg_ctx* ctx, int* out) {
     int c = 0;
     PG_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, k_jump32_coop, kBlock, 0));
     *out = sms * std::max(1, std::min(std::min(std::min(a, b), c), 4));
+    if (cached) g_coop_blocks[ctx->device].store(*out);
     return PG_OK;
 }
 
@@ -1747,10 +1787,13 @@ pg_status coop_blocks_for(pg_ctx* ctx, int* out) {
 // tiles: the walks' lengths vary, and a warp with many tiles averages them out,
 // where one tile per warp would hold each block until its longest walk ends.
 pg_status chain1_blocks_for(pg_ctx* ctx, int* out) {
+    const bool cached = ctx->device >= 0 && ctx->device < kClusterDevices;
+    if (cached && (*out = g_chain1_blocks[ctx->device].load())) return PG_OK;
     int sms = 0, a = 0;
     PG_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
     PG_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_chain1, kBlock, 0));
     *out = sms * std::max(1, a);
+    if (cached) g_chain1_blocks[ctx->device].store(*out);
     return PG_OK;
 }
 
@@ -2144,8 +2187,11 @@ pg_status build_player_split(pg_game* g) {
 pg_status sync_counters(pg_game* g) {
     pg_ctx* ctx = g->ctx;
     cudaStream_t s = ctx->stream;
-    PG_CUDA_TRY(ctx, cudaMemcpyAsync(g->hcnt, g->cnt, sizeof(Counters), cudaMemcpyDeviceToHost, s));
+    // (a static valuation's context has no pinned block)
+    Counters* to = ctx->pinned ? (Counters*)(ctx->pinned + 16) : g->hcnt;
+    PG_CUDA_TRY(ctx, cudaMemcpyAsync(to, g->cnt, sizeof(Counters), cudaMemcpyDeviceToHost, s));
     PG_CUDA_TRY(ctx, cudaStreamSynchronize(s));
+    if (to != g->hcnt) *g->hcnt = *to;
     prof_collect(g);
     if (g->hcnt->err & kErrBarrier) return fail(ctx, PG_ECUDA, "valuation: a grid barrier timed out");
     if (g->hcnt->err & kErrJumpRounds) return fail(ctx, PG_ECUDA, "valuation: pointer jumping did not converge");
