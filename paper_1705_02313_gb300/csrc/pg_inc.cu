@@ -1,4 +1,4 @@
-// Incremental iterations of the compare-mode loop, for one game.
+// Incremental iterations of the compare-mode loop: for one game, and for all games of a small batch at once.
 //
 // After a switching pass only vertices whose play passes a switched vertex
 // can change their valuation (Section 3: a valuation is a function of the
@@ -633,6 +633,12 @@ __global__ void __launch_bounds__(kIncThreads / DIV, DIV) k_inc(IncArgs a) {
 // counters and lists), count and fill: one pass 196 + 887 us, ranges of 16 MB
 // 329 + 739, 32 MB 205 + 407, 48 MB 151 + 337, 64 MB 197 + 371.
 constexpr size_t kRvBytes = 48 << 20;
+// Every pass reads all edges, while one pass moves a sector per edge each way:
+// random games of 20M and 40M vertices (11 and 21 ranges), load and solve, 44.6
+// and 117.0 ms in ranges, 47.0 and 118.2 in one pass; more ranges are not worth
+// it. Packed games' targets are near their sources and take one pass (4,096 games,
+// 590M vertices: loop 1,789 ms with 64 ranges, 1,364 in one pass).
+constexpr size_t kRvPasses = 24;
 
 // In-degree of every id: all edges in the low half, Odd's in the high half.
 template <typename OffT>
@@ -736,7 +742,8 @@ static pg_status make_reverse(pg_game* g, int64_t odd_edges) {
     const unsigned grid = grid_for(n);
     PG_CUDA_TRY(ctx, cudaMemsetAsync(deg, 0, sizeof(uint64_t) * (size_t)n, s));
     auto ranges = [&](size_t bytes, auto&& pass) {
-        const int32_t np = (int32_t)std::max<size_t>(1, std::min<size_t>(64, (bytes + kRvBytes / 2) / kRvBytes));
+        const size_t want = (bytes + kRvBytes / 2) / kRvBytes;
+        const int32_t np = g->vgame || want > kRvPasses || want < 1 ? 1 : (int32_t)want;
         for (int32_t i = 0; i < np; ++i)
             pass((int32_t)((int64_t)n * i / np), (int32_t)((int64_t)n * (i + 1) / np));
         ctx->launches += np;
