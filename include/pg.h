@@ -236,7 +236,7 @@ typedef struct {
     int64_t *inner;        /* host, ngames */
     int32_t *status;       /* host, ngames */
     int64_t *dummy_base;   /* host, ngames + 1, out */
-    int64_t iterations;    /* out: lockstep iterations run for the whole batch */
+    int64_t iterations;    /* out: iterations of the game that took the most */
     double load_ms, pack_ms, loop_ms; /* out: wall time loading the games, packing them, and in the loop */
 } pg_result_batch;
 
@@ -250,7 +250,7 @@ typedef struct {
  * vtx_base and edge_base are host arrays of ngames + 1 entries starting at 0;
  * the other inputs use mem_kind. Each game is validated and preprocessed as in
  * pg_load_csr (same errors); the batch may hold up to 2^30 vertices after
- * preprocessing and any number of edges. max_inner caps the lockstep
+ * preprocessing and any number of edges. max_inner caps each game's
  * iterations (0 = 64 * (largest game + 64)). Returns PG_ETIMEOUT or
  * PG_ENOTADMISSIBLE if any game ended that way (results are still written). */
 pg_status pg_solve_batch(pg_ctx *ctx, int32_t ngames, const int64_t *vtx_base, const int64_t *edge_base,

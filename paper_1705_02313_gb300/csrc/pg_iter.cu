@@ -25,7 +25,8 @@
 // Passes of one valuation (no host synchronisation between them):
 //   k_walk        nearest greater vertex by a direct walk of <= kWalkCap steps
 //   k_jump_coop   pointer jumping over smaller vertices for the rest
-//   k_chain1      classification, g-subtree sizes and children counts
+//   k_chain1      classification, g-subtree sizes and children counts (k_lv_sizes: the sizes of a forest with few
+//                 roots, whose walks pg_level.cuh shortens)
 //   scan          children counts -> contiguous child segments
 //   k_scatter     children into their segments; the sink's children marked
 //   k_siblings    sibling weights inside each segment (k_big_parents for
@@ -1693,8 +1694,8 @@ pg_status alloc_scratch(pg_game* g) {
     pg_ctx* ctx = g->ctx;
     const int64_t n = g->n;
     // The arrays of a game of up to kSlabIds ids lie in one allocation: an allocation and its release cost 2 us on the
-    // host, and there are 22 arrays (1k vertices, load and solve: 873 -> 829 us, events and the pinned block included). Larger games take one each, which
-    // the pool serves from whatever it holds in pieces.
+    // host, and there are 22 arrays (1k vertices, load and solve: 873 -> 829 us, with the events and the pinned block
+    // that a game no longer has). Larger games take one each, which the pool serves from whatever it holds in pieces.
     size_t at = 0;
     bool place = false;  // the first pass of a slab only counts
     const bool slab = n <= kSlabIds;
