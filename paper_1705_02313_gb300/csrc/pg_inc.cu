@@ -46,9 +46,8 @@ constexpr int kIncSet = 10240;       // vertices of A a block holds
 constexpr int kIncQueue = 8192;      // Odd's queue of a block (the rest spills to global memory)
 constexpr int kIncEven = 16384;      // Even's queue of a block (beyond it Even's next pass is full)
 constexpr int kIncFanIn = 1024;      // a vertex of A with more predecessors ends the incremental iteration
-constexpr int kIncLevels = 256;      // levels of the closure
 constexpr int kIncRounds = 128;      // rounds of the resolution
-constexpr int kIncWalk = 2048;       // count-vector mode: steps of a play inside A
+constexpr int kIncWalk = 256;        // count-vector mode: steps of a play inside A
 constexpr int kIncSteps = 128;       // steps of one resolution round
 // A block has kIncThreads / div threads and that share of the lists.
 constexpr size_t inc_shared(int div) { return sizeof(int32_t) * (3 * kIncSet + kIncQueue + kIncEven) / div; }
@@ -85,6 +84,21 @@ constexpr int32_t kIncBlockIds = 12800;      // (a block of 1,024 threads; a qua
 // 2.3 ms (9 games of 20,000).
 constexpr int kIncGameShare = 64;
 
+// A closure that takes too long is abandoned, and a full iteration follows. The
+// budget counts vertices that a block has found (45 ns each) and levels, which
+// take as long as 44 of them (2 us). It is about one and a half full iterations
+// of a game whose plays are short: these take 45 us and 17 us per million ids,
+// 45 and 62 with keys; over all ids in one launch 16 us and 1 us per 128 ids of a
+// block. Where plays are long (a torus, a ring with chords) half of the attempts
+// went on to 256 levels, or to as many vertices as a block holds, 260 us (200k
+// vertices) to 600 us (4M), for nothing. Solving a torus of 4M vertices by full
+// iterations, by these attempts, and with the budget and the waits: 1,332, 2,254
+// and 1,320 ms; a ring of 4M 5,321, 8,735 and 5,490; a torus of 200k 180, 185 and
+// 158; a random game of 1M 6.7, 5.1 and 5.1.
+constexpr int32_t kIncLevelCost = 44;
+// An abandoned attempt is followed by 1 full iteration; by 2, 4, ... 32 while they keep failing.
+constexpr int32_t kIncFails = 5;
+
 struct IncArgs {
     int32_t n;       // ids, the sink slot included
     int32_t sink0;
@@ -102,7 +116,8 @@ struct IncArgs {
     int32_t* qlist;        // [n] Odd's queue beyond the blocks' own
     GameState* gst;
     Counters* cnt;
-    IncState* st;          // (GAMES: one per game)
+    IncState* st;
+    int32_t* n_q;          // its length (GAMES: one per game)
     const int2* games;     // GAMES: first id and index of each cluster's game,
     const int32_t* gsink;  //    and the games' sinks
     int32_t* gactive;
@@ -111,12 +126,18 @@ struct IncArgs {
     Levels lev;
     int64_t cap;
     int32_t max_seeds;  // more switched vertices than this take a full iteration
+    int32_t budget;     // of a block's closure (kIncLevelCost)
     int32_t whole;      // 1: the launch runs the whole loop, full iterations included (over all ids)
     int32_t even;       // 0: best response (the inner loop only)
     int32_t reset;      // SI-Reset
     int32_t deep_cut;
     int32_t deep_fallback;
 };
+
+// (a launch that runs the whole loop, by its ids and blocks; inc_budget: a launch after a full iteration)
+__host__ __device__ inline int32_t inc_budget_whole(int32_t ids, int32_t blocks) {
+    return kIncLevelCost * (16 + ids / (128 * blocks));
+}
 
 // Sets bit b of byte p (in a 4-byte aligned array); returns whether it was clear.
 __device__ inline bool claim_byte(uint8_t* base, int32_t i, uint32_t b) {
@@ -254,7 +275,7 @@ __device__ inline void inc_queue(const IncArgs& a, int32_t e0, int32_t nodd, int
             if (e + j < nodd) {
                 const int32_t p = atomicAdd(c_q, 1);
                 if (p < kIncQueue / DIV) lq[p] = y[j];
-                else __stcg(a.qlist + atomicAdd(&a.st->n_q, 1), y[j]);
+                else __stcg(a.qlist + atomicAdd(a.n_q, 1), y[j]);
             } else {
                 const int32_t p = atomicAdd(c_e, 1);
                 if (p < kIncEven / DIV) le[p] = y[j];
@@ -279,8 +300,9 @@ __global__ void __launch_bounds__(kIncThreads / DIV, DIV) k_inc(IncArgs a) {
         a.sink0 = a.gsink[game.y];
         a.n = a.sink0 + 1;
         a.max_seeds = min(max(1, (a.n - lo0) / kIncGameShare), CL * (SET / 2));
+        a.budget = inc_budget_whole(a.n - lo0, CL);
         a.gst += game.y;
-        a.st += game.y;
+        a.n_q += game.y;
         a.qlist += lo0;
     }
     const auto whole = [&] { return GAMES || a.whole; };
@@ -292,6 +314,8 @@ __global__ void __launch_bounds__(kIncThreads / DIV, DIV) k_inc(IncArgs a) {
     int32_t* le = lq + QUEUE;  //    and of Even's
     __shared__ int2 xb[2][kIncCluster];
     __shared__ int32_t lvl[3], c_bad, c_left, c_q, c_odd, c_s, c_e, c_zero;
+    // incremental iterations: none for the next p_wait iterations, p_fails abandoned in a row, p_since done since
+    __shared__ int32_t p_wait, p_fails, p_since;
     int par = 0;
     // The sums over the cluster of two counts, final in each block when all its threads call: every block stores
     // its pair in every block's shared memory and sums after the barrier. Two buffers in turn: a block that is
@@ -320,22 +344,31 @@ __global__ void __launch_bounds__(kIncThreads / DIV, DIV) k_inc(IncArgs a) {
     bool even_full = whole() || __ldcg(&a.st->even_full);
     int32_t ns = fresh ? 0 : __ldcg(&a.cnt->n_list);  // switched vertices, all blocks
     // nothing to do here (the state stays as k_bookkeep left it: a full iteration is next)
-    if (dead || (!whole() && (fresh || ns > a.max_seeds))) return;
+    if (dead || (!whole() && (fresh || ns > a.max_seeds || __ldcg(&a.st->wait) > 0))) return;
     int32_t nsl = ns > rank ? (ns - rank + CL - 1) / CL : 0;  // this block's, in la
     for (int32_t i = tid; i < nsl; i += TH) la[i] = __ldcg(a.alist + rank + i * CL);
-    if (tid == 0) c_e = c_zero = 0;
-    int32_t mode = kIncFull;
-    int64_t iters = 0;
+    if (tid == 0) {
+        c_e = c_zero = p_wait = p_since = 0;
+        p_fails = whole() ? 0 : __ldcg(&a.st->fails);
+    }
+    int32_t mode = kIncFull, iters = 0;
     bool done = false;
+    auto abandoned = [&] {  // (by one thread of each block, where a barrier follows)
+        if (p_since > 1) p_fails = 0;
+        p_wait = 1 << p_fails;
+        p_fails = min(p_fails + 1, kIncFails);
+        p_since = 0;
+    };
     cl.sync();
     while (!done) {
         bool all = fresh || ns > a.max_seeds;
         if (all && !whole()) break;
+        all |= p_wait > 0;
         if (tid == 0) {
             c_bad = c_left = c_q = c_odd = 0;
             lvl[1] = 0;
         }
-        if (t0 == 0) a.st->n_q = 0;
+        if (t0 == 0) *a.n_q = 0;
         __syncthreads();
         int32_t na = nsl;
         if (!all) {
@@ -350,7 +383,7 @@ __global__ void __launch_bounds__(kIncThreads / DIV, DIV) k_inc(IncArgs a) {
             }
             cl.sync();
             // level r expands la[lo .. na) into la[na ..]; lvl[] rotates, so a count is stable while it is read. A
-            // level that cannot be held (kIncBig) ends the closure.
+            // level that cannot be held (kIncBig) or that passes the budget ends the closure.
             bool bad = c_bad != 0;
             int32_t lo = 0;
             for (int32_t r = 0; !bad && lo < na; ++r) {
@@ -394,12 +427,13 @@ __global__ void __launch_bounds__(kIncThreads / DIV, DIV) k_inc(IncArgs a) {
                 }
                 __syncthreads();
                 const int32_t found = *next;
-                bad = found >= kIncBig || r + 1 >= kIncLevels;
+                bad = found >= kIncBig || (r + 1) * kIncLevelCost + na + found > a.budget;
                 lo = na;
                 if (!bad) na += found;
             }
             if (bad && tid == 0) c_bad = 1;
             all = exchange(&c_bad, &c_zero).x != 0;
+            if (all && tid == 0) abandoned();
             if (all && !whole()) break;
         }
         if (all) {
@@ -432,7 +466,7 @@ __global__ void __launch_bounds__(kIncThreads / DIV, DIV) k_inc(IncArgs a) {
             unresolved = exchange(&c_left, &c_zero).x != 0;
             for (int32_t i = tid; i < na; i += TH) __stcg(a.gd32 + la[i], kG32None);  // no longer in A
             if (unresolved) {  // Odd's queue is dropped (Even's: its next pass is full)
-                const int32_t nq = min(c_q, QUEUE), spill = __ldcg(&a.st->n_q);
+                const int32_t nq = min(c_q, QUEUE), spill = __ldcg(a.n_q);
                 for (int32_t i = tid; i < nq; i += TH) a.omark[lq[i]] = 0;
                 for (int32_t i = t0; i < spill; i += T) a.omark[__ldcg(a.qlist + i)] = 0;
             }
@@ -476,6 +510,7 @@ __global__ void __launch_bounds__(kIncThreads / DIV, DIV) k_inc(IncArgs a) {
             }
         }
         if (unresolved) {
+            if (!all && tid == 0) abandoned();
             if (!whole()) break;  // the full iteration decides
             if (!all) {  // over all ids once
                 ns = a.n;
@@ -529,7 +564,11 @@ __global__ void __launch_bounds__(kIncThreads / DIV, DIV) k_inc(IncArgs a) {
                 inc_queue<DIV>(a, ls[i], nodd, even_full ? nodd : lc[i] >> 16, changed, lq, &c_q, le, &c_e);
             }
         }
-        if (tid == 0) c_s = 0;
+        if (tid == 0) {
+            c_s = 0;
+            if (all) p_wait -= p_wait > 0;
+            else ++p_since;
+        }
         const int2 bad_odd = exchange(&c_bad, &c_odd);
         if (bad_odd.x) {  // the iteration is abandoned
             if (!GAMES && t0 == 0) a.cnt->deep = 1;
@@ -549,7 +588,7 @@ __global__ void __launch_bounds__(kIncThreads / DIV, DIV) k_inc(IncArgs a) {
             for (int32_t v = lo0 + t0; v < a.n; v += T)
                 if ((a.flags[v] & (kOwnerOdd | kSinkSlot)) == kOwnerOdd) odd_vertex(v);
         } else {
-            const int32_t nq = min(c_q, QUEUE), spill = __ldcg(&a.st->n_q);
+            const int32_t nq = min(c_q, QUEUE), spill = __ldcg(a.n_q);
             for (int32_t i = tid; i < nq; i += TH) odd_vertex(lq[i]);
             for (int32_t i = t0; i < spill; i += T) odd_vertex(__ldcg(a.qlist + i));
         }
@@ -621,6 +660,8 @@ __global__ void __launch_bounds__(kIncThreads / DIV, DIV) k_inc(IncArgs a) {
         a.gactive[0] = gs.phase == kPhaseActive;
         a.st->mode = mode;
         a.st->even_full = even_full;
+        a.st->wait = p_wait;
+        a.st->fails = p_since > 1 ? 0 : p_fails;
         *a.loop_iters += iters;
     }
 }
@@ -767,6 +808,10 @@ static pg_status make_reverse(pg_game* g, int64_t odd_edges) {
     return PG_OK;
 }
 
+static int32_t inc_budget(const pg_game* g) {
+    return kIncLevelCost * (33 + (int32_t)((int64_t)g->n * (g->cv ? 31 : 14) / 1000000));
+}
+
 int32_t inc_max_seeds(const pg_game* g) {
     return g->cv ? std::max(1, std::min(g->n / kIncSeedShareCv, kIncSeedsCv))
                  : std::max(1, std::min(g->n / kIncSeedShare, kIncSeeds));
@@ -794,6 +839,7 @@ static IncArgs inc_args(const pg_game* g, int64_t cap, bool even) {
     a.gst = g->gst;
     a.cnt = g->cnt;
     a.st = g->inc;
+    a.n_q = g->inc ? &g->inc->n_q : nullptr;
     a.gactive = g->gactive;
     a.loop_iters = g->loop_iters;
     a.key = g->key128;
@@ -833,6 +879,7 @@ pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole) {
     const int c = std::min(want, cluster_blocks((const void*)kern, kIncThreads, kIncShared, kIncCluster, g->device,
                                                 g_inc_cluster[g->cv ? 1 : 0]));
     a.max_seeds = std::min(whole ? std::max(1, g->n / kIncWholeShare) : inc_max_seeds(g), c * (kIncSet / 2));
+    a.budget = whole ? inc_budget_whole(g->n, c) : inc_budget(g);
     IncLaunch l(1, c, 1, ctx->stream);
     PG_CUDA_TRY(ctx, cudaLaunchKernelEx(&l.cfg, kern, a));
     ctx->launches += 1;
@@ -888,7 +935,7 @@ pg_status run_games(pg_game* g, int64_t cap, int div, int blocks, bool* done) {
     int2* list = (int2*)g->slot;  // (scratch that is free during a loop; a game has two ids at least)
     PG_CUDA_TRY(ctx, cudaMemcpyAsync(list, games.data(), sizeof(int2) * ng, cudaMemcpyHostToDevice, s));
     IncArgs a = inc_args(g, cap, true);
-    a.st = (IncState*)g->cl_ks;  // (for the queues' lengths)
+    a.n_q = (int32_t*)g->cl_ks;
     a.gsink = g->gsink;
     a.games = list;
     IncLaunch l(ng, blocks, div, s);

@@ -106,6 +106,8 @@ struct IncState {
     int32_t mode;       // what the loop's next full body is for (kIncFull, kIncEvenOnly)
     int32_t even_full;  // the next Even pass evaluates every Even vertex
     int32_t n_q;        // k_inc: Odd's queue beyond the blocks' own
+    int32_t wait;       // full iterations before the next incremental one is tried, and
+    int32_t fails;      //    attempts abandoned in a row
 };
 // Games of up to this many ids run their whole loop in one launch of k_inc (41k ids: 17-32 us for an iteration
 // over all ids, against 45 us for the passes of a full iteration as graph nodes; they grow with the ids, and

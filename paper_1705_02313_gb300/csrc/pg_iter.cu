@@ -1202,10 +1202,12 @@ __global__ void k_bookkeep(int32_t ngames, GameState* gst, int64_t cap, int even
     int32_t act = 0;
     for (int32_t gi = blockIdx.x * blockDim.x + threadIdx.x; gi < ngames; gi += gridDim.x * blockDim.x) {
         GameState st = gst[gi];
+        const int32_t wait = inc ? inc->wait : 0;
         st.reset = 0;
         if (inc) {  // one game: Even's marks are exact after an Even pass, and not kept by a full iteration
             inc->mode = kIncFull;
             inc->even_full = !(even_phase && st.sw_odd == 0);
+            inc->wait = max(wait - 1, 0);
         }
         if (st.phase == kPhaseActive) {
             st.inner += 1;
