@@ -501,7 +501,7 @@ bool runs_whole(const pg_game* g, const Timer& tm) {
 // device and a later call continues them).
 pg_status run_loop_once(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t limit, int64_t* ran) {
     pg_ctx* ctx = g->ctx;
-    g->last_graph = false;
+    g->last_graph = g->last_stale = false;
     *ran = 0;
     const bool cmp = loop_compares(g);
     const int64_t hard = limit > 0 ? std::min<int64_t>(limit, cap + 2) : cap + 2;
@@ -526,7 +526,13 @@ pg_status run_loop_once(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t l
         PG_CUDA_TRY(ctx, cudaGraphLaunch(g->loop_exec[w], s));
         int64_t* it = (int64_t*)ctx->pinned;
         PG_CUDA_TRY(ctx, cudaMemcpyAsync(it, g->loop_iters, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+        IncState* inc = (IncState*)(it + 2);
+        inc->stale = 0;
+        static_assert(2 * sizeof(int64_t) + sizeof(IncState) <= 64, "pinned holds both before the counters");
+        if (g->cv && inc_of(g))
+            PG_CUDA_TRY(ctx, cudaMemcpyAsync(inc, g->inc, sizeof(IncState), cudaMemcpyDeviceToHost, s));
         pg_status st = sync_counters(g);
+        g->last_stale = inc->stale != 0;
         const int64_t iters = it[0], bodies = it[1];
         *ran = iters;
         g->t_vals += iters;
@@ -592,7 +598,7 @@ pg_status run_loop(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t limit)
         pg_status st = run_loop_once(g, cap, even, tm, limit > 0 ? limit - done : 0, &ran);
         if (st) return st;
         // (k_inc keeps the keys of a count-vector game, not its classes and walk lengths)
-        g->last_cmp = loop_compares(g) || (g->cv && g->last_graph && inc_of(g));
+        g->last_cmp = loop_compares(g) || g->last_stale;
         if (g->cv || g->deep_mode || !g->hcnt->deep) return PG_OK;
         g->deep_mode = true;
         st = prepare_deep(g);
@@ -874,11 +880,8 @@ pg_status pg_solve(pg_game* g, const pg_solve_opts* opts, pg_result* out) {
     if (gs.phase == kPhaseOddCycle)
         return fail(ctx, PG_ENOTADMISSIBLE, "pg_solve: an odd cycle was reached: sigma is not admissible");
     const bool timed_out = gs.phase == kPhaseTimeout;
-    if (timed_out || g->last_cmp) {
-        st = full_valuation(g, false);  // the full valuation of the profile being returned
-        if (st) return st;
-        g->last_cmp = false;
-    }
+    st = finish_loop(g, timed_out, out->val_depth != nullptr);  // the valuation of the profile being returned
+    if (st) return st;
     tm.mark(2);
     g->t_total = tm.since(3, 2);
     out->major = gs.major;
@@ -910,7 +913,7 @@ pg_status pg_best_response(pg_game* g, const int32_t* sigma, const int8_t* dummy
     if (gs.phase == kPhaseOddCycle)
         return fail(ctx, PG_ENOTADMISSIBLE, "an odd cycle was reached: sigma is not admissible");
     const bool timed_out = gs.phase == kPhaseTimeout;
-    st = finish_loop(g);  // ranks of the best response's valuation
+    st = finish_loop(g, false, out && out->val_depth);  // ranks of the best response's valuation
     if (st) return st;
     tm.mark(2);
     g->t_total = tm.since(3, 2);

@@ -420,6 +420,18 @@ __global__ void __launch_bounds__(kBlock) k_chain_cv(int32_t n, const uint32_t* 
     block_add32(nodd, &cnt->n_odd);
 }
 
+__global__ void __launch_bounds__(kBlock) k_class_cv(int32_t n, const i128* __restrict__ key,
+                                                     const uint8_t* __restrict__ flags, uint8_t* __restrict__ cls,
+                                                     Counters* cnt) {
+    int32_t nfin = 0;
+    for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+        const bool top = key[v] == top_key();
+        cls[v] = top ? kTop : kFin;
+        nfin += !top && !(flags[v] & kSinkSlot);
+    }
+    block_add32(nfin, &cnt->n_fin);
+}
+
 // The switching rules on keys (first minimiser for Odd; the sink first, then
 // the first maximiser for Even; strictly better only), one thread per vertex.
 // inc: the switched vertices are listed for k_inc, Even's pass clears its
@@ -659,6 +671,15 @@ pg_status enqueue_valuation_cv(pg_game* g, bool want_dom) {
     prof_end(g, KID_CHAIN2, 1);
     PG_CUDA_TRY(ctx, cudaGetLastError());
     return PG_OK;
+}
+
+pg_status classes_cv(pg_game* g) {
+    pg_ctx* ctx = g->ctx;
+    PG_CUDA_TRY(ctx, cudaMemsetAsync(g->cnt, 0, sizeof(Counters), ctx->stream));
+    k_class_cv<<<grid_n(g->n), kBlock, 0, ctx->stream>>>(g->n, g->key128, g->flags, g->cls, g->cnt);
+    ctx->launches += 1;
+    PG_CUDA_TRY(ctx, cudaGetLastError());
+    return sync_counters(g);
 }
 
 pg_status enqueue_switch_cv(pg_game* g, int player) {

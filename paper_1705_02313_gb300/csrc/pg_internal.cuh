@@ -108,6 +108,8 @@ struct IncState {
     int32_t n_q;        // k_inc: Odd's queue beyond the blocks' own
     int32_t wait;       // full iterations before the next incremental one is tried, and
     int32_t fails;      //    attempts abandoned in a row
+    int32_t stale;      // k_inc has valuated since the last full iteration (count vectors: the classes and walk
+                        // lengths are not the current ones)
 };
 // Games of up to this many ids run their whole loop in one launch of k_inc (41k ids: 17-32 us for an iteration
 // over all ids, against 45 us for the passes of a full iteration as graph nodes; they grow with the ids, and
@@ -303,7 +305,9 @@ struct pg_game {
     int64_t loop_launch[2] = {0, 0};                  // kernels per iteration of each graph
     int64_t loop_klaunch[2][pg::KID_COUNT] = {};      // per kernel class
     bool last_graph = false;     // the last loop ran as a graph
+    bool last_stale = false;     //   and ended with incremental iterations (count vectors: IncState::stale)
     bool last_cmp = false;       // the last loop compared valuations: key, cls and depth are not the current ones
+                                 // (count vectors: the keys are)
     // the switching player's view (built before the first loop that compares valuations): for p = 0
     // (Even, dummies included) and 1 (Odd) the ids of p's vertices in increasing order and their edge
     // lists, contiguous (int32 offsets; a player with 2^31 or more edges keeps the unsplit passes)
@@ -453,7 +457,8 @@ uint8_t* omark_of(const pg_game* g);  // the Odd marks in use by the loop, or nu
 pg_status enqueue_valuation_cmp(pg_game* g);
 pg_status enqueue_switch_cmp(pg_game* g, int player);
 // After a loop that compared valuations: the full valuation of the current profile (key, cls, depth).
-pg_status finish_loop(pg_game* g);
+// (timed_out: the last switching pass came after the last valuation; depths: they are asked for).
+pg_status finish_loop(pg_game* g, bool timed_out, bool depths);
 // Builds the switching players' views (pl_*) if they are missing; not under stream capture.
 pg_status build_player_split(pg_game* g);
 // Incremental iterations (pg_inc.cu): whether the game takes them, the reverse adjacency they and the marks
@@ -488,6 +493,8 @@ pg_status alloc_cv(pg_game* g);
 pg_status enqueue_valuation_cv(pg_game* g, bool want_dom);
 pg_status enqueue_switch_cv(pg_game* g, int player);
 pg_status write_counts(pg_game* g, int32_t mem_kind, int32_t* counts);
+// The classes from the keys of the last iteration (no odd cycle was met).
+pg_status classes_cv(pg_game* g);
 // Bellman-Ford best response against the sigma in g->strat (count-vector mode).
 pg_status bellman_ford_cv(pg_game* g, int64_t* rounds);
 }  // namespace pg

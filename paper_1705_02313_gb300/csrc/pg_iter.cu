@@ -1202,12 +1202,13 @@ __global__ void k_bookkeep(int32_t ngames, GameState* gst, int64_t cap, int even
     int32_t act = 0;
     for (int32_t gi = blockIdx.x * blockDim.x + threadIdx.x; gi < ngames; gi += gridDim.x * blockDim.x) {
         GameState st = gst[gi];
-        const int32_t wait = inc ? inc->wait : 0;
+        const int32_t wait = inc ? inc->wait : 0, was = inc ? inc->mode : 0;
         st.reset = 0;
         if (inc) {  // one game: Even's marks are exact after an Even pass, and not kept by a full iteration
             inc->mode = kIncFull;
             inc->even_full = !(even_phase && st.sw_odd == 0);
             inc->wait = max(wait - 1, 0);
+            if (was == kIncFull) inc->stale = 0;
         }
         if (st.phase == kPhaseActive) {
             st.inner += 1;
@@ -2101,9 +2102,10 @@ pg_status enqueue_switch_cmp(pg_game* g, int player) {
     return PG_OK;
 }
 
-pg_status finish_loop(pg_game* g) {
-    if (!g->last_cmp) return PG_OK;
-    pg_status st = full_valuation(g, false);
+pg_status finish_loop(pg_game* g, bool timed_out, bool depths) {
+    if (!timed_out && !g->last_cmp) return PG_OK;
+    // (with keys, only the classes are missing unless the depths are asked for)
+    pg_status st = g->cv && !timed_out && !depths ? classes_cv(g) : full_valuation(g, false);
     if (!st) g->last_cmp = false;
     return st;
 }
