@@ -947,7 +947,8 @@ pg_status load_union(pg_ctx* ctx, int32_t ng, const int64_t* vb, const int64_t* 
         if (top > INT32_MAX - 1) return PG_OK;
         G[i].words = (int32_t)words;
         words += (top >> 5) + 1;
-        if (words > NP + 64 * (int64_t)ng) return PG_OK;  // sparse priorities: at most a word per vertex here
+        // sparse priorities: a word per vertex, or 32 MB with the prefix
+        if (words > std::max<int64_t>(NP + 64 * (int64_t)ng, 1 << 22)) return PG_OK;
     }
 
     pg_game* g = new pg_game();
