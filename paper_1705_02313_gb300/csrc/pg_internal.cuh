@@ -30,7 +30,8 @@ constexpr int kCoopTile = 4096;       // elements per tile of the id-ordered sca
 constexpr int kClusterDevices = 64;   // devices whose cluster sizes are remembered
 constexpr int32_t kLoadSmall = 1 << 22;  // a game of up to this many vertices is loaded in one launch (pg_load_small.cu)
 constexpr int32_t kSlabIds = 1 << 20;  // a game of up to this many ids has its scratch in one allocation
-constexpr int32_t kSmallIds = (1 << 18) + 1;  // a game of up to this many ids is valuated by one cluster (pg_small.cu)
+constexpr int32_t kSmallIds = (1 << 18) + 1;  // a game of up to this many ids is valuated in one launch (pg_small.cu)
+constexpr int kSmallBlocks = 512;  // of at most this many blocks (the array of their sums)
 // Count-vector mode (repeated priorities): at most kMaxLevels distinct
 // priorities; a count vector is one signed 128-bit key with one digit per
 // level (Levels::shift), each wide enough that its signed count stays below

@@ -1737,7 +1737,7 @@ pg_status alloc_scratch(pg_game* g) {
         PG_A(A((void**)&g->depth, sizeof(int32_t) * n));
         PG_A(A((void**)&g->dom, sizeof(int32_t) * n));
         g->ntiles = std::max<int64_t>(1, (n + kCoopTile - 1) / kCoopTile);
-        PG_A(A((void**)&g->tiles, sizeof(int64_t) * std::max<int64_t>(2 * g->ntiles + 2, 256)));
+        PG_A(A((void**)&g->tiles, sizeof(int64_t) * std::max<int64_t>(2 * g->ntiles + 2, kSmallBlocks)));
         PG_A(A((void**)&g->tsum, sizeof(int64_t) * (2 * g->ntiles + 2)));
         PG_A(A((void**)&g->gscan, sizeof(int64_t) * 3 * (size_t)g->ngames));
         PG_A(A((void**)&g->gst, sizeof(GameState) * (size_t)g->ngames));

@@ -54,7 +54,7 @@ constexpr Layout make_layout() {
     L.depth = p;    p = al256(p + 4 * N);
     L.hugelist = p; p = al256(p + 4 * N);
     L.flags = p;    p = al256(p + N);
-    L.tiles = p;    p = al256(p + 8 * std::max<size_t>(2 * ntiles + 2, 256));
+    L.tiles = p;    p = al256(p + 8 * std::max<size_t>(2 * ntiles + 2, kSmallBlocks));
     L.gst = p;      p = al256(p + sizeof(GameState));
     L.cnt = p;      p = al256(p + sizeof(Counters));
     L.bytes = p;

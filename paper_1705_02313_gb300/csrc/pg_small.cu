@@ -5,8 +5,8 @@
 // enqueue_valuation are latency only: each pass takes 2 to 10 us for reads that
 // take one, plus the gap to the next. k_val_small runs them all in one launch:
 // of a cluster of up to 16 blocks with the cluster barrier (about 0.4 us)
-// between the passes or, beyond kSmallGrid ids, of one block per SM with the
-// software barrier (about 1.3 us). The ranks and depths are those of the
+// between the passes or, beyond kSmallGrid ids, of one or two blocks per SM with
+// the software barrier (about 1.3 us). The ranks and depths are those of the
 // separate kernels. pg_valuate_static of 100k vertices: 158 -> 76 us.
 #include <cooperative_groups.h>
 
@@ -18,14 +18,25 @@ namespace pg {
 namespace {
 
 // Up to the sibling weights, cluster against grid: 10k ids 22 / 33 us, 40k 40 /
-// 35 us, 100k 76 / 36 us, 262k 170 / 47 us.
-constexpr int32_t kSmallGrid = 24576;
+// 35 us, 100k 76 / 36 us, 262k 170 / 47 us. The cluster takes what its threads hold
+// at once: beyond, a second round of chains doubles the time of deep forests (20k
+// vertices in runs of 50: 202 / 161 us). For the same reason the grid has two
+// blocks per SM beyond 155,648 ids (260k: 276 / 172 us).
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallCluster = 16;
+constexpr int32_t kSmallGrid = kSmallCluster * kSmallThreads;
+// A warp orders up to this many children of one parent, a block more (that many,
+// in blocks: 260k vertices, 100 to a parent, 497 us, 407 with warps).
+constexpr int kSmallWarpKids = 128;
 constexpr int kSmallHot = 2048;  // the block's table of additions near the roots (as in k_chain1)
 constexpr int kSmallHotBits = 11;
+constexpr int kSmallTop = 8;     // takes the last this many g-ancestors of a chain
+// With two blocks per SM the lanes of a warp add to the table in step, or else
+// several chains wait for each other's: plays through 160k, 200k and 260k vertices
+// 304, 372 and 390 us, in step 259, 292 and 351 (by the separate kernels 312, 344
+// and 341); runs of 50 rising vertices 206, 220 and 218, in step 211, 214 and 220
+// (100k, one block: 191, in step 262).
 constexpr int kSmallSteps = 128;   // steps of one resolution round
-constexpr int kSmallBlocks = 256;  // at most this many blocks (the array of their sums)
 
 // Three sums in one word: children of vertices, sizes of the sink's even and of its odd children. Each is at
 // most kSmallIds < 2^21.
@@ -79,16 +90,17 @@ __device__ inline uint64_t small_sums(const SmallArgs& a, int32_t v, uint8_t kd)
     return s;
 }
 
-// GRID: the launch is cooperative and its blocks meet at the software barrier
-// (which gives up after a bounded wait: every block then returns); otherwise it
-// is one cluster. Reads of what the kernel itself writes go to L2 (__ldcg): the
-// barrier makes them visible there.
-template <bool GRID>
-__global__ void __launch_bounds__(kSmallThreads, 1) k_val_small(SmallArgs a) {
+// PER_SM > 0: the launch is cooperative, of up to that many blocks per SM, and its
+// blocks meet at the software barrier (which gives up after a bounded wait: every
+// block then returns); otherwise it is one cluster. Reads of what the kernel itself
+// writes go to L2 (__ldcg): the barrier makes them visible there.
+template <int PER_SM>
+__global__ void __launch_bounds__(kSmallThreads, PER_SM == 2 ? 2 : 1) k_val_small(SmallArgs a) {
+    constexpr bool kInStep = PER_SM == 2;
     const int32_t tid = threadIdx.x, CL = (int32_t)gridDim.x, rank = (int32_t)blockIdx.x;
     const int32_t T = CL * kSmallThreads, t0 = rank * kSmallThreads + tid;
     auto sync = [&] {
-        if constexpr (GRID) return grid_sync(a.cnt);
+        if constexpr (PER_SM > 0) return grid_sync(a.cnt);
         cg::this_cluster().sync();
         return true;
     };
@@ -182,20 +194,14 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_val_small(SmallArgs a) {
     }
     // classification, g-subtree sizes, children counts (as k_chain1)
     int32_t nfin = 0, nodd = 0;
-    for (int32_t v = t0; v < n; v += T) {
-        const uint32_t w = __ldcg(a.gd32 + v);
-        const uint8_t f = a.flags[v];
-        if (f & kSinkSlot) {
-            a.kind[v] = kKSinkSlot;
-            a.cls[v] = kFin;
-            if (a.want_dom) a.dom[v] = -1;
-            a.slot[v] = -1;
-            continue;
-        }
-        const int32_t g = g32_ptr(w);
-        int32_t cyc = g32_none(w) ? g : -1, len = 0, x = g;
+    for (int32_t b = t0 - lane; b < n; b += T) {
+        const int32_t v = b + lane;
+        const uint32_t w = v < n ? __ldcg(a.gd32 + v) : kG32Sink;
+        const uint8_t f = v < n ? a.flags[v] : kSinkSlot;
+        const bool slot = (f & kSinkSlot) != 0;
+        int32_t x = g32_ptr(w), cyc = !slot && g32_none(w) ? x : -1, len = 0;
         bool cut = false;
-        for (bool act = !g32_none(w) && !g32_sink(w); act;) {
+        for (bool act = !slot && !g32_none(w) && !g32_sink(w); act;) {
             if (len >= a.deep_cut) {
                 cut = true;
                 cnt->deep = 1;
@@ -211,20 +217,41 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_val_small(SmallArgs a) {
                 act = !g32_sink(wx);
             }
         }
+        // one more for each of the len g-ancestors of a finite vertex, the last ones of a long chain in the block's
+        // table (in step: with all lanes at the same distance from their roots)
         int32_t sl = -1;
-        if (cyc < 0 && !g32_sink(w) && !cut) {
-            sl = atomicAdd(a.ccnt + g, 1);
-            const bool deep = len >= 4;
-            x = g;
+        const bool child = !slot && cyc < 0 && !g32_sink(w) && !cut, table = child && len >= 4;
+        x = g32_ptr(w);
+        if (child) {
+            sl = atomicAdd(a.ccnt + x, 1);
             for (;; --len) {
-                if (deep && len <= 8) small_hot_add(x, tkey, tcnt, a.sz);
-                else atomicAdd(a.sz + x, 1);
+                if (table && len <= kSmallTop) {
+                    if (kInStep) break;
+                    small_hot_add(x, tkey, tcnt, a.sz);
+                } else {
+                    atomicAdd(a.sz + x, 1);
+                }
                 const uint32_t wx = __ldcg(a.gd32 + x);
                 if (g32_sink(wx)) break;
                 x = g32_ptr(wx);
             }
         }
-        if (cyc < 0) {
+        if (kInStep && __any_sync(kFull, table)) {
+            for (int32_t l = kSmallTop; l > 0; --l) {
+                if (table && len >= l) {
+                    small_hot_add(x, tkey, tcnt, a.sz);
+                    if (l > 1) x = g32_ptr(__ldcg(a.gd32 + x));
+                }
+                __syncwarp();
+            }
+        }
+        if (v >= n) continue;
+        a.slot[v] = sl;
+        if (slot) {
+            a.kind[v] = kKSinkSlot;
+            a.cls[v] = kFin;
+            if (a.want_dom) a.dom[v] = -1;
+        } else if (cyc < 0) {
             a.kind[v] = kKFin | (g32_sink(w) ? kKSinkChild : 0) | ((f & kPriOdd) ? kKOdd : 0);
             a.cls[v] = kFin;
             if (a.want_dom) a.dom[v] = -1;
@@ -236,7 +263,6 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_val_small(SmallArgs a) {
             if (a.want_dom) a.dom[v] = a.pri[cyc];
             nodd += odd;
         }
-        a.slot[v] = sl;
     }
     __syncthreads();
     for (int i = tid; i < kSmallHot; i += kSmallThreads)
@@ -345,9 +371,37 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_val_small(SmallArgs a) {
     }
     if (!sync()) return;
     const int32_t nb = __ldcg(&cnt->n_big), nh = __ldcg(&cnt->n_huge);
+    // parents with up to kSmallWarpKids children: a warp each, four children to a lane
+    for (int32_t b = t0 >> 5; b < nb; b += T >> 5) {
+        const int32_t p = __ldcg(a.biglist + b), s0 = __ldcg(a.coff + p), k = __ldcg(a.coff + p + 1) - s0;
+        if (k > kSmallWarpKids) continue;
+        int2 c[4];
+        int32_t pre[4] = {0, 0, 0, 0}, os = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            c[i] = lane + 32 * i < k ? __ldcg(a.cl_ks + s0 + lane + 32 * i) : make_int2(INT32_MAX, 0);
+            if (c[i].x < 0) os += c[i].y;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int kn = min(32, k - 32 * i);
+            for (int j = 0; j < kn; ++j) {
+                const int32_t kx = __shfl_sync(kFull, c[i].x, j), ky = __shfl_sync(kFull, c[i].y, j);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (kx < c[q].x) pre[q] += ky;
+            }
+        }
+        os = __reduce_add_sync(kFull, os);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (lane + 32 * i < k) a.wgt[c[i].x >= 0 ? c[i].x : -c[i].x - 1] = pre[i] + (c[i].x >= 0 ? 1 : 0);
+        if (lane == 0) a.oddsz[p] = os;
+    }
     // parents with up to kHugeChildren children: a block each sorts the segment and scans it
     for (int32_t b = rank; b < nb; b += CL) {
         const int32_t p = __ldcg(a.biglist + b), s0 = __ldcg(a.coff + p), k = __ldcg(a.coff + p + 1) - s0;
+        if (k <= kSmallWarpKids) continue;
         int p2 = 64;
         while (p2 < k) p2 <<= 1;
         for (int i = tid; i < p2; i += kSmallThreads) sk[i] = i < k ? __ldcg(a.cl_ks + s0 + i) : make_int2(INT32_MAX, 0);
@@ -506,15 +560,16 @@ pg_status enqueue_val_small(pg_game* g, bool want_dom) {
     if (g->n > kSmallGrid) {
         int sms = 0;
         PG_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device));
-        const int blocks = std::max(1, std::min({sms, kSmallBlocks, (g->n + kSmallThreads - 1) / kSmallThreads}));
+        const int per = g->n > sms * kSmallThreads ? 2 : 1;
+        const int blocks = std::max(1, std::min({per * sms, kSmallBlocks, (g->n + kSmallThreads - 1) / kSmallThreads}));
         void* args[] = {(void*)&a};
-        PG_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((void*)k_val_small<true>, blocks, kSmallThreads, args, 0,
-                                                     ctx->stream));
+        PG_CUDA_TRY(ctx, cudaLaunchCooperativeKernel(per == 2 ? (void*)k_val_small<2> : (void*)k_val_small<1>, blocks,
+                                                     kSmallThreads, args, 0, ctx->stream));
         return PG_OK;
     }
     int c = kSmallCluster;
     while (c > 1 && (int64_t)c * kSmallThreads / 2 >= g->n) c >>= 1;
-    c = std::min(c, cluster_blocks((const void*)k_val_small<false>, kSmallThreads, 0, kSmallCluster, g->device,
+    c = std::min(c, cluster_blocks((const void*)k_val_small<0>, kSmallThreads, 0, kSmallCluster, g->device,
                                    g_small_cluster));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(c);
@@ -526,7 +581,7 @@ pg_status enqueue_val_small(pg_game* g, bool want_dom) {
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    PG_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, k_val_small<false>, a));
+    PG_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, k_val_small<0>, a));
     return PG_OK;
 }
 
