@@ -448,7 +448,10 @@ bool build_loop_graph(pg_game* g, int64_t cap, bool even, int64_t limit) {
         ok = cudaStreamBeginCaptureToGraph(ctx->cap_stream, body, nullptr, nullptr, 0,
                                            cudaStreamCaptureModeThreadLocal) == cudaSuccess;
         if (ok) {
+            g->val_deep = g->depth_ok = false;
             bool enq = enqueue_body(g, cap, even) == PG_OK;
+            g->loop_val_deep[w] = g->val_deep;  // what the valuations of the body leave, for every run of the graph
+            g->loop_depth_ok[w] = g->depth_ok;
             if (enq) {
                 k_loop_cond<<<1, 1, 0, ctx->cap_stream>>>(h, g->gactive, g->cnt, g->loop_iters, limit);
                 enq = cudaGetLastError() == cudaSuccess;
@@ -524,6 +527,8 @@ pg_status run_loop_once(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t l
         cudaStream_t s = ctx->stream;
         PG_CUDA_TRY(ctx, cudaMemsetAsync(g->loop_iters, 0, 2 * sizeof(int64_t), s));
         PG_CUDA_TRY(ctx, cudaGraphLaunch(g->loop_exec[w], s));
+        g->val_deep = g->loop_val_deep[w];
+        g->depth_ok = g->loop_depth_ok[w];
         int64_t* it = (int64_t*)ctx->pinned;
         PG_CUDA_TRY(ctx, cudaMemcpyAsync(it, g->loop_iters, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
         IncState* inc = (IncState*)(it + 2);

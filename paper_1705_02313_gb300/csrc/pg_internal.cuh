@@ -353,6 +353,7 @@ struct pg_game {
     bool loop_reset[2] = {false, false};  // the SI-Reset setting each loop graph was built with
     bool loop_cmp[2] = {false, false};    // each loop graph compares valuations (loop_compares)
     bool loop_deep[2] = {false, false};   // each loop graph ranks through the ruling-set path
+    bool loop_val_deep[2] = {false, false}, loop_depth_ok[2] = {false, false};  // val_deep, depth_ok after it ran
     pg::Tune loop_tune[2];                // the partitioning each loop graph was built with
     pg::Tune tune;                        // the partitioning of the current call (tune_for, at its start)
     // timing of the last call
