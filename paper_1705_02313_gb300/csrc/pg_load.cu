@@ -857,6 +857,7 @@ pg_status load_game(pg_ctx* ctx, int32_t n, int64_t m, const int32_t* off_in, co
     if (out && off_in && tgt_in && own_in && pri_in && n >= 1 && n <= kLoadSmall && m >= n && m <= 8 * (int64_t)kLoadSmall &&
         (mem_kind == PG_MEM_HOST || mem_kind == PG_MEM_DEVICE)) {
         bool general = false;
+        const std::string err = ctx->err;
         pg_status st = load_small(ctx, n, m, off_in, tgt_in, own_in, pri_in, mem_kind, out, &general);
         if (st == PG_OK && !general && with_scratch) {
             st = alloc_scratch(*out);
@@ -865,7 +866,13 @@ pg_status load_game(pg_ctx* ctx, int32_t n, int64_t m, const int32_t* off_in, co
                 *out = nullptr;
             }
         }
-        if (st || !general) return st;
+        if (st == PG_OK && !general) return st;
+        // a game it leaves, a launch that was refused, or too little memory: the general path's arrays have the
+        // game's exact sizes, and its kernels no conditions
+        if (st) {
+            cudaGetLastError();
+            ctx->err = err;
+        }
     }
     bool again = false;
     pg_status st = load_game_pass(ctx, n, m, off_in, tgt_in, own_in, pri_in, mem_kind, out, with_scratch, false, &again);
