@@ -71,6 +71,17 @@ cudaError_t dev_alloc(pg_ctx* ctx, void** p, size_t bytes, cudaStream_t s) {
     return cudaMallocFromPoolAsync(p, bytes ? bytes : 1, pool, s);
 }
 
+cudaError_t game_alloc(pg_game* g, void** p, size_t bytes) {
+    pg_ctx* ctx = g->ctx;
+    cudaError_t e = dev_alloc(ctx, p, bytes, ctx->stream);
+    if (e != cudaErrorMemoryAllocation || !g->rv) return e;
+    cudaGetLastError();
+    drop_loop_graphs(g);  // (they hold the lists' addresses)
+    drop_reverse(g);
+    e = dev_trim(ctx->device);  // (waits for the device)
+    return e == cudaSuccess ? dev_alloc(ctx, p, bytes, ctx->stream) : e;
+}
+
 cudaError_t dev_trim(int device) {
     cudaMemPool_t pool = nullptr;
     cudaError_t e = game_pool(device, &pool);
@@ -274,7 +285,7 @@ pg_status write_outputs(pg_game* g, int32_t mem_kind, uint8_t* win, int32_t* sig
     OutPtrs o = {g->cv ? 1 : 0, win, sigma, tau, vclass, vdepth, vrank, vdom, dsig};
     Stage L = stage_layout(g->n0, g->k);
     if (mem_kind == PG_MEM_HOST) {
-        if (!g->stage) PG_CUDA_TRY(ctx, dev_alloc(ctx, &g->stage, L.bytes, s));
+        if (!g->stage) PG_CUDA_TRY(ctx, game_alloc(g, &g->stage, L.bytes));
         char* b = (char*)g->stage;
         o = {g->cv ? 1 : 0,
              win ? (uint8_t*)(b + L.off_win) : nullptr,     sigma ? (int32_t*)(b + L.off_sigma) : nullptr,
@@ -323,7 +334,7 @@ pg_status apply_profile(pg_game* g, const int32_t* sigma, const int32_t* tau, co
     cudaError_t e = cudaSuccess;
     if (mem_kind == PG_MEM_HOST && (sigma || tau || dsig)) {
         size_t bytes = 8 * (size_t)g->n0 + (size_t)g->k + 16;
-        PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&buf, bytes, s));
+        PG_CUDA_TRY(ctx, game_alloc(g, (void**)&buf, bytes));
         char* b = (char*)buf;
         if (sigma) {
             e = cudaMemcpyAsync(b, sigma, 4 * (size_t)g->n0, cudaMemcpyHostToDevice, s);

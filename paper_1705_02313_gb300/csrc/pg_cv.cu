@@ -701,7 +701,7 @@ pg_status write_counts(pg_game* g, int32_t mem_kind, int32_t* counts) {
     cudaStream_t s = ctx->stream;
     const size_t bytes = sizeof(int32_t) * (size_t)g->n0 * (size_t)g->lev.n;
     int32_t* dst = counts;
-    if (mem_kind == PG_MEM_HOST) PG_CUDA_TRY(ctx, cudaMallocAsync((void**)&dst, bytes ? bytes : 4, s));
+    if (mem_kind == PG_MEM_HOST) PG_CUDA_TRY(ctx, game_alloc(g, (void**)&dst, bytes));
     ctx->launches += 1;
     k_counts<<<grid_n(g->n0), kBlock, 0, s>>>(g->n0, g->nid0, g->key128, g->cls, g->lev, dst);
     cudaError_t e = cudaGetLastError();

@@ -749,7 +749,7 @@ __global__ void __launch_bounds__(kBlock) k_rv_fill(int32_t n, const OffT* __res
 
 bool inc_applies(const pg_game* g) { return !g->vgame && g->ngames == 1 && g->off != nullptr && !g->no_inc; }
 
-static void drop_reverse(pg_game* g) {
+void drop_reverse(pg_game* g) {
     g->rv_ok = false;
     for (void** q : {(void**)&g->rv, (void**)&g->rv_src, (void**)&g->omark, (void**)&g->emark}) {
         if (*q) cudaFreeAsync(*q, g->ctx->stream);

@@ -435,6 +435,9 @@ void free_game(pg_game* g);
 // memory) for the next game, instead of mapping and unmapping it each time.
 // Everything free_game releases comes from here.
 cudaError_t dev_alloc(pg_ctx* ctx, void** p, size_t bytes, cudaStream_t s);
+// What a call on a loaded game needs beside them: when there is no memory for it, the game's reverse lists, which
+// only save time, make room.
+cudaError_t game_alloc(pg_game* g, void** p, size_t bytes);
 // Returns the pool's cached memory to the device (pg_release_cached_memory).
 cudaError_t dev_trim(int device);
 // Co-resident blocks of the cooperative valuation kernels on a device.
@@ -473,6 +476,7 @@ bool games_apply(const pg_game* g, int* div, int* blocks);
 pg_status run_games(pg_game* g, int64_t cap, int div, int blocks, bool* done);
 IncState* inc_of(const pg_game* g);  // the state, when the loop's full iterations prepare incremental ones, or null
 pg_status build_reverse(pg_game* g, int64_t odd_edges);
+void drop_reverse(pg_game* g);
 int32_t inc_max_seeds(const pg_game* g);
 pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole);
 // The valuation of a small game, depths included, in one launch (pg_small.cu; the counters are clear).

@@ -13,7 +13,7 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-CASES = ["load", "load_all", "batch"]
+CASES = ["load", "load_all", "solve_whole", "solve_graph", "solve_levels", "batch"]
 
 
 @pytest.mark.parametrize("case", CASES)
