@@ -652,15 +652,10 @@ namespace pg {
 // Scratch of the ruling-set path, allocated before the game's first deep
 // valuation (outside any stream capture: the loops call this before they
 // build their graph).
-pg_status prepare_deep(pg_game* g) {
+static pg_status alloc_deep(pg_game* g, int32_t rcap) {
     pg_ctx* ctx = g->ctx;
     const int64_t n = g->n;
-    const int bits = std::max(1, std::min(g->tune.ruler_bits, 16));
-    // rulers: list heads plus about 2n / 2^bits hashed ones, with room for twice that
-    const int64_t want = 2 * ((2 * n) >> bits) + g->ngames + 1024;
-    const int32_t rcap = (int32_t)std::min<int64_t>(want, 2 * n + g->ngames + 1024);
-    if (g->d_anc && g->d_rcap >= rcap) return PG_OK;
-    auto A = [&](void** p, size_t bytes) { return dev_alloc(ctx, p, bytes, ctx->stream); };
+    auto A = [&](void** p, size_t bytes) { return game_alloc(g, p, bytes); };
     if (!g->d_anc) {
         PG_CUDA_TRY(ctx, A((void**)&g->d_anc, sizeof(int32_t) * n));
         PG_CUDA_TRY(ctx, A((void**)&g->d_sc, 2 * (size_t)n));
@@ -679,19 +674,38 @@ pg_status prepare_deep(pg_game* g) {
         PG_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_deep_wyllie_coop, kBlock, 0));
         g->d_coop = sms * std::max(1, std::min(std::min(a, b), 4));
     }
-    if (g->d_rl) {  // a denser ruler setting than the scratch was made for
-        cudaFreeAsync(g->d_rl, ctx->stream);
-        cudaFreeAsync(g->d_val, ctx->stream);
-        cudaFreeAsync(g->d_rnx, ctx->stream);
-        g->d_rl = nullptr;
-        g->d_val = nullptr;
-        g->d_rnx = nullptr;
-    }
     PG_CUDA_TRY(ctx, A((void**)&g->d_rl, sizeof(int32_t) * rcap));
     PG_CUDA_TRY(ctx, A((void**)&g->d_val, sizeof(int2) * 2 * (size_t)rcap));
     PG_CUDA_TRY(ctx, A((void**)&g->d_rnx, sizeof(int32_t) * 2 * (size_t)rcap));
     g->d_rcap = rcap;
     return PG_OK;
+}
+
+// Gives back the rulers' arrays (a denser ruler setting), or all.
+static void free_deep(pg_game* g, bool all) {
+    auto F = [&](auto*& p) {
+        if (p) cudaFreeAsync(p, g->ctx->stream);
+        p = nullptr;
+    };
+    g->d_rcap = 0;
+    F(g->d_rl), F(g->d_val), F(g->d_rnx);
+    if (all)
+        F(g->d_anc), F(g->d_sc), F(g->d_podd), F(g->d_peven), F(g->d_oddL), F(g->d_evenL), F(g->d_nxt), F(g->d_wt),
+            F(g->d_loc), F(g->d_own), F(g->d_rid);
+}
+
+pg_status prepare_deep(pg_game* g) {
+    const int64_t n = g->n;
+    const int bits = std::max(1, std::min(g->tune.ruler_bits, 16));
+    // rulers: list heads plus about 2n / 2^bits hashed ones, with room for twice that
+    const int64_t want = 2 * ((2 * n) >> bits) + g->ngames + 1024;
+    const int32_t rcap = (int32_t)std::min<int64_t>(want, 2 * n + g->ngames + 1024);
+    if (g->d_anc && g->d_rcap >= rcap) return PG_OK;
+    drop_loop_graphs(g);  // (a captured loop holds the arrays' addresses)
+    free_deep(g, false);
+    pg_status st = alloc_deep(g, rcap);
+    if (st) free_deep(g, true);  // (all of them or none: the valuation asks for d_anc and the rulers only)
+    return st;
 }
 
 pg_status enqueue_valuation_deep(pg_game* g, bool want_dom) {

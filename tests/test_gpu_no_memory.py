@@ -13,7 +13,7 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-CASES = ["load", "load_all", "solve_whole", "solve_graph", "solve_levels", "batch"]
+CASES = ["load", "load_all", "solve_whole", "solve_graph", "solve_levels", "solve_deep", "batch"]
 
 
 @pytest.mark.parametrize("case", CASES)
