@@ -481,7 +481,7 @@ int32_t inc_max_seeds(const pg_game* g);
 pg_status enqueue_inc(pg_game* g, int64_t cap, bool even, bool whole);
 // The valuation of a small game, depths included, in one launch (pg_small.cu; the counters are clear).
 pg_status enqueue_val_small(pg_game* g, bool want_dom);
-// The largest cluster of at most want blocks that the device runs for kern (asked once per device: cache).
+// The largest cluster of at most want blocks that the device runs for kern (an answer is kept per device: cache).
 int cluster_blocks(const void* kern, int threads, size_t shared, int want, int device, std::atomic<int>* cache);
 // K1 alone (counters cleared, nearest-greater walks and pointer jumping with walk lengths).
 pg_status enqueue_k1(pg_game* g);

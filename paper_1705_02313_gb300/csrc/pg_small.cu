@@ -492,12 +492,12 @@ __global__ void __launch_bounds__(kSmallThreads, PER_SM == 2 ? 2 : 1) k_val_smal
 }  // namespace
 
 int cluster_blocks(const void* kern, int threads, size_t shared, int want, int device, std::atomic<int>* cache) {
-    if (device < 0 || device >= kClusterDevices) return 1;
-    int c = cache[device].load();
-    if (c) return c;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (shared) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared);
-    for (c = want; c > 1; c >>= 1) {
+    const bool cached = device >= 0 && device < kClusterDevices;
+    if (int c = cached ? cache[device].load() : 0) return c;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);  // (refused: smaller clusters)
+    bool ready = !shared || cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared) ==
+                                cudaSuccess;
+    for (int c = want; ready && c >= 1; c >>= 1) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(c);
         cfg.blockDim = dim3(threads);
@@ -509,11 +509,14 @@ int cluster_blocks(const void* kern, int threads, size_t shared, int want, int d
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int k = 0;
-        if (cudaOccupancyMaxActiveClusters(&k, kern, &cfg) == cudaSuccess && k > 0) break;
-        cudaGetLastError();
+        if (cudaOccupancyMaxActiveClusters(&k, kern, &cfg) == cudaSuccess && k > 0) {
+            cudaGetLastError();
+            if (cached) cache[device].store(c);
+            return c;
+        }
     }
-    cache[device].store(c);
-    return c;
+    cudaGetLastError();
+    return 1;  // (asked again next time: the launch says what is wrong)
 }
 
 namespace {
