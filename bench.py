@@ -18,10 +18,11 @@ bounded sample of the same workload: each step runs the first iterations of
 the same solve.
 
 Beside the headline the line carries: the end-to-end rate from pinned host
-memory, the roofline of the inner iteration (B_alg = 8 m' + 20 n' bytes per
-valuation + switching pass, over the solve time of the timed steps, against
-the measured HBM bandwidth; DRAM traffic from the committed ncu summary while
-the kernels' sources are unchanged), the dominant kernel, per-kernel times, SI-Reset, the 4-priority count-vector game, the
+memory, the roofline of a full inner iteration (B_alg = 8 m' + 20 n' bytes per
+valuation + switching pass over all vertices, against the measured HBM
+bandwidth; DRAM traffic from the committed ncu summary while the kernels'
+sources are unchanged) with the solve's mean iteration beside it, the dominant
+kernel, per-kernel times, SI-Reset, the 4-priority count-vector game, the
 4,096-game batch (--batch batch-256 for a small one), a Poisson serving
 stream (--serve seconds, 60 by default), an optional long-chain valuation (--chain n), and
 the oracle timed on the host cores (one core for the solve; all cores, one
@@ -164,6 +165,29 @@ def algorithmic_bytes(name, s):
     return table.get(name)
 
 
+def iteration_roofline(m, np_, mp, full_s, mean_s, hbm):
+    """The inner iteration of a solve (valuation and switching) of a game of m
+    edges, np_ vertices and mp edges of G'. A full iteration (full_s seconds,
+    over all vertices) is set against B_alg = 8 m' + 20 n' bytes, one pass over
+    the edges and a few per-id arrays, at the measured HBM copy bandwidth. The
+    solve's mean iteration (mean_s) is shorter: many work on the few vertices
+    that the last switches affect (incremental iterations) and move a fraction of
+    those bytes, so its rate in B_alg is a rate of the algorithm and no share of
+    the memory's bandwidth."""
+    b_alg = 8 * mp + 20 * np_
+    gbs = b_alg / full_s / 1e9 if full_s else None
+    return {"bound": "hbm", "kernel": "full inner iteration (valuation + switching over all vertices)",
+            "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm if gbs else None,
+            "algorithmic_bytes_per_launch": b_alg, "avg_launch_us": full_s * 1e6 if full_s else None,
+            "units": "one full iteration: B_alg = 8 m' + 20 n' bytes, m' = %d edges and n' = %d vertices of G' "
+                     "(the Odd switching pass evaluates only the vertices some of whose successors changed their top "
+                     "word, so it moves less)" % (mp, np_),
+            "timing": "host-driven timing pass (one launch per kernel, events around each class)",
+            "mean_iteration": {"us": mean_s * 1e6, "b_alg_per_s": b_alg / mean_s, "edges_per_s": m / mean_s,
+                               "timing": "solve time of the timed steps (CUDA events around pg_solve on the library's "
+                                         "stream) / valuations, full and incremental"}}
+
+
 def kernel_entry(name, v, s, hbm):
     """Per kernel class: device ms over the timed solve, launches, calls, and
     algorithmic GB/s per call against the measured HBM copy bandwidth."""
@@ -180,8 +204,8 @@ def kernel_entry(name, v, s, hbm):
 # where each kernel class whose DRAM traffic is recorded is defined
 KERNEL_SOURCE = {"chain1": ("pg_iter.cu", "k_chain1("), "classify": ("pg_iter.cu", "k_classify("),
                  "walk": ("pg_iter.cu", "k_walk_cmp("), "switch_odd": ("pg_iter.cu", "k_switch_cmp_pl(")}
-# the files holding the kernels of one inner iteration (their traffic is recorded as "iteration")
-ITERATION_SOURCES = ("pg_iter.cu", "pg_device.cuh", "pg_scan.cu")
+# the files holding the kernels of the loop's iterations (the traffic of a full one is recorded as "iteration")
+ITERATION_SOURCES = ("pg_iter.cu", "pg_device.cuh", "pg_scan.cu", "pg_inc.cu")
 
 
 def kernel_text(path, marker):
@@ -787,8 +811,7 @@ def run_ours(args):
     d2h = sum(v.numel() * v.element_size() for v in h_out.values()) + k
     e2e = {"value": m * e_inner / e_wall, "unit": UNIT, "h2d_bytes_per_step": int(h2d), "d2h_bytes_per_step": int(d2h)}
 
-    # roofline: the inner iteration against B_alg = 8 m' + 20 n' (one pass over the edges and a few per-id arrays),
-    # its time taken from the timed steps (solve time, CUDA events around pg_solve, over the valuations computed)
+    # roofline: a full inner iteration against B_alg = 8 m' + 20 n' (iteration_roofline)
     own = game.owner
     deg = np.diff(game.offsets).astype(np.int64)
     s = {"n": n + k, "m": m + k, "n_odd": int(own.sum()), "m_odd": int(deg[own == 1].sum()),
@@ -798,16 +821,11 @@ def run_ours(args):
     hbm, src = peaks()
     b_alg = 8 * (m + k) + 20 * (n + k)
     iter_s = solve_ms / 1000.0 / max(inner_total, 1)
-    roof = {"bound": "hbm", "kernel": "inner iteration (valuation + switching, the CUDA-graph loop of pg_solve)",
-            "achieved": b_alg / iter_s / 1e9, "peak": hbm, "unit": "GB/s", "frac": b_alg / iter_s / 1e9 / hbm,
-            "peak_source": src + " (hbm_gbs, burst copy)", "traffic": measured_traffic("iteration", args.workload),
-            "algorithmic_bytes_per_launch": b_alg, "avg_launch_us": iter_s * 1e6,
-            "units": "one inner iteration: B_alg = 8 m' + 20 n' bytes, m' = %d edges and n' = %d vertices of G' "
-                     "(the Odd switching pass evaluates only the vertices some of whose successors changed their top "
-                     "word, so an iteration moves less)" % (m + k, n + k),
-            "timing": "solve time of the timed steps (CUDA events around pg_solve on the library's stream) / "
-                      "valuations; the loads (%.2f ms per step) are outside" % (load_ms / args.steps),
-            "inner_loop_edges_per_s": m / iter_s}
+    full_s = ((tinfo["valuation_ms"] + tinfo["switch_ms"]) / tinfo["valuations"] / 1000.0 if tinfo["valuations"]
+              else None)
+    roof = iteration_roofline(m, n + k, m + k, full_s, iter_s, hbm)
+    roof.update(peak_source=src + " (hbm_gbs, burst copy)", traffic=measured_traffic("iteration", args.workload),
+                loads="the loads (%.2f ms per step) are outside" % (load_ms / args.steps))
     dominant = None
     if dom_name:
         ms, _, calls = per[dom_name]
@@ -818,13 +836,6 @@ def run_ours(args):
                     "frac": (ach / hbm if ach else None), "traffic": measured_traffic(dom_name, args.workload),
                     "algorithmic_bytes_per_launch": ab, "avg_launch_us": avg_s * 1e6,
                     "timing": "host-driven timing pass (per-kernel CUDA events)"}
-    valuation_path = None
-    if tinfo["valuations"]:
-        per_iter_s = (tinfo["valuation_ms"] + tinfo["switch_ms"]) / tinfo["valuations"] / 1000.0
-        valuation_path = {"inner_iteration_us": per_iter_s * 1e6, "b_alg_bytes": b_alg,
-                          "achieved_gbs": b_alg / per_iter_s / 1e9, "frac_of_hbm": b_alg / per_iter_s / 1e9 / hbm,
-                          "inner_loop_edges_per_s": m / per_iter_s,
-                          "timing": "host-driven timing pass (one launch per kernel, events around each class)"}
 
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps, "warmup": args.warmup,
@@ -838,7 +849,6 @@ def run_ours(args):
         "wall_s": wall,
         "roofline": roof,
         "dominant_kernel": dominant,
-        "inner_iteration_host_loop": valuation_path,
         "load_ms": load_ms / args.steps,
         "kernels": {nm: kernel_entry(nm, v, s, hbm) for nm, v in kstats.items() if v[1]},
         "e2e": e2e,
