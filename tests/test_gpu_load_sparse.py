@@ -39,8 +39,10 @@ def sparse(n, top, seed):
     """Distinct random priorities up to top (which occurs), of both parities."""
     g = gen.native_random_game(n, 1, 5, seed=seed)
     rng = np.random.default_rng(seed)
-    pri = rng.permutation(n).astype(np.int64) * (top // n) + rng.integers(0, max(top // n, 1), n)
-    pri[np.argmax(pri)] = top
+    pri = rng.permutation(n).astype(np.int64) * max(top // n, 1)
+    if top >= 2 * n:
+        pri += rng.integers(0, top // n, n)
+        pri[np.argmax(pri)] = top
     assert np.unique(pri).size == n and set(pri % 2) == {0, 1}
     return Game(n, g.offsets, g.targets, g.owner, pri.astype(np.int32))
 
@@ -72,9 +74,12 @@ def test_sparse_host_arrays_are_not_tried(pg, ctx):
     assert load_launches(pg, ctx, g, False) == load_launches(pg, ctx, g, True) - 1
 
 
-@pytest.mark.parametrize("spread", [7, 100, 3000])
-def test_batches(pg, ctx, spread):
+@pytest.mark.parametrize("wide", [0, 1])
+@pytest.mark.parametrize("spread", [1, 7, 100, 3000])
+def test_batches(pg, ctx, spread, wide):
+    """One union while the priorities are dense enough, game by game beyond; odd and even priorities in all."""
     from test_gpu_batch import KEYS, run_batch
+    pg.pg_set_wide_offsets(ctx, wide)
     games = [sparse(n, n * spread, n) for n in (900, 60, 5000, 2500)]
     vb, res, out = run_batch(pg, ctx, games)
     assert res["rc"] == pg.PG_OK
