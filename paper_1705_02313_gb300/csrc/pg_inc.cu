@@ -687,22 +687,18 @@ constexpr size_t kRvBytes = 48 << 20;
 // Every pass reads all edges, while one pass moves a sector per edge each way:
 // random games of 20M and 40M vertices (11 and 21 ranges), load and solve, 44.6
 // and 117.0 ms in ranges, 47.0 and 118.2 in one pass; more ranges are not worth
-// it. Packed games' targets are near their sources and take one pass (4,096 games,
-// 590M vertices: loop 1,789 ms with 64 ranges, 1,364 in one pass).
+// it.
 constexpr size_t kRvPasses = 24;
 
 // In-degree of every id: all edges in the low half, Odd's in the high half.
-template <typename OffT>
-__global__ void __launch_bounds__(kBlock) k_rv_count(int32_t n, const OffT* __restrict__ off,
+__global__ void __launch_bounds__(kBlock) k_rv_count(int32_t n, const int32_t* __restrict__ off,
                                                      const int32_t* __restrict__ tgt,
-                                                     const uint8_t* __restrict__ flags, int odd_only, int32_t lo,
-                                                     int32_t hi, unsigned long long* __restrict__ deg) {
+                                                     const uint8_t* __restrict__ flags, int32_t lo, int32_t hi,
+                                                     unsigned long long* __restrict__ deg) {
     for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-        const bool odd = (flags[v] & kOwnerOdd) != 0;
-        if (odd_only && !odd) continue;
-        const unsigned long long one = odd ? (1ull << 32) + 1ull : 1ull;
-        const OffT e1 = off[v + 1];
-        for (OffT e = off[v]; e < e1; ++e) {
+        const unsigned long long one = (flags[v] & kOwnerOdd) ? (1ull << 32) + 1ull : 1ull;
+        const int32_t e1 = off[v + 1];
+        for (int32_t e = off[v]; e < e1; ++e) {
             const int32_t t = tgt[e];
             if (t >= lo && t < hi) atomicAdd(deg + t, one);
         }
@@ -721,15 +717,12 @@ __global__ void __launch_bounds__(kBlock) k_rv_bounds(int32_t n, const int32_t* 
     }
 }
 
-template <typename OffT>
-__global__ void __launch_bounds__(kBlock) k_rv_fill(int32_t n, const OffT* __restrict__ off,
+__global__ void __launch_bounds__(kBlock) k_rv_fill(int32_t n, const int32_t* __restrict__ off,
                                                     const int32_t* __restrict__ tgt,
-                                                    const uint8_t* __restrict__ flags, int odd_only, int32_t lo,
-                                                    int32_t hi, int2* __restrict__ cur,
-                                                    int32_t* __restrict__ rv_src) {
+                                                    const uint8_t* __restrict__ flags, int32_t lo, int32_t hi,
+                                                    int2* __restrict__ cur, int32_t* __restrict__ rv_src) {
     for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
         const bool odd = (flags[v] & kOwnerOdd) != 0;
-        if (odd_only && !odd) continue;
         const int64_t e1 = off[v + 1];
         for (int64_t e = off[v]; e < e1; e += 4) {  // four cursor steps in flight
             int32_t t[4], p[4];
@@ -742,6 +735,35 @@ __global__ void __launch_bounds__(kBlock) k_rv_fill(int32_t n, const OffT* __res
             for (int j = 0; j < 4; ++j)
                 if (t[j] >= lo && t[j] < hi) rv_src[p[j]] = v;
         }
+    }
+}
+
+// Odd's edges alone (the marks of k_classify), from Odd's view, whose edges lie
+// together: a server makes these lists again for every layout. Counting over all
+// vertices instead, in 8-byte counters, made a round of a stream of 200 games/s
+// 3% longer.
+__global__ void __launch_bounds__(kBlock) k_rv_count_odd(int32_t m, const int32_t* __restrict__ ptgt,
+                                                         int32_t* __restrict__ deg) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x)
+        atomicAdd(deg + ptgt[e], 1);
+}
+
+__global__ void __launch_bounds__(kBlock) k_rv_bounds_odd(int32_t n, const int32_t* __restrict__ start,
+                                                          int32_t* __restrict__ cur, int2* __restrict__ rv) {
+    for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v <= n; v += gridDim.x * blockDim.x) {
+        const int32_t s = start[v];
+        rv[v] = make_int2(s, v < n ? start[v + 1] : s);
+        if (v < n) cur[v] = s;
+    }
+}
+
+__global__ void __launch_bounds__(kBlock) k_rv_fill_odd(int32_t np, const int32_t* __restrict__ vid,
+                                                        const int32_t* __restrict__ poff,
+                                                        const int32_t* __restrict__ ptgt, int32_t* __restrict__ cur,
+                                                        int32_t* __restrict__ rv_src) {
+    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < np; i += gridDim.x * blockDim.x) {
+        const int32_t e1 = poff[i + 1], v = vid[i];
+        for (int32_t e = poff[i]; e < e1; ++e) rv_src[atomicAdd(cur + ptgt[e], 1)] = v;
     }
 }
 
@@ -776,7 +798,8 @@ static pg_status make_reverse(pg_game* g, int64_t odd_edges) {
     pg_ctx* ctx = g->ctx;
     cudaStream_t s = ctx->stream;
     const int32_t n = g->n;
-    // packed games take no incremental iterations: their lists hold Odd's edges only (the marks of k_classify)
+    // packed games take no incremental iterations: their lists hold Odd's edges only (odd_edges of them; Odd's view
+    // is complete then)
     const int odd_only = inc_applies(g) || g->by_game ? 0 : 1;
     const size_t edges = (size_t)(odd_only ? odd_edges : g->m), mark_bytes = ((size_t)n + 16) & ~(size_t)15;
     PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->rv, sizeof(int2) * ((size_t)n + 1), s));
@@ -788,30 +811,37 @@ static pg_status make_reverse(pg_game* g, int64_t odd_edges) {
         PG_CUDA_TRY(ctx, cudaMemsetAsync(g->emark, 0, mark_bytes, s));
         if (!g->inc && !g->by_game) PG_CUDA_TRY(ctx, dev_alloc(ctx, (void**)&g->inc, sizeof(IncState), s));
     }
-    // the valuation's scratch is free before a loop: degrees and cursors in gd, the scan's output in hugelist/coff
+    // the valuation's scratch is free before a loop: degrees and cursors in gd, the scan's output in coff
     unsigned long long* deg = (unsigned long long*)g->gd;
     const unsigned grid = grid_for(n);
+    if (odd_only) {
+        int32_t* cur = (int32_t*)g->gd;
+        const int32_t np = (int32_t)g->pl_n[1], mp = (int32_t)odd_edges;
+        PG_CUDA_TRY(ctx, cudaMemsetAsync(cur, 0, sizeof(int32_t) * (size_t)n, s));
+        k_rv_count_odd<<<grid_for(std::max(mp, 1)), kBlock, 0, s>>>(mp, g->pl_tgt[1], cur);
+        PG_CUDA_TRY(ctx, exclusive_scan_i32(cur, g->coff, n, nullptr, g->scan_tmp, g->scan_tmp_bytes, s));
+        k_rv_bounds_odd<<<grid, kBlock, 0, s>>>(n, g->coff, cur, g->rv);
+        k_rv_fill_odd<<<grid_for(std::max(np, 1)), kBlock, 0, s>>>(np, g->pl_vid[1], g->pl_off[1], g->pl_tgt[1], cur,
+                                                                   g->rv_src);
+        PG_CUDA_TRY(ctx, cudaGetLastError());
+        ctx->launches += 6;
+        return PG_OK;
+    }
     PG_CUDA_TRY(ctx, cudaMemsetAsync(deg, 0, sizeof(uint64_t) * (size_t)n, s));
     auto ranges = [&](size_t bytes, auto&& pass) {
         const size_t want = (bytes + kRvBytes / 2) / kRvBytes;
-        const int32_t np = g->vgame || want > kRvPasses || want < 1 ? 1 : (int32_t)want;
+        const int32_t np = want > kRvPasses || want < 1 ? 1 : (int32_t)want;
         for (int32_t i = 0; i < np; ++i)
             pass((int32_t)((int64_t)n * i / np), (int32_t)((int64_t)n * (i + 1) / np));
         ctx->launches += np;
     };
     ranges(sizeof(uint64_t) * (size_t)n, [&](int32_t lo, int32_t hi) {
-        if (g->off64) k_rv_count<int64_t><<<grid, kBlock, 0, s>>>(n, g->off64, g->tgt, g->flags, odd_only, lo, hi, deg);
-        else k_rv_count<int32_t><<<grid, kBlock, 0, s>>>(n, g->off, g->tgt, g->flags, odd_only, lo, hi, deg);
+        k_rv_count<<<grid, kBlock, 0, s>>>(n, g->off, g->tgt, g->flags, lo, hi, deg);
     });
     PG_CUDA_TRY(ctx, exclusive_scan_low32(g->gd, g->coff, n, g->scan_tmp, g->scan_tmp_bytes, s));
     k_rv_bounds<<<grid, kBlock, 0, s>>>(n, g->coff, g->gd, g->rv);
     ranges(sizeof(int2) * (size_t)n + sizeof(int32_t) * edges, [&](int32_t lo, int32_t hi) {
-        if (g->off64)
-            k_rv_fill<int64_t><<<grid, kBlock, 0, s>>>(n, g->off64, g->tgt, g->flags, odd_only, lo, hi, (int2*)g->gd,
-                                                       g->rv_src);
-        else
-            k_rv_fill<int32_t><<<grid, kBlock, 0, s>>>(n, g->off, g->tgt, g->flags, odd_only, lo, hi, (int2*)g->gd,
-                                                       g->rv_src);
+        k_rv_fill<<<grid, kBlock, 0, s>>>(n, g->off, g->tgt, g->flags, lo, hi, (int2*)g->gd, g->rv_src);
     });
     PG_CUDA_TRY(ctx, cudaGetLastError());
     ctx->launches += 4;

@@ -376,7 +376,7 @@ pg_status fail(pg_ctx* ctx, pg_status code, const char* msg);
 pg_status cuda_fail(pg_ctx* ctx, cudaError_t e, const char* where);
 pg_status load_game(pg_ctx* ctx, int32_t n, int64_t m, const int32_t* off, const int32_t* tgt,
                     const uint8_t* own, const int32_t* pri, int32_t mem_kind, pg_game** out,
-                    bool with_scratch = true);
+                    bool with_scratch = true, bool one_launch = true);
 // A chunk of a batch loaded as one union into the packed layout (without scratch); *general: it needs load_game.
 pg_status load_union(pg_ctx* ctx, int32_t ngames, const int64_t* vb, const int64_t* eb, const int32_t* off,
                      const int32_t* tgt, const uint8_t* own, const int32_t* pri, int32_t mem_kind, pg_game** out,

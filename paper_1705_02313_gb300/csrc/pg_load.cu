@@ -853,8 +853,9 @@ pg_status load_game_pass(pg_ctx* ctx, int32_t n, int64_t m, const int32_t* off_i
 }
 
 pg_status load_game(pg_ctx* ctx, int32_t n, int64_t m, const int32_t* off_in, const int32_t* tgt_in,
-                    const uint8_t* own_in, const int32_t* pri_in, int32_t mem_kind, pg_game** out, bool with_scratch) {
-    if (out && off_in && tgt_in && own_in && pri_in && n >= 1 && n <= kLoadSmall && m >= n && m <= 8 * (int64_t)kLoadSmall &&
+                    const uint8_t* own_in, const int32_t* pri_in, int32_t mem_kind, pg_game** out, bool with_scratch,
+                    bool one_launch) {
+    if (one_launch && out && off_in && tgt_in && own_in && pri_in && n >= 1 && n <= kLoadSmall && m >= n && m <= 8 * (int64_t)kLoadSmall &&
         (mem_kind == PG_MEM_HOST || mem_kind == PG_MEM_DEVICE)) {
         bool general = false;
         const std::string err = ctx->err;
