@@ -29,6 +29,7 @@ constexpr int kHugeChildren = 4096;   // a parent with more children is ranked b
 constexpr int kCoopTile = 4096;       // elements per tile of the id-ordered scans
 constexpr int kClusterDevices = 64;   // devices whose cluster sizes are remembered
 constexpr int32_t kLoadSmall = 1 << 22;  // a game of up to this many vertices is loaded in one launch (pg_load_small.cu)
+constexpr int32_t kLoadCluster = 24576;  //   by one block per SM beyond this many vertices, by a cluster up to there
 constexpr int32_t kSlabIds = 1 << 20;  // a game of up to this many ids has its scratch in one allocation
 constexpr int32_t kSmallIds = (1 << 18) + 1;  // a game of up to this many ids is valuated in one launch (pg_small.cu)
 constexpr int kSmallBlocks = 512;  // of at most this many blocks (the array of their sums)
@@ -376,7 +377,7 @@ pg_status fail(pg_ctx* ctx, pg_status code, const char* msg);
 pg_status cuda_fail(pg_ctx* ctx, cudaError_t e, const char* where);
 pg_status load_game(pg_ctx* ctx, int32_t n, int64_t m, const int32_t* off, const int32_t* tgt,
                     const uint8_t* own, const int32_t* pri, int32_t mem_kind, pg_game** out,
-                    bool with_scratch = true, bool one_launch = true);
+                    bool with_scratch = true, bool one_launch = true);  // one_launch: load_small may be tried
 // A chunk of a batch loaded as one union into the packed layout (without scratch); *general: it needs load_game.
 pg_status load_union(pg_ctx* ctx, int32_t ngames, const int64_t* vb, const int64_t* eb, const int32_t* off,
                      const int32_t* tgt, const uint8_t* own, const int32_t* pri, int32_t mem_kind, pg_game** out,

@@ -20,7 +20,6 @@ namespace cg = cooperative_groups;
 namespace pg {
 namespace {
 
-constexpr int32_t kLsGrid = 24576;   // beyond this many vertices one block per SM instead of a cluster
 constexpr int kLsThreads = 1024;
 constexpr int kLsCluster = 16;
 constexpr int kLsBlocks = 256;      // at most this many blocks (the array of their sums)
@@ -384,7 +383,7 @@ pg_status load_small(pg_ctx* ctx, int32_t n, int64_t m, const int32_t* off, cons
     a.strat = g->strat;
     a.gsink = g->gsink;
     a.gflags = g->flags;
-    if (n > kLsGrid) {
+    if (n > kLoadCluster) {
         int sms = 0;
         LS_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
         const int blocks = std::max(1, std::min({sms, kLsBlocks, (n + kLsThreads - 1) / kLsThreads}));

@@ -334,9 +334,13 @@ void loader_main(pg_server* sv) {
             sv->queue.pop_front();
             sv->inflight[p.tag] = 1;
         }
+        // A load by one block of 1,024 threads on every SM would keep the worker's cooperative passes waiting for
+        // room until it ends; the general path's kernels are small and leave it. A stream of 200 games/s of 10k to
+        // 4M vertices for 60 s: median 25 to 29 ms, 99th percentile 135 to 276 with all loads in one launch, 19 to
+        // 21 and 86 to 89 so (8 games at once: 16.4 ms either way).
         pg_game* gi = nullptr;
         pg_status st = load_game(ctx, p.n, p.m, p.off.data(), p.tgt.data(), p.own.data(), p.pri.data(), PG_MEM_HOST,
-                                 &gi, false);
+                                 &gi, false, p.n <= kLoadCluster);
         if (st == PG_OK && gi->cv) {  // the packed batch ranks distinct priorities only
             free_game(gi);
             st = PG_EUNSUPPORTED;
