@@ -8,6 +8,7 @@
 #include <vector>
 
 #include <mutex>
+#include <shared_mutex>
 
 #include "pg_internal.cuh"
 
@@ -34,6 +35,24 @@ void drop_loop_graphs(pg_game* g) {
 }
 
 namespace {
+// A device must not be waited for while one of its streams is being captured, in whatever thread: the runtime then
+// drops the capture, and has crashed. Captures exclude the library's waits for a device, and each other; g_turn keeps
+// new waits from overtaking a capture.
+std::shared_mutex g_capture_mu;
+std::mutex g_turn;
+
+cudaError_t wait_for_device() {
+    std::unique_lock<std::mutex> turn(g_turn);
+    std::shared_lock<std::shared_mutex> lock(g_capture_mu);
+    turn.unlock();
+    return cudaDeviceSynchronize();
+}
+
+std::unique_lock<std::shared_mutex> capture_lock() {
+    std::lock_guard<std::mutex> turn(g_turn);
+    return std::unique_lock<std::shared_mutex>(g_capture_mu);
+}
+
 constexpr int kPoolDevices = 64;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pool[kPoolDevices] = {};
@@ -86,7 +105,7 @@ cudaError_t dev_trim(int device) {
     cudaMemPool_t pool = nullptr;
     cudaError_t e = game_pool(device, &pool);
     if (e != cudaSuccess) return e;
-    e = cudaDeviceSynchronize();
+    e = wait_for_device();
     return e == cudaSuccess ? cudaMemPoolTrimTo(pool, 0) : e;
 }
 
@@ -106,7 +125,7 @@ void free_game(pg_game* g) {
     int prev = -1;
     const bool switched =
         cudaGetDevice(&prev) == cudaSuccess && prev != g->device && cudaSetDevice(g->device) == cudaSuccess;
-    cudaDeviceSynchronize();
+    wait_for_device();
     for (void* p : ptrs)
         if (p && !((char*)p >= g->slab && (char*)p < g->slab + g->slab_bytes)) cudaFreeAsync(p, 0);
     if (g->slab) cudaFreeAsync(g->slab, 0);
@@ -431,6 +450,7 @@ bool build_loop_graph(pg_game* g, int64_t cap, bool even, int64_t limit) {
         cudaGetLastError();
         return false;
     }
+    const auto lock = capture_lock();  // (0.2 ms, with the graph's instantiation)
     cudaGraph_t graph = nullptr;
     if (cudaGraphCreate(&graph, 0) != cudaSuccess) {
         cudaGetLastError();
