@@ -94,10 +94,11 @@ constexpr int kIncGameShare = 64;
 
 // A closure that takes too long is abandoned, and a full iteration follows. The
 // budget counts vertices that a block has found (45 ns each) and levels, which
-// take as long as 44 of them (2 us). It is about one and a half full iterations
-// of a game whose plays are short: these take 45 us and 17 us per million ids,
-// 45 and 62 with keys; over all ids in one launch 16 us and 1 us per 128 ids of a
-// block. Where plays are long (a torus, a ring with chords) half of the attempts
+// take as long as 44 of them (2 us). It is about two full iterations of a game
+// whose plays are short: these take 45 us and 17 us per million ids, 45 and 62
+// with keys; over all ids in one launch it is one, 16 us and 1 us per 128 ids of a
+// block. (A third less: 300k vertices 5.97 ms, so 5.89; 400k ladder 5.41 and 5.27;
+// 663k with 4 priorities 14.5 and 14.0; the long plays below do not change.) Where plays are long (a torus, a ring with chords) half of the attempts
 // went on to 256 levels, or to as many vertices as a block holds, 260 us (200k
 // vertices) to 600 us (4M), for nothing. Solving a torus of 4M vertices by full
 // iterations, by these attempts, and with the budget and the waits: 1,332, 2,254
@@ -352,13 +353,14 @@ __global__ void __launch_bounds__(kIncThreads / DIV, DIV) k_inc(IncArgs a) {
     bool fresh = whole() || __ldcg(a.gactive + 1);
     bool even_full = whole() || __ldcg(&a.st->even_full);
     int32_t ns = fresh ? 0 : __ldcg(&a.cnt->n_list);  // switched vertices, all blocks
+    const int32_t wait = whole() ? 0 : __ldcg(&a.st->wait), fails = whole() ? 0 : __ldcg(&a.st->fails);
     // nothing to do here (the state stays as k_bookkeep left it: a full iteration is next)
-    if (dead || (!whole() && (fresh || ns > a.max_seeds || __ldcg(&a.st->wait) > 0))) return;
+    if (dead || (!whole() && (fresh || ns > a.max_seeds || wait > 0))) return;
     int32_t nsl = ns > rank ? (ns - rank + CL - 1) / CL : 0;  // this block's, in la
     for (int32_t i = tid; i < nsl; i += TH) la[i] = __ldcg(a.alist + rank + i * CL);
     if (tid == 0) {
         c_e = c_zero = p_wait = p_since = 0;
-        p_fails = whole() ? 0 : __ldcg(&a.st->fails);
+        p_fails = fails;
     }
     int32_t mode = kIncFull, iters = 0;
     bool done = false;
@@ -849,7 +851,7 @@ static pg_status make_reverse(pg_game* g, int64_t odd_edges) {
 }
 
 static int32_t inc_budget(const pg_game* g, bool even) {
-    const int64_t base = g->cv && !even ? 12 : 33, per = !g->cv ? 14 : even ? 31 : 12;
+    const int64_t base = !g->cv ? 50 : even ? 66 : 12, per = !g->cv ? 20 : even ? 62 : 12;
     return kIncLevelCost * (int32_t)(base + g->n * per / 1000000);
 }
 
