@@ -11,9 +11,8 @@
  *    pri[n] >= 0. Every vertex has at least one out-edge (Section 2: no
  *    terminal vertices). Pairwise distinct priorities (the random workloads'
  *    permuted priorities) are ranked by the nearest-greater forest; a game
- *    whose priorities repeat runs in count-vector mode (below), which needs
- *    at most 5 distinct priorities after preprocessing and fewer than 2^24
- *    vertices, else PG_EUNSUPPORTED.
+ *    whose priorities repeat runs in count-vector mode (below), whose
+ *    limits pg_load_csr states, else PG_EUNSUPPORTED.
  *  - mem_kind says where caller arrays live: PG_MEM_HOST (pageable or pinned
  *    host memory) or PG_MEM_DEVICE (device memory of the context's GPU).
  *    Caller arrays are read or written during the call only and never
@@ -202,8 +201,9 @@ pg_status pg_valuate(pg_game *game, const int32_t *sigma, const int8_t *dummy_si
  * (times only while timing is enabled; launch counts always). name is the
  * class (walk, jump, chain1, parents, big_parents, sink_scan, chain2,
  * switch_odd, switch_even); calls counts timed event pairs, launches counts
- * kernels. out has room for cap entries (host memory); count receives the
- * number of classes. The paper reports wall-clock time only (Section 6); this
+ * kernels; the launches that run a whole loop, a whole valuation or incremental
+ * iterations belong to no class. out has room for cap entries (host memory);
+ * count receives the number of classes. The paper reports wall-clock time only (Section 6); this
  * breakdown has no counterpart there. */
 typedef struct {
     char name[24];

@@ -71,10 +71,6 @@ __host__ __device__ inline bool gd_sink(uint64_t w) { return (w & kSinkBit) != 0
 __host__ __device__ inline bool gd_resolved(uint64_t w) { return (w & kResolved) != 0; }
 __host__ __device__ inline bool gd_none(uint64_t w) { return (w & kNone) != 0; }
 
-// kind[v] written by the first chain pass
-constexpr uint8_t kKindFin = 1;        // finite valuation
-constexpr uint8_t kKindSinkChild = 2;  // nearest greater ancestor is the sink
-
 // Device counters of one valuation (reset at its start).
 struct Counters {
     int32_t n_pending;   // walks that ran out of steps (length of the pending list)
