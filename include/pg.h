@@ -389,9 +389,11 @@ pg_status pg_last_timing(const pg_game *game, double *total_ms, double *valuatio
  * between iterations; the graph is built on first use per game and kept with
  * it. For one game an iteration after which few vertices switched is followed,
  * in the same body, by iterations over the vertices they affect alone; a small
- * game's whole loop is one kernel launch. With graphs disabled, or when timing is enabled, or if the CUDA runtime
- * refuses to build the graph, the host launches each iteration and
- * synchronises once per iteration. Both give identical results. The paper has
+ * game's whole loop is one kernel launch. The host launches the first two
+ * iterations of a solve from a given strategy on a game that has had no loop
+ * yet (they may be all). With graphs disabled, or when timing is enabled, or if
+ * the CUDA runtime refuses to build the graph, the host launches each iteration
+ * and synchronises once per iteration. Both give identical results. The paper has
  * no counterpart (it concerns launching work on the device only). */
 pg_status pg_set_graphs(pg_ctx *ctx, int32_t enable);
 /* Work partitioning of the valuation (the paper has no counterpart; results
@@ -457,8 +459,8 @@ pg_status pg_set_wide_offsets(pg_ctx *ctx, int32_t enable);
  * does less work per iteration. */
 pg_status pg_set_loop_ranks(pg_ctx *ctx, int32_t enable);
 
-/* graph: 1 if the last loop on game ran on the device (as a graph or, for a
- * small game, as one kernel launch), else 0; iterations: the valuations it
+/* graph: 1 if the last loop on game ran (or ended) on the device (as a graph or,
+ * for a small game, as one kernel launch), else 0; iterations: the valuations it
  * computed (each may be NULL). */
 pg_status pg_last_loop(const pg_game *game, int32_t *graph, int64_t *iterations);
 

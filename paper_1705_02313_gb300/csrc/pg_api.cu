@@ -533,13 +533,13 @@ bool runs_whole(const pg_game* g, const Timer& tm) {
 // synchronises once per iteration. A positive limit ends the call after that
 // many iterations even if games are still active (their state stays on the
 // device and a later call continues them).
-pg_status run_loop_once(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t limit, int64_t* ran) {
+pg_status run_loop_once(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t limit, int64_t* ran, bool host) {
     pg_ctx* ctx = g->ctx;
     g->last_graph = g->last_stale = false;
     *ran = 0;
     const bool cmp = loop_compares(g);
     const int64_t hard = limit > 0 ? std::min<int64_t>(limit, cap + 2) : cap + 2;
-    if (runs_whole(g, tm)) {  // the whole loop is one launch
+    if (!host && runs_whole(g, tm)) {  // the whole loop is one launch
         cudaStream_t s = ctx->stream;
         PG_CUDA_TRY(ctx, cudaMemsetAsync(g->loop_iters, 0, 2 * sizeof(int64_t), s));
         PG_CUDA_TRY(ctx, cudaMemsetAsync(g->cnt, 0, sizeof(Counters), s));
@@ -553,7 +553,7 @@ pg_status run_loop_once(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t l
         g->last_graph = true;
         return st;
     }
-    if (!tm.on && ctx->graphs && build_loop_graph(g, cap, even, hard)) {
+    if (!host && !tm.on && ctx->graphs && build_loop_graph(g, cap, even, hard)) {
         const int w = even ? 1 : 0;
         cudaStream_t s = ctx->stream;
         PG_CUDA_TRY(ctx, cudaMemsetAsync(g->loop_iters, 0, 2 * sizeof(int64_t), s));
@@ -601,12 +601,19 @@ pg_status run_loop_once(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t l
     }
 }
 
+// A solve from a given strategy (a warm start) runs this many iterations before it
+// has views and lists made and the loop captured: a solution that still holds ends
+// with the second. On a game of 4M vertices just loaded 1,540 us with them (1,340
+// before Even's predecessors were in the lists), 930 without; with 4 priorities
+// 1,600 (870, no lists), 800.
+constexpr int64_t kWarmIters = 2;
+
 // The loop of Algorithm 1 (run_loop_once) until its end, a cap or the limit.
 // When an iteration finds a g-chain longer than the cutover depth, it is
 // abandoned before anything is switched or counted, the loop stops, and the
 // game continues from the same profile with the ruling-set ranks (for the
 // rest of this call), so the trajectory is unchanged.
-pg_status run_loop(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t limit) {
+pg_status run_loop(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t limit, bool warm) {
     g->depth_ok = false;
     int div = 1, blocks = 1;
     if (even && limit <= 0 && !tm.on && g->ctx->graphs && games_apply(g, &div, &blocks)) {
@@ -616,23 +623,42 @@ pg_status run_loop(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t limit)
         g->last_cmp = g->last_graph = true;
         if (done) return PG_OK;
     }
-    if (runs_whole(g, tm) || (g->cv && !tm.on && g->ctx->graphs && inc_applies(g))) {
-        pg_status st = build_reverse(g, 0);
-        if (st == PG_ENOMEM) g->no_inc = true;  // the loop without incremental iterations
-        else if (st) return st;
-    }
-    if (!runs_whole(g, tm) && loop_compares(g) && !g->pl_ok) {
-        pg_status st = build_player_split(g);
-        if (st) return st;
-    }
-    if (omark_of(g))  // the first Odd pass of the call evaluates every Odd vertex (a nonzero flag)
-        PG_CUDA_TRY(g->ctx, cudaMemsetAsync(g->gactive + 1, 0xff, sizeof(int32_t), g->ctx->stream));
-    if (g->inc) PG_CUDA_TRY(g->ctx, cudaMemsetAsync(g->inc, 0, sizeof(IncState), g->ctx->stream));
+    // the views and lists of the loop's passes
+    auto prepare = [&]() -> pg_status {
+        if (runs_whole(g, tm) || (g->cv && !tm.on && g->ctx->graphs && inc_applies(g))) {
+            pg_status st = build_reverse(g, 0);
+            if (st == PG_ENOMEM) g->no_inc = true;  // the loop without incremental iterations
+            else if (st) return st;
+        }
+        if (!runs_whole(g, tm) && loop_compares(g) && !g->pl_ok) {
+            pg_status st = build_player_split(g);
+            if (st) return st;
+        }
+        if (omark_of(g))  // the first Odd pass of the call evaluates every Odd vertex (a nonzero flag)
+            PG_CUDA_TRY(g->ctx, cudaMemsetAsync(g->gactive + 1, 0xff, sizeof(int32_t), g->ctx->stream));
+        if (g->inc) PG_CUDA_TRY(g->ctx, cudaMemsetAsync(g->inc, 0, sizeof(IncState), g->ctx->stream));
+        return PG_OK;
+    };
+    // a solve from a given strategy may end at once: its first iterations do without views, lists and a graph
+    bool host = warm && limit <= 0 && !tm.on && g->ctx->graphs && inc_applies(g) && !g->rv_ok && !g->pl_ok &&
+                !runs_whole(g, tm);
+    if (!host)
+        if (pg_status st = prepare()) return st;
     int64_t done = 0;
     for (;;) {
         int64_t ran = 0;
-        pg_status st = run_loop_once(g, cap, even, tm, limit > 0 ? limit - done : 0, &ran);
+        pg_status st = run_loop_once(g, cap, even, tm, host ? kWarmIters : limit > 0 ? limit - done : 0, &ran, host);
         if (st) return st;
+        if (host) {
+            host = false;
+            const bool active = g->ctx->pinned[0] != 0;
+            g->last_cmp = loop_compares(g);
+            if (active && (g->cv || !g->hcnt->deep)) {
+                st = prepare();
+                if (st) return st;
+                continue;
+            }
+        }
         // (k_inc keeps the keys of a count-vector game, not its classes and walk lengths)
         g->last_cmp = loop_compares(g) || g->last_stale;
         if (g->cv || g->deep_mode || !g->hcnt->deep) return PG_OK;
@@ -908,7 +934,7 @@ pg_status pg_solve(pg_game* g, const pg_solve_opts* opts, pg_result* out) {
     Timer tm(g);
     tm.mark(3);
     g->reset_tau = opts && opts->reset_tau;
-    st = run_loop(g, cap, true, tm);
+    st = run_loop(g, cap, true, tm, 0, opts && opts->sigma_init);
     g->reset_tau = false;
     if (st) return st;
     GameState gs;

@@ -415,7 +415,8 @@ pg_status write_outputs(pg_game* g, int32_t mem_kind, uint8_t* win, int32_t* sig
                         int32_t* vdepth, int32_t* vrank, int32_t* vdom, int8_t* dsig, bool depth_ready = false);
 // Algorithm 1 for all games of g (even = false: inner loop only).
 // limit > 0: return after at most limit iterations (games may still be active).
-pg_status run_loop(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t limit = 0);
+// warm: from a strategy that the caller gave.
+pg_status run_loop(pg_game* g, int64_t cap, bool even, Timer& tm, int64_t limit = 0, bool warm = false);
 // Launches of the iteration loop graph are invalidated (sizes of g changed).
 void drop_loop_graphs(pg_game* g);
 // Packs loaded single games (freed by the call) into one batch game.
