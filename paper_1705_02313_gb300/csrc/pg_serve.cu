@@ -323,6 +323,7 @@ void loader_main(pg_server* sv) {
     }
     for (;;) {
         Pending p;
+        size_t waiting = 0;  // behind it
         {
             std::unique_lock<std::mutex> lk(sv->mu);
             sv->cv_load.wait(lk, [&] {
@@ -332,15 +333,17 @@ void loader_main(pg_server* sv) {
             if (sv->stop || sv->fatal) return;
             p = std::move(sv->queue.front());
             sv->queue.pop_front();
+            waiting = sv->queue.size();
             sv->inflight[p.tag] = 1;
         }
         // A load by one block of 1,024 threads on every SM would keep the worker's cooperative passes waiting for
-        // room until it ends; the general path's kernels are small and leave it. A stream of 200 games/s of 10k to
-        // 4M vertices for 60 s: median 25 to 29 ms, 99th percentile 135 to 276 with all loads in one launch, 19 to
-        // 21 and 86 to 89 so (8 games at once: 16.4 ms either way).
+        // room until it ends; the general path's kernels are small and leave it. When more than one game waits
+        // behind it (a burst), the shorter load wins (30 games of 200k at once: 45.8 ms, so 43.0). A stream of 200
+        // games/s of 10k to 4M vertices for 60 s: median 25 to 29 ms, 99th percentile 135 to 276 with all loads in
+        // one launch, 19 to 21 and 83 to 89 so (8 games at once: 16.4 and 16.6 ms).
         pg_game* gi = nullptr;
         pg_status st = load_game(ctx, p.n, p.m, p.off.data(), p.tgt.data(), p.own.data(), p.pri.data(), PG_MEM_HOST,
-                                 &gi, false, p.n <= kLoadCluster);
+                                 &gi, false, p.n <= kLoadCluster || waiting > 1);
         if (st == PG_OK && gi->cv) {  // the packed batch ranks distinct priorities only
             free_game(gi);
             st = PG_EUNSUPPORTED;
