@@ -98,12 +98,12 @@ constexpr int kIncGameShare = 64;
 // whose plays are short: these take 45 us and 17 us per million ids, 45 and 62
 // with keys; over all ids in one launch it is one, 16 us and 1 us per 128 ids of a
 // block. (A third less: 300k vertices 5.97 ms, so 5.89; 400k ladder 5.41 and 5.27;
-// 663k with 4 priorities 14.5 and 14.0; the long plays below do not change.) Where plays are long (a torus, a ring with chords) half of the attempts
-// went on to 256 levels, or to as many vertices as a block holds, 260 us (200k
-// vertices) to 600 us (4M), for nothing. Solving a torus of 4M vertices by full
-// iterations, by these attempts, and with the budget and the waits: 1,332, 2,254
-// and 1,320 ms; a ring of 4M 5,321, 8,735 and 5,490; a torus of 200k 180, 185 and
-// 158; a random game of 1M 6.7, 5.1 and 5.1.
+// 663k with 4 priorities 14.5 and 14.0.) Where plays are long (a torus, a ring with
+// chords) half of the attempts went on to 256 levels, or to as many vertices as a
+// block holds, 260 us (200k vertices) to 600 us (4M), for nothing. Solving a torus
+// of 4M vertices by full iterations, by these attempts, and with the budget and
+// the waits: 1,324, 2,254 and 1,298 ms; a ring of 4M 5,299, 8,735 and 5,510; a
+// torus of 200k 180, 185 and 156; a random game of 1M 6.7, 5.1 and 5.1.
 constexpr int32_t kIncLevelCost = 44;
 // An abandoned attempt is followed by 1 full iteration; by 2, 4, ... 32 while they keep failing.
 constexpr int32_t kIncFails = 5;
